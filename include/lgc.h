@@ -166,10 +166,12 @@ enum {
   LGC_OPT_PULL = 7,             /* deterministic rounds gather from the frontier instead of
                                    sorting pushed records: 0 automatic (rounds of >= 2m/16
                                    edges), 1 never, 2 always; same results either way */
-  LGC_OPT_DEVICE_ROUNDS = 8,    /* 1 (default): consecutive small rounds of atomic-mode
-                                   PR-Nibble run in one cooperative launch without returning
-                                   to the host in between; 0: one launch per step.  Request-
-                                   loop workers never use it.  Same results either way */
+  LGC_OPT_DEVICE_ROUNDS = 8,    /* 1 (default): consecutive small rounds of PR-Nibble (both
+                                   modes, seed sets and beta fractions too; deterministic
+                                   ones unless LGC_OPT_PULL is 2) and of atomic-mode Nibble
+                                   run in one cooperative launch without returning to the
+                                   host in between; 0: one launch per step.  Request-loop
+                                   workers never use it.  Same results either way */
   LGC_OPT_PULL_BATCH = 9,       /* edges per lane per batch in the heavy-vertex pull gather:
                                    0 (default) the graph's tuned value (see
                                    lgc_graph_autotune), or 4, 8, 16 */

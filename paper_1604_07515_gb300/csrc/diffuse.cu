@@ -34,9 +34,11 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "foldwarp.cuh"
 #include "fx128.cuh"
 #include "lookback.cuh"
 #include "prim.cuh"
+#include "rounds.cuh"
 
 namespace cg = cooperative_groups;
 
@@ -464,15 +466,8 @@ __global__ void __launch_bounds__(kBlock)
 }
 
 // ---------------------------------------------------------------------------
-// Consecutive small PR-Nibble rounds (atomic mode) in one cooperative launch:
-// vertexMap, prefix sum of the frontier degrees, edge push with the
-// threshold-crossing append, and the frontier swap, separated by grid-wide
-// barriers, with no return to the host between rounds.  The kernel stops
-// (leaving the state for the host, which continues with the same rounds
-// one launch per step) when the frontier is empty, the round limit is
-// reached, or the next round is not small: more than e_max edges, a next
-// frontier that might not fit the buffers, or a table that might pass its
-// load limit.  Each round computes exactly what the host-driven round does.
+// Consecutive small Nibble rounds in one cooperative launch (rounds_nibble_kernel;
+// PR-Nibble's are in rounds.cu).
 // ---------------------------------------------------------------------------
 struct RoundsState {
   int32_t cur;   // frontier buffer of the current round (0 or 1)
@@ -546,70 +541,13 @@ __device__ inline int64_t grid_scan_tail(const int64_t* cnt, int64_t nf, int64_t
 // chunk's record count | barrier | the scan | barrier | the edge push |
 // barrier.  The current round's counters are cleared after the first
 // barrier (nothing reads them after it), for their reuse as the next
-// round's "next".
-__global__ void __launch_bounds__(kBlock)
-    rounds_prnibble_kernel(Table T, const int64_t* __restrict__ off,
-                           const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
-                           double alpha, double cs, double cn, double eps, int rule,
-                           int32_t* fv0, int32_t* fs0, int32_t* fv1, int32_t* fs1, int32_t fcap,
-                           double* share, int64_t* cnt, int64_t* epos, int64_t* foff,
-                           int64_t* bsum, Counters* Cn, RoundsState* S, int64_t max_rounds,
-                           int64_t e_max, int64_t key_limit) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ int64_t s_red[kBlock / 32];
-  int cur = __ldcg(&S->cur);
-  int64_t count = __ldcg(&S->count), rounds = __ldcg(&S->rounds);
-  int64_t pushes = __ldcg(&S->pushes), pushed = __ldcg(&S->pushed_edges);
-  for (;;) {
-    const int nxt = cur ^ 1;
-    const int64_t nf = __ldcg(&Cn[cur].next_size);
-    const int64_t E = __ldcg(&Cn[cur].next_edges);
-    const int err = __ldcg(&Cn[cur].err) | __ldcg(&Cn[nxt].err);
-    int stop = 0;
-    if (err) stop = 4;
-    else if (nf == 0) stop = 1;
-    else if (rounds >= max_rounds) stop = 2;
-    else if (E > e_max || nf + E > fcap || count + E > key_limit) stop = 3;
-    if (stop) {  // the same decision in every thread: no barrier is left waiting
-      if (blockIdx.x == 0 && threadIdx.x == 0) {
-        S->cur = cur;
-        S->stop = stop;
-        S->count = count;
-        S->rounds = rounds;
-        S->pushes = pushes;
-        S->pushed_edges = pushed;
-      }
-      return;
-    }
-    int32_t* fv = cur ? fv1 : fv0;
-    int32_t* fs = cur ? fs1 : fs0;
-    int32_t* nfv = cur ? fv0 : fv1;
-    int32_t* nfs = cur ? fs0 : fs1;
-    // vertexMap (the original rule keeps a vertex whose reduced residual
-    // still reaches the threshold)
-    int64_t c0, c1;
-    grid_chunk(nf, &c0, &c1);
-    int64_t part = prnibble_vmap_body(c0, c1, blockDim.x, fv, fs, T, off, alpha, cs, cn, eps,
-                                      rule, 0, 1, share, cnt, foff, nfv, nfs, fcap, &Cn[nxt]);
-    part = block_sum_i64(part, s_red);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = part;
-    grid.sync();
-    if (blockIdx.x == 0 && threadIdx.x == 0) Cn[cur] = Counters{};
-    const int64_t tot = grid_scan_tail(cnt, nf, epos, bsum);
-    grid.sync();
-    // edge push into the same table, appending crossings to the next frontier
-    emap_atomic_body(col, deg, share, epos, foff, nf, min(E, tot), T, eps, kFmThreshold, nfv,
-                     nfs, fcap, &Cn[nxt]);
-    grid.sync();
-    rounds += 1;
-    pushes += nf;
-    pushed += E;
-    count += __ldcg(&Cn[nxt].inserted);
-    cur = nxt;
-  }
-}
-
-// Nibble (Fig. alg:nibble, atomic mode) the same way: each round fills a
+// round's "next".  The kernel stops (leaving the state for the host, which
+// continues with the same rounds one launch per step) when the frontier is
+// empty, the round limit is reached, or the next round is not small: more
+// than e_max edges, a next frontier that might not fit the buffers, or a
+// table that might pass its load limit.
+//
+// Nibble (Fig. alg:nibble, atomic mode): each round fills a
 // fresh p' from p, so two hashed tables of capacity cap alternate as p'
 // (A in device round 0, 2, ..., B in 1, 3, ...; both clear at launch) and p
 // starts in T0 (any form), the table the host's rounds left.  A round runs
@@ -852,78 +790,6 @@ __device__ inline int pull_finish(const Table& D, int32_t w, int64_t d, double a
   const int ins = !present && !(atomicOr(&D.bits[w >> 5], m) & m);
   if (pull_qualifies(acc, d, c, fmode)) atomicOr(&qbits[w >> 5], m);
   return ins;
-}
-
-// ---------------------------------------------------------------------------
-// The ordered fold acc <- RN(acc + s_k) of 256 shares by a warp, without a
-// chain of dependent FP64 adds (the segment-parallel fold of long lists
-// refolds a segment with it where its composed step does not apply).
-//
-// While acc stays in one binade it is A * u with the integer A below 2^53,
-// and each share is an integer step A -> A + g[A & 1] (fold_step in
-// fx128.cuh); steps compose, so a warp scan of the compositions gives every
-// partial fold.  The first position whose value reaches 2^53 leaves the
-// binade: that one add is done in FP64 (the rounding of the next binade
-// applies), and the scan restarts after it with the new binade.  Every
-// result equals the sequential fold's bit for bit.
-// ---------------------------------------------------------------------------
-// Folds the 32 * 8 shares v (lane l holds positions 8l .. 8l+7, in list
-// order) into acc, lane-uniformly.
-__device__ inline double fold_batch(double acc, const double v[8], int lane) {
-  int start = 0;
-  while (start < 256) {
-    const int bu = fold_binade(acc);
-    const int64_t A0 = fold_int(acc);
-    FoldStep st[8];
-    FoldStep F = {0, 0};
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      st[j] = 8 * lane + j >= start ? fold_step(v[j], bu) : FoldStep{0, 0};
-      F = fold_compose(F, st[j]);
-    }
-    // inclusive scan over lanes, then shift to exclusive
-    FoldStep P = F;
-#pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      FoldStep q;
-      q.g0 = __shfl_up_sync(0xffffffffu, P.g0, o);
-      q.g1 = __shfl_up_sync(0xffffffffu, P.g1, o);
-      if (lane >= o) P = fold_compose(q, P);
-    }
-    FoldStep E;
-    E.g0 = __shfl_up_sync(0xffffffffu, P.g0, 1);
-    E.g1 = __shfl_up_sync(0xffffffffu, P.g1, 1);
-    if (lane == 0) E = {0, 0};
-    int64_t A = fold_apply(E, A0);
-    int cj = -1;
-    int64_t before = 0;
-#pragma unroll
-    for (int j = 0; j < 8; j++) {
-      const int64_t nx = fold_apply(st[j], A);
-      if (cj < 0 && nx >= kFoldTop) {
-        cj = j;
-        before = A;
-      }
-      A = nx;
-    }
-    const unsigned crossed = __ballot_sync(0xffffffffu, cj >= 0);
-    if (!crossed) {
-      const int64_t Aend = __shfl_sync(0xffffffffu, A, 31);
-      return fold_double(Aend, bu);
-    }
-    const int lc = __ffs(crossed) - 1;
-    double nacc = 0.0;
-    if (lane == lc) {
-      double sj = 0.0;
-#pragma unroll
-      for (int j = 0; j < 8; j++)
-        if (j == cj) sj = v[j];
-      nacc = fold_double(before, bu) + sj;  // the add that leaves the binade
-    }
-    acc = __shfl_sync(0xffffffffu, nacc, lc);
-    start = 8 * lc + __shfl_sync(0xffffffffu, cj, lc) + 1;
-  }
-  return acc;
 }
 
 // Deterministic mode, vertices of degree (kPullLight, kDetBig]: one lane per
@@ -1852,6 +1718,7 @@ struct PushWork {
   DBuf<int64_t> xbsum;
   DBuf<Counters> xcn;
   DBuf<RoundsState> xst;
+  RoundsMem rmem;
   lgc_stats st{};
   explicit PushWork(lgc_ctx* c, lgc_graph* gr) : ctx(c), g(gr) {}
   ~PushWork() {
@@ -1874,6 +1741,7 @@ struct PushWork {
     xbsum.release(ctx);
     xcn.release(ctx);
     xst.release(ctx);
+    rmem.release(ctx);
     share.release(ctx);
     cnt.release(ctx);
     epos.release(ctx);
@@ -2224,91 +2092,45 @@ struct PushWork {
     return read_counters(out);
   }
 
-  // Consecutive small rounds of atomic PR-Nibble on the device (see
-  // rounds_prnibble_kernel).  Runs at least one round when small_round()
-  // holds for the current one; afterwards F, T's key count and st describe
-  // the state reached, and the host continues from there.
+  // Nibble's small rounds on the device (rounds_nibble_kernel).
   static constexpr int64_t kRoundsEmax = int64_t{1} << 20;
   static constexpr int64_t kRoundsPerLaunch = 1024;
   int64_t rounds_emax() const { return std::min<int64_t>(kRoundsEmax, g->nnz / 16); }
   int64_t rounds_fcap() const { return std::min<int64_t>(g->n, 2 * kRoundsEmax); }
-  static int64_t key_limit(const Table& T) { return T.dense ? INT64_MAX : T.cap / 2; }
+  // keys T takes within load 1/2 (no set has more than n)
+  int64_t key_limit(const Table& T) const {
+    return T.dense || T.cap >= 2 * g->n ? INT64_MAX : T.cap / 2;
+  }
   bool small_round_nibble() const {
     return ctx->device_rounds && !ctx->trace && F.size > 0 && F.edges <= rounds_emax() &&
            F.size + F.edges <= rounds_fcap();
   }
-  bool small_round(const Table& T, int64_t count) const {
-    return ctx->device_rounds && !ctx->trace && F.size > 0 && F.edges <= rounds_emax() &&
-           F.size + F.edges <= rounds_fcap() && count + F.edges <= key_limit(T);
+  // The edges from which a round is a pull round (use_pull), automatic policy.
+  int64_t pull_min() const {
+    if (ctx->table_form == 1 || ctx->pull_policy == 1 || g->n < 1024) return INT64_MAX;
+    return g->nnz / 16;
   }
+  // PR-Nibble's small rounds on the device (rounds.cu) from the state in F, T
+  // and count; afterwards those and st describe the state reached.
   int device_rounds_prnibble(Table& T, int64_t* count, double alpha, double cs, double cn,
-                             double eps, int rule, int64_t rounds_left) {
+                             double eps, int rule, bool det, double beta, int64_t rounds_left) {
     cudaStream_t s = ctx->stream;
-    static int blocks_per_sm = -1;  // the same for every device of this build
-    if (blocks_per_sm < 0) {
-      int nb = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, rounds_prnibble_kernel, kBlock, 0) !=
-          cudaSuccess)
-        nb = 0;
-      blocks_per_sm = nb;
+    RoundsOut o;
+    LGC_TRY(rounds_prnibble(ctx, g, rmem, T, F.v.ptr, F.s.ptr, F.size, F.edges, *count, alpha, cs,
+                            cn, eps, rule, det, beta, pull_min(), rounds_left, key_limit(T), &o));
+    if (o.rounds == 0) return LGC_OK;  // no room for them: the rounds stay on the host
+    LGC_TRY(F.v.reserve(ctx, std::max<int64_t>(o.nf, 1024)));
+    LGC_TRY(F.s.reserve(ctx, std::max<int64_t>(o.nf, 1024)));
+    if (o.nf > 0) {
+      LGC_CUDA_TRY(cudaMemcpyAsync(F.v.ptr, o.v, 4 * o.nf, cudaMemcpyDeviceToDevice, s));
+      LGC_CUDA_TRY(cudaMemcpyAsync(F.s.ptr, o.s, 4 * o.nf, cudaMemcpyDeviceToDevice, s));
     }
-    int sms = 0;
-    LGC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-    // one block per SM: the rounds are small, and fewer blocks wait at each
-    // grid barrier (two per SM measured 0.3% slower on the bench step)
-    const int G = sms * std::min(blocks_per_sm, 1);
-    if (G < 1) {  // no co-resident grid possible: rounds stay on the host
-      ctx->device_rounds = false;
-      return LGC_OK;
-    }
-    const int64_t fcap = rounds_fcap();
-    for (int k = 0; k < 2; k++) {
-      LGC_TRY(X[k].v.reserve(ctx, fcap));
-      LGC_TRY(X[k].s.reserve(ctx, fcap));
-    }
-    LGC_TRY(reserve_frontier_scratch(fcap));
-    LGC_TRY(xbsum.reserve(ctx, G));
-    LGC_TRY(xcn.reserve(ctx, 2));
-    LGC_TRY(xst.reserve(ctx, 1));
-    LGC_TRY(total.reserve(ctx, 8));
-    LGC_CUDA_TRY(cudaMemcpyAsync(X[0].v.ptr, F.v.ptr, 4 * F.size, cudaMemcpyDeviceToDevice, s));
-    LGC_CUDA_TRY(cudaMemcpyAsync(X[0].s.ptr, F.s.ptr, 4 * F.size, cudaMemcpyDeviceToDevice, s));
-    rounds_init_kernel<<<1, 1, 0, s>>>(xcn.ptr, xst.ptr, F.size, F.edges, *count);
-    LGC_COUNT_LAUNCH(ctx);
-    int32_t fc = (int32_t)fcap;
-    // at most kRoundsPerLaunch rounds per launch: the host regains control
-    // at least that often
-    int64_t mr = std::min<int64_t>(rounds_left, kRoundsPerLaunch), em = rounds_emax(),
-            kl = key_limit(T);
-    void* args[] = {&T, &g->off, &g->col, &g->deg, &alpha, &cs, &cn, &eps, &rule,
-                    &X[0].v.ptr, &X[0].s.ptr, &X[1].v.ptr, &X[1].s.ptr, &fc, &share.ptr, &cnt.ptr,
-                    &epos.ptr, &foff.ptr, &xbsum.ptr, &xcn.ptr, &xst.ptr, &mr, &em, &kl};
-    {
-      ProfScope ps(ctx, LGC_PROF_EDGEMAP, 0.0);
-      LGC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)rounds_prnibble_kernel, G, kBlock,
-                                               args, 0, s));
-      LGC_COUNT_LAUNCH(ctx);
-    }
-    rounds_pack_kernel<<<1, 1, 0, s>>>(xcn.ptr, xst.ptr, total.ptr);
-    LGC_COUNT_LAUNCH(ctx);
-    LGC_CUDA_TRY(cudaMemcpyAsync(ctx->h_scratch, total.ptr, 64, cudaMemcpyDeviceToHost, s));
-    LGC_CUDA_TRY(cudaStreamSynchronize(s));
-    const int64_t* o = ctx->h_scratch;
-    const int64_t cur = o[1], nf = o[2], E = o[3], rounds = o[5];
-    if (ctx->profile && !ctx->prof_pending.empty())
-      ctx->prof_pending.back().bytes += 24.0 * (double)o[7] + 88.0 * (double)o[6];
-    if ((o[0] >> 8) != 0) return LGC_ETABLEFULL;
-    if (rounds < 1) return LGC_ECUDA;  // the host checked that the first round is small
-    LGC_TRY(F.v.reserve(ctx, std::max<int64_t>(nf, 1024)));
-    LGC_TRY(F.s.reserve(ctx, std::max<int64_t>(nf, 1024)));
-    LGC_CUDA_TRY(cudaMemcpyAsync(F.v.ptr, X[cur].v.ptr, 4 * nf, cudaMemcpyDeviceToDevice, s));
-    LGC_CUDA_TRY(cudaMemcpyAsync(F.s.ptr, X[cur].s.ptr, 4 * nf, cudaMemcpyDeviceToDevice, s));
-    F.size = nf;
-    F.edges = E;
-    *count = o[4];
-    st.rounds += rounds;
-    st.pushes += o[6];
-    st.pushed_edges += o[7];
+    F.size = o.nf;
+    F.edges = o.E;
+    *count = o.count;
+    st.rounds += o.rounds;
+    st.pushes += o.pushes;
+    st.pushed_edges += o.pushed;
     return LGC_OK;
   }
 
@@ -2564,6 +2386,33 @@ int ensure_capacity(lgc_ctx* ctx, Table* T, int64_t count, int64_t add, int64_t 
   return LGC_OK;
 }
 
+// Sets of a graph of up to kDenseSmall vertices are dense from the start
+// (automatic form): clearing 16 bytes a vertex costs 4 us at that size,
+// growing and converting a table on the way 40 us and more.
+constexpr int64_t kDenseSmall = int64_t{1} << 20;
+// Keys a table has room for ahead of the device-driven rounds.
+constexpr int64_t kRoomKeys = 16384;
+
+bool dense_small(const lgc_ctx* ctx, int64_t n) {
+  return ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
+}
+
+// Before device-driven rounds: as ensure_capacity for the next round, with
+// room for 16 times its keys (a hashed table that would take more memory
+// than the dense form becomes dense).
+int ensure_room_ahead(lgc_ctx* ctx, Table* T, int64_t count, int64_t add, int64_t n,
+                      const int32_t* fv, int32_t* fs, int64_t nf) {
+  if (T->dense) return LGC_OK;
+  const int64_t need = min64(count + add, n);
+  if (want_dense(ctx, need, n) || dense_small(ctx, n)) return table_to_dense(ctx, T, n, fv, fs, nf);
+  if (2 * need <= T->cap) return LGC_OK;
+  const int64_t room = min64(n, std::max<int64_t>(16 * need, kRoomKeys));
+  const int64_t cap = pow2_at_least(2 * room);
+  if (ctx->table_form == 0 && n >= 1024 && 24 * cap >= 16 * n + n / 8)
+    return table_to_dense(ctx, T, n, fv, fs, nf);
+  return table_grow(ctx, T, cap, fv, fs, nf);
+}
+
 int finish_svec(lgc_ctx* ctx, lgc_graph* g, const Table& T, const double* vals, lgc_svec** p,
                 lgc_stats* st_out, lgc_stats& st) {
   int32_t* d_idx = nullptr;
@@ -2737,8 +2586,13 @@ int prnibble_rounds(lgc_ctx* ctx, lgc_graph* g, PushWork& W, Table& T, int64_t& 
   lgc_stats& st = W.st;
   while (W.F.size > 0) {
     if (st.rounds >= max_rounds) return LGC_EMAXROUNDS;
-    if (!det && beta >= 1.0 && W.small_round(T, count)) {
-      status = W.device_rounds_prnibble(T, &count, alpha, cs, cn, eps, prm->rule,
+    if (rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, beta < 1.0)) {
+      // room for the rounds to come: the set grows with them, and a table
+      // that fills up costs another launch
+      if ((status = ensure_room_ahead(ctx, &T, count, W.F.edges, g->n, W.F.v.ptr, W.F.s.ptr,
+                                      W.F.size)) != LGC_OK)
+        return status;
+      status = W.device_rounds_prnibble(T, &count, alpha, cs, cn, eps, prm->rule, det, beta,
                                         max_rounds - st.rounds);
       if (status != LGC_OK) return status;
       continue;
@@ -2843,7 +2697,8 @@ int run_prnibble_set(lgc_ctx* ctx, lgc_graph* g, int64_t k, const int32_t* seeds
 
   PushWork W(ctx, g);
   Table T;
-  LGC_TRY(table_create(ctx, &T, 2 * (k + dsum), true));
+  if (dense_small(ctx, g->n)) LGC_TRY(table_create_dense(ctx, &T, g->n, true));
+  else LGC_TRY(table_create(ctx, &T, 2 * std::max<int64_t>(k + dsum, kRoomKeys), true));
   int64_t count = k;  // keys in T
   int status = LGC_OK;
   int32_t* d_x = nullptr;
