@@ -550,7 +550,7 @@ PULL_TRAFFIC = {"sources": [
                     (_CSRC + "diffuse.cu", "__device__ inline bool pull_qualifies(",
                      "// Deterministic pull, vertices of degree 1..kPullLight"),
                     (_CSRC + "diffuse.cu", "// Writes a heavy vertex's gathered value",
-                     "// The ordered fold acc <- RN(acc + s_k)"),
+                     "// Deterministic mode, vertices of degree (kPullLight, kDetBig]"),
                     (_CSRC + "diffuse.cu", "__device__ inline int round_scale(",
                      "// edgeMap, deterministic mode."),
                     (_CSRC + "fx128.cuh", None, None),
