@@ -294,6 +294,22 @@ int build_heavy_list(lgc_ctx* ctx, lgc_graph* g) {
   return st;
 }
 
+// 1 / d by degree (fp64lite.cuh), 16 bytes a degree.
+__global__ void recip_kernel(Recip* __restrict__ recip, int32_t n) {
+  for (int32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < n; d += gridDim.x * blockDim.x)
+    recip[d] = recip_of((double)max(d, 1));
+}
+
+int build_recip(lgc_ctx* ctx, lgc_graph* g) {
+  const int32_t n = (int32_t)std::min<int64_t>((int64_t)g->max_deg + 1, kRecipMax);
+  LGC_TRY(dalloc_t(ctx, &g->recip, (size_t)n));
+  recip_kernel<<<std::min(grid_for(n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(g->recip, n);
+  LGC_COUNT_LAUNCH(ctx);
+  LGC_CUDA_TRY(cudaGetLastError());
+  g->recip_n = n;
+  return LGC_OK;
+}
+
 }  // namespace
 
 namespace lgc {
@@ -880,6 +896,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     st = build_heavy_list(ctx, g);
     if (st == LGC_OK) st = build_big_segments(ctx, g);
     if (st == LGC_OK) st = build_light_items(ctx, g);
+    if (st == LGC_OK) st = build_recip(ctx, g);
   } while (0);
   if (st != LGC_OK) {
     dfree(ctx, g->off);
@@ -893,6 +910,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     dfree(ctx, g->det_mid);
     if (g->light_det != g->light) dfree(ctx, g->light_det);
     dfree(ctx, g->light);
+    dfree(ctx, g->recip);
     cudaStreamSynchronize(s);
     delete g;
     return st;
@@ -932,6 +950,7 @@ void lgc_graph_destroy(lgc_graph* g) {
   dfree(ctx, g->det_mid);
   if (g->light_det != g->light) dfree(ctx, g->light_det);
   dfree(ctx, g->light);
+  dfree(ctx, g->recip);
   cudaStreamSynchronize(ctx->stream);
   delete g;
 }

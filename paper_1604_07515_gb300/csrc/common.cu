@@ -8,6 +8,7 @@
 #include <unordered_map>
 
 #include "common.cuh"
+#include "lookback.cuh"
 #include "prim.cuh"
 
 namespace lgc {
@@ -61,10 +62,13 @@ void ctx_fini(lgc_ctx* ctx) {
   if (ctx->d_endpoints) cudaFree(ctx->d_endpoints);
   dfree(ctx, ctx->sort_status);
   dfree(ctx, ctx->sort_aux);
+  dfree(ctx, ctx->cmp);
   if (ctx->stream) cudaStreamSynchronize(ctx->stream);
   if (ctx->h_sort_err) cudaFreeHost(ctx->h_sort_err);
   ctx->sort_status = nullptr;
   ctx->sort_aux = nullptr;
+  ctx->cmp = nullptr;
+  ctx->cmp_cap = 0;
   ctx->sort_status_cap = 0;
   ctx->h_sort_err = nullptr;
   ctx->d_sort_err = nullptr;
@@ -275,49 +279,38 @@ __global__ void extract_kernel(Table T, const double* vals, Counters* C, uint32_
   }
 }
 
-// Dense extraction in vertex order: count the kept keys of each bitmap word,
-// then (after a scan of the counts) write them in ascending id.
-__device__ inline uint32_t dense_kept(const Table& T, const double* vals, int64_t w, int64_t n,
-                                      int positive_only) {
-  uint32_t m = T.bits[w];
-  if (positive_only) {
-    uint32_t k = 0;
-    while (m) {
-      const int b = __ffs(m) - 1;
-      m &= m - 1;
-      const int64_t v = w * 32 + b;
-      if (v < n && (vals ? vals[v] : T.dval[v]) > 0.0) k |= 1u << b;
-    }
-    return k;
+// Dense extraction in vertex order (words_compact): the kept keys of each
+// bitmap word, written with their values at their positions; *total becomes
+// their number.
+struct DenseKeptWord {
+  Table T;
+  const double* src;
+  int64_t n;
+  int positive_only;
+  __device__ uint32_t operator()(int64_t w, bool in) const {
+    const uint32_t m = in ? T.bits[w] : 0u;
+    if (!positive_only) return m;
+    return filter_words(
+        m, w, n, [&](int64_t v) { return src[v]; }, [](int64_t, double x) { return x > 0.0; });
   }
-  return m;
-}
-
-__global__ void dense_count_kernel(Table T, const double* vals, int64_t n, int positive_only,
-                                   int64_t* cnt) {
-  const int64_t words = (n + 31) / 32;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
-       w += (int64_t)gridDim.x * blockDim.x)
-    cnt[w] = __popc(dense_kept(T, vals, w, n, positive_only));
-}
-
-__global__ void dense_write_kernel(Table T, const double* vals, int64_t n, int positive_only,
-                                   const int64_t* pos, uint32_t* keys, double* out) {
-  const int64_t words = (n + 31) / 32;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
-       w += (int64_t)gridDim.x * blockDim.x) {
-    uint32_t m = dense_kept(T, vals, w, n, positive_only);
-    int64_t at = pos[w];
-    while (m) {
-      const int b = __ffs(m) - 1;
-      m &= m - 1;
-      const int64_t v = w * 32 + b;
+};
+struct ExtractOut {
+  const double* src;
+  uint32_t* keys;
+  double* vals;
+  int64_t cap;
+  int64_t* total;
+  __device__ int64_t put(int64_t at, int64_t v) const {
+    if (at < cap) {
       keys[at] = (uint32_t)v;
-      out[at] = vals ? vals[v] : T.dval[v];
-      at++;
+      vals[at] = src[v];
     }
+    return 0;
   }
-}
+  __device__ void finish(int64_t n, bool last, int64_t) const {
+    if (last) *total = n;
+  }
+};
 
 }  // namespace
 
@@ -356,39 +349,39 @@ int table_grow(lgc_ctx* ctx, Table* T, int64_t new_cap, const int32_t* fv, int32
 }
 
 int table_extract_sorted(lgc_ctx* ctx, const Table& T, const double* vals, int64_t n_vertices,
-                         int32_t** d_idx, double** d_val, int64_t* nnz, bool positive_only) {
+                         int32_t** d_idx, double** d_val, int64_t* nnz, bool positive_only,
+                         int64_t keys) {
   cudaStream_t st = ctx->stream;
   *d_idx = nullptr;
   *d_val = nullptr;
   *nnz = 0;
   if (T.dense) {
     const int64_t n = T.cap, words = (n + 31) / 32;
-    int64_t *cnt = nullptr, *tot = nullptr;
+    const double* src = vals ? vals : T.dval;
+    int64_t* tot = nullptr;
     uint32_t* k = nullptr;
     double* v = nullptr;
-    int s = dalloc_t(ctx, &cnt, words);
-    if (s == LGC_OK) s = dalloc_t(ctx, &tot, 1);
-    if (s == LGC_OK) {
-      dense_count_kernel<<<grid_for(words), kBlock, 0, st>>>(T, vals, n, positive_only, cnt);
-      LGC_COUNT_LAUNCH(ctx);
-      s = scan_i64(ctx, cnt, cnt, words, false, tot);
-    }
-    int64_t count = 0;
-    if (s == LGC_OK) {
+    int64_t cap = keys >= 0 && keys < n ? keys : n, count = 0;
+    int s = dalloc_t(ctx, &tot, 1);
+    while (s == LGC_OK) {
+      if ((s = dalloc_t(ctx, &k, cap)) != LGC_OK || (s = dalloc_t(ctx, &v, cap)) != LGC_OK) break;
+      if ((s = words_compact(ctx, DenseKeptWord{T, src, n, positive_only ? 1 : 0}, nullptr, words,
+                             ExtractOut{src, k, v, cap, tot})) != LGC_OK)
+        break;
       if (cudaMemcpyAsync(ctx->h_scratch, tot, 8, cudaMemcpyDeviceToHost, st) != cudaSuccess ||
-          cudaStreamSynchronize(st) != cudaSuccess)
+          cudaStreamSynchronize(st) != cudaSuccess) {
         s = LGC_ECUDA;
-      else
-        count = ctx->h_scratch[0];
+        break;
+      }
+      count = ctx->h_scratch[0];
+      if (count <= cap) break;
+      // more than the caller's count: once more, with room for them
+      dfree(ctx, k);
+      dfree(ctx, v);
+      k = nullptr;
+      v = nullptr;
+      cap = count;
     }
-    if (s == LGC_OK) s = dalloc_t(ctx, &k, count);
-    if (s == LGC_OK) s = dalloc_t(ctx, &v, count);
-    if (s == LGC_OK) {
-      dense_write_kernel<<<grid_for(words), kBlock, 0, st>>>(T, vals, n, positive_only, cnt, k, v);
-      LGC_COUNT_LAUNCH(ctx);
-      if (cudaGetLastError() != cudaSuccess) s = LGC_ECUDA;
-    }
-    dfree(ctx, cnt);
     dfree(ctx, tot);
     if (s != LGC_OK) {
       dfree(ctx, k);

@@ -13,6 +13,7 @@
 #include <vector>
 
 #include "../../include/lgc.h"
+#include "fp64lite.cuh"
 
 #define LGC_CUDA_TRY(expr)                                  \
   do {                                                      \
@@ -218,6 +219,8 @@ struct lgc_ctx {
   uint64_t lb_ticket = 0;  // tickets taken so far from the auxiliary block's counter
   int* h_sort_err = nullptr;
   int* d_sort_err = nullptr;
+  uint32_t* cmp = nullptr;  // bitmap compactions: kept words and tile counts
+  int64_t cmp_cap = 0;
   // small pinned host block for per-round read-back
   lgc::Counters* h_counters = nullptr;
   lgc::Counters* d_counters = nullptr;
@@ -276,6 +279,8 @@ struct lgc_graph {
   int32_t* col = nullptr;  // device, nnz
   int32_t* deg = nullptr;  // device, n (int32 degree, read where off[] pairs would cost more)
   int32_t max_deg = 0;
+  lgc::Recip* recip = nullptr;  // 1 / d by degree d < recip_n (device)
+  int32_t recip_n = 0;
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
   int pull_batch = 8;          // edges per lane per batch in heavy pull gathers (tuned)
   int pull_group = 32;         // lanes per work item in heavy pull gathers (tuned)
@@ -421,10 +426,11 @@ int make_svec(lgc_ctx* ctx, const int32_t* d_idx, const double* d_val, int64_t n
               bool on_device, lgc_svec** out);
 
 // Extracts {(key - 1, value) : value > 0} from a table, sorted by vertex id.
-// vals == nullptr uses T.s[].val, else vals[slot].
+// vals == nullptr uses T.s[].val, else vals[slot].  keys: the table's key
+// count, where the caller knows it (the arrays' first size; -1: unknown).
 int table_extract_sorted(lgc_ctx* ctx, const Table& T, const double* vals, int64_t n_vertices,
                          int32_t** d_idx, double** d_val, int64_t* nnz,
-                         bool positive_only = true);
+                         bool positive_only = true, int64_t keys = -1);
 
 // Algorithm drivers (diffuse.cu, rwalk.cu, sweep.cu).  ctx supplies the
 // stream and scratch; g is read-only and may be shared by several contexts.
@@ -482,8 +488,8 @@ void profile_collect(lgc_ctx* ctx);
 #define LGC_COUNT_LAUNCH(ctx) ((ctx)->n_launches++)
 
 namespace lgc {
-// The flags of the context's look-back launches (one-launch scans, sorts
-// and compactions), once: LGC_ETIMEOUT if a look-back wait gave up, else
+// The flags of the context's look-back launches (one-launch scans and
+// sorts), once: LGC_ETIMEOUT if a look-back wait gave up, else
 // LGC_ECUDA if a partial sum left the status words' range or a launch's
 // tiles were out of step.  Call after the context's stream has synchronised.
 inline int sort_check(lgc_ctx* ctx) {

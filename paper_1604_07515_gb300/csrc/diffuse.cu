@@ -34,7 +34,9 @@
 #include <cooperative_groups.h>
 
 #include "common.cuh"
+#include "edges.cuh"
 #include "foldwarp.cuh"
+#include "fp64lite.cuh"
 #include "fx128.cuh"
 #include "lookback.cuh"
 #include "prim.cuh"
@@ -47,72 +49,9 @@ namespace lgc {
 namespace {
 
 constexpr int kEdgeItems = 4;
-constexpr int kEdgeTile = kBlock * kEdgeItems;  // edges per CTA tile
+constexpr int kEdgeTile = kBlock * kEdgeItems;  // edges per block and pass
 
 enum FrontierMode { kFmNone = 0, kFmThreshold = 1, kFmInserted = 2 };
-
-// The first index of a[0, n) (non-decreasing) whose entry exceeds x, found
-// by all 32 lanes of a warp (the same result in each): every step probes the
-// last entry of 32 equal chunks of the range and keeps the chunk where the
-// entries start to exceed x, so a search over n entries takes about
-// log32(n) dependent loads instead of log2(n).
-__device__ inline int64_t warp_upper_bound(const int64_t* a, int64_t n, int64_t x) {
-  const int lane = threadIdx.x & 31;
-  int64_t lo = 0, hi = n;  // the answer lies in [lo, hi]
-  while (hi - lo > 32) {
-    const int64_t step = (hi - lo + 31) / 32;
-    const int64_t pos = lo + (int64_t)(lane + 1) * step - 1;
-    const bool le = pos < hi && a[pos] <= x;  // true on a prefix of the lanes
-    const int c = __popc(__ballot_sync(0xffffffffu, le));
-    lo += (int64_t)c * step;
-    if (lo >= hi) return hi;
-    hi = min(hi, lo + step);
-  }
-  const bool le = lo + lane < hi && a[lo + lane] <= x;
-  return lo + __popc(__ballot_sync(0xffffffffu, le));
-}
-
-// Stages, for the block's record range [e0, e1), the exclusive prefix sums of
-// the sources owning those records into s_epos[0..cnt] (the last entry is
-// the end of the last staged source) and returns cnt <= kEdgeTile.  All
-// threads of the block must call it; the caller synchronizes after staging
-// its own per-source arrays.
-__device__ inline int stage_sources(const int64_t* epos, int64_t nf, int64_t total,
-                                    int64_t e0, int64_t e1, int64_t* s_i0, int64_t* s_i1,
-                                    int64_t* s_epos) {
-  const int warp = threadIdx.x >> 5;
-  if (warp < 2) {  // the two ends at once, each by a whole warp
-    const int64_t b = warp_upper_bound(epos, nf, warp == 0 ? e0 : e1 - 1) - 1;
-    if ((threadIdx.x & 31) == 0) *(warp == 0 ? s_i0 : s_i1) = b;
-  }
-  __syncthreads();
-  const int64_t i0 = *s_i0;
-  int64_t c = *s_i1 - i0 + 1;
-  if (i0 < 0 || c < 0) c = 0;
-  if (c > kEdgeTile) c = kEdgeTile;
-  const int cnt = (int)c;
-  for (int j = threadIdx.x; j <= cnt; j += kBlock)
-    s_epos[j] = (i0 + j < nf) ? epos[i0 + j] : total;
-  __syncthreads();
-  return cnt;
-}
-
-// Source j (within the staged range) of record e and its local index *q;
-// -1 if e is not a record of a staged source.
-__device__ inline int find_source(const int64_t* s_epos, int cnt, int64_t e, int64_t* q) {
-  int lo = 0, hi = cnt;
-  while (lo < hi) {
-    const int mid = (lo + hi) >> 1;
-    if (s_epos[mid] <= e) lo = mid + 1;
-    else hi = mid;
-  }
-  const int j = lo - 1;
-  if (j < 0) return -1;
-  const int64_t local = e - s_epos[j];
-  if (local >= s_epos[j + 1] - s_epos[j]) return -1;
-  *q = local;
-  return j;
-}
 
 // Adds every thread's count n into *counter with one atomic per block (a
 // per-warp atomic on one address queues when a launch has many warps).  All
@@ -280,46 +219,31 @@ __global__ void vmap_hkpr_kernel(int64_t nf, const int32_t* __restrict__ fv,
 }
 
 // ---------------------------------------------------------------------------
-// edgeMap, atomic mode.  Edge-balanced: CTA tile k covers edges
-// [k*kEdgeTile, (k+1)*kEdgeTile) of the frontier's concatenated adjacency
-// lists; the tile's sources are found by binary search in the exclusive
-// prefix sums of the frontier degrees and staged in shared memory, and each
-// thread then finds its edge's source there.  Consecutive threads read
-// consecutive col[] entries.
+// edgeMap, atomic mode, edge-balanced over warps (edges.cuh).  Each thread
+// takes kEdgeItems edges through the phases side by side: all columns, first
+// probes, slots, adds and crossings.  Consecutive threads read consecutive
+// col[] entries.
 // ---------------------------------------------------------------------------
-// The tiles [first tile, ntiles) of the edge push with the given stride.
+// The warps [warp, nwarps) of the edge push.
 __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
                                         const int32_t* __restrict__ deg, const double* share,
                                         const int64_t* epos, const int64_t* foff, int64_t nf,
                                         int64_t E, Table D, double c, int fmode, int32_t* nfv,
                                         int32_t* nfs, int32_t ncap, Counters* C) {
-  __shared__ int64_t s_epos[kEdgeTile + 1];
-  __shared__ int64_t s_off[kEdgeTile];
-  __shared__ double s_share[kEdgeTile];
-  __shared__ int64_t s_i0, s_i1;
-  const int64_t ntiles = (E + kEdgeTile - 1) / kEdgeTile;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;  // counted once per block
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t e0 = tile * kEdgeTile;
-    const int64_t e1 = min(E, e0 + kEdgeTile);
-    const int cntsrc = stage_sources(epos, nf, E, e0, e1, &s_i0, &s_i1, s_epos);
-    const int64_t i0 = s_i0;
-    for (int j = threadIdx.x; j < cntsrc; j += kBlock) {
-      s_off[j] = foff[i0 + j];
-      s_share[j] = share[i0 + j];
-    }
-    __syncthreads();
+  warp_edges<kEdgeItems>(epos, foff, nf, E, warp, nwarps, [&](const int32_t* src,
+                                                              const int64_t* at) {
     int32_t w[kEdgeItems];
     double sh[kEdgeItems];
 #pragma unroll
     for (int k = 0; k < kEdgeItems; k++) {
-      const int64_t e = e0 + k * kBlock + threadIdx.x;
       w[k] = -1;
-      int64_t q;
-      const int j = e < e1 ? find_source(s_epos, cntsrc, e, &q) : -1;
-      if (j >= 0) {
-        w[k] = col[s_off[j] + q];
-        sh[k] = s_share[j];
+      sh[k] = 0.0;
+      if (src[k] >= 0) {
+        w[k] = col[at[k]];
+        sh[k] = share[src[k]];
       }
     }
     // Resolve every item's slot before any atomic, so the first-probe loads
@@ -379,8 +303,7 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
       nins += ins[k];
       frontier_append(pred[k], w[k], slot[k], dw[k], nfv, nfs, C, ncap);
     }
-    __syncthreads();
-  }
+  });
   flush_count(nins, &C->inserted);
 }
 
@@ -402,66 +325,58 @@ __global__ void __launch_bounds__(kBlock)
 // afterwards by the dense filter.  Also used for the last HK-PR level (no
 // frontier) in either table form.
 // ---------------------------------------------------------------------------
+constexpr int kRedItems = 8;
+
 __global__ void __launch_bounds__(kBlock)
     emap_red_kernel(const int32_t* __restrict__ col, const double* __restrict__ share,
                     const int64_t* __restrict__ epos, const int64_t* __restrict__ foff,
                     int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev, Table D,
                     Counters* C) {
-  __shared__ int64_t s_epos[kEdgeTile + 1];
-  __shared__ int64_t s_off[kEdgeTile];
-  __shared__ double s_share[kEdgeTile];
-  __shared__ int64_t s_i0, s_i1;
   const int64_t E = min(E_host, *E_dev);
-  const int64_t ntiles = (E + kEdgeTile - 1) / kEdgeTile;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;  // counted once per block
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t e0 = tile * kEdgeTile;
-    const int64_t e1 = min(E, e0 + kEdgeTile);
-    const int cntsrc = stage_sources(epos, nf, E, e0, e1, &s_i0, &s_i1, s_epos);
-    const int64_t i0 = s_i0;
-    for (int j = threadIdx.x; j < cntsrc; j += kBlock) {
-      s_off[j] = foff[i0 + j];
-      s_share[j] = share[i0 + j];
-    }
-    __syncthreads();
-    int32_t w[kEdgeItems];
-    double sh[kEdgeItems];
+  warp_edges<kRedItems>(epos, foff, nf, E, warp, nwarps, [&](const int32_t* src,
+                                                             const int64_t* at) {
+    int32_t w[kRedItems];
+    double sh[kRedItems];
 #pragma unroll
-    for (int k = 0; k < kEdgeItems; k++) {
-      const int64_t e = e0 + k * kBlock + threadIdx.x;
+    for (int k = 0; k < kRedItems; k++) {
       w[k] = -1;
-      int64_t q;
-      const int j = e < e1 ? find_source(s_epos, cntsrc, e, &q) : -1;
-      if (j >= 0) {
-        w[k] = col[s_off[j] + q];
-        sh[k] = s_share[j];
+      sh[k] = 0.0;
+      if (src[k] >= 0) {
+        w[k] = col[at[k]];
+        sh[k] = share[src[k]];
       }
     }
-    int ins[kEdgeItems];
     if (D.dense) {
-      // nothing waits here: the add and the presence bit are both reductions
-      // (results unused); the keys this round inserted are counted by the
-      // caller from the bitmap's population before and after
+      // nothing waits for a result here: the add and the presence bit are both
+      // reductions; the keys this round inserted are counted by the caller
+      // from the bitmap's population before and after.  A bit that is set
+      // already is not set again (a read that may be served from L1: stale, it
+      // only misses bits)
+      uint32_t b[kRedItems];
 #pragma unroll
-      for (int k = 0; k < kEdgeItems; k++) {
-        ins[k] = 0;
-        if (w[k] < 0) continue;
-        atomicAdd(&D.dval[w[k]], sh[k]);
-        atomicOr(&D.bits[w[k] >> 5], 1u << (w[k] & 31));
+      for (int k = 0; k < kRedItems; k++) {
+        b[k] = w[k] >= 0 ? D.bits[w[k] >> 5] : ~0u;
+        if (w[k] >= 0) atomicAdd(&D.dval[w[k]], sh[k]);
+      }
+#pragma unroll
+      for (int k = 0; k < kRedItems; k++) {
+        const uint32_t m = 1u << (w[k] & 31);
+        if (!(b[k] & m)) atomicOr(&D.bits[w[k] >> 5], m);
       }
     } else {
 #pragma unroll
-      for (int k = 0; k < kEdgeItems; k++) {
-        ins[k] = 0;
+      for (int k = 0; k < kRedItems; k++) {
         if (w[k] < 0) continue;
-        const int64_t s = ht_find_or_insert(D, w[k], &ins[k], &C->err);
+        int ins = 0;
+        const int64_t s = ht_find_or_insert(D, w[k], &ins, &C->err);
         if (s >= 0) atomicAdd(&D.s[s].val, sh[k]);
+        nins += ins;
       }
     }
-#pragma unroll
-    for (int k = 0; k < kEdgeItems; k++) nins += ins[k];
-    __syncthreads();
-  }
+  });
   flush_count(nins, &C->inserted);
 }
 
@@ -676,31 +591,20 @@ __global__ void bits_pop_kernel(const uint32_t* __restrict__ bits, int64_t words
 
 // Filter of a dense set, in ascending vertex order: vertex v qualifies when it
 // is a key and its value reaches c*d(v) (kFmThreshold) or always
-// (kFmInserted); the qualifying vertices are compacted in one launch
-// (compact_words_kernel), which also sums their degrees.
-__device__ inline uint32_t dense_qualifying(const Table& D, const int32_t* __restrict__ deg,
-                                            int64_t w, int64_t n, double c, int fmode) {
-  uint32_t m = D.bits[w];
-  if (fmode != kFmThreshold) return m;
-  uint32_t q = 0;
-  while (m) {
-    const int b = __ffs(m) - 1;
-    m &= m - 1;
-    const int64_t v = w * 32 + b;
-    if (v < n && D.dval[v] >= c * (double)deg[v]) q |= 1u << b;
-  }
-  return q;
-}
-
-// The filter's bitmap word w, for compact_words_kernel.
+// (kFmInserted); the qualifying vertices are compacted (words_compact), their
+// degrees summed.
 struct DenseQualWord {
   Table D;
   const int32_t* deg;
   int64_t n;
-  double c;
+  LiteThr c;
   int fmode;
-  __device__ uint32_t operator()(int64_t w) const {
-    return dense_qualifying(D, deg, w, n, c, fmode);
+  __device__ uint32_t operator()(int64_t w, bool in) const {
+    const uint32_t m = in ? D.bits[w] : 0u;
+    if (fmode != kFmThreshold) return m;
+    return filter_words(
+        m, w, n, [&](int64_t v) { return D.dval[v]; },
+        [&](int64_t v, double x) { return lite_reaches(x, c, deg[v]); });
   }
 };
 
@@ -737,7 +641,7 @@ __global__ void pull_scatter_kernel(int64_t nf, const int32_t* __restrict__ fv,
 }
 
 __device__ inline bool pull_qualifies(double acc, int64_t d, double c, int fmode) {
-  if (fmode == kFmThreshold) return acc >= c * (double)d;
+  if (fmode == kFmThreshold) return lite_reaches(acc, lite_thr(c), (int32_t)d);
   return fmode == kFmInserted;
 }
 
@@ -1061,9 +965,17 @@ __global__ void share_range_kernel(int64_t nf, const double* __restrict__ share,
 // array the gathers read (pull_scatter_kernel's membership encoding) and, in
 // atomic mode (range non-null, zeroed before), the shares' exponent range
 // reduced here; a pull round needs no push records.
+// The denominators' reciprocals 1 / (m d) by degree d < tab_n, m = j + 1 (1 on
+// the last level), come from recip (recip_level_kernel; null: divide).
+__global__ void recip_level_kernel(Recip* __restrict__ recip, int32_t tab_n, double m) {
+  for (int32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < tab_n; d += gridDim.x * blockDim.x)
+    recip[d] = recip_of(m * (double)max(d, 1));
+}
+
 __global__ void vmap_hkpr_pull_kernel(int64_t nf, const int32_t* __restrict__ fv,
                                       const int32_t* __restrict__ fs, Table S, Table P,
                                       const int32_t* __restrict__ deg, double t, int j, int last,
+                                      const Recip* __restrict__ recip, int32_t tab_n,
                                       double* __restrict__ sh, int32_t* __restrict__ range,
                                       Counters* C) {
   int emin = 0, emax = 0;
@@ -1078,7 +990,8 @@ __global__ void vmap_hkpr_pull_kernel(int64_t nf, const int32_t* __restrict__ fv
       const int64_t d = deg[v];
       const int64_t ps = tb_find_or_insert(P, v, &ins, &C->err);
       if (ps >= 0) *tb_val(P, ps) = *tb_val(P, ps) + r;
-      const double x = last ? r / (double)d : (t * r) / ((double)(j + 1) * (double)d);
+      const double a = last ? r : t * r, b = last ? (double)d : (double)(j + 1) * (double)d;
+      const double x = d < tab_n ? div_by(a, recip[d], b) : a / b;
       sh[v] = pull_member(x) ? x : -0.0;
       range_take(x, emin, emax);
     }
@@ -1345,40 +1258,26 @@ __global__ void __launch_bounds__(kBlock)
                         const double* __restrict__ share, const int64_t* __restrict__ epos,
                         const int64_t* __restrict__ foff, int64_t nf, int64_t R, int self_rec,
                         uint32_t* __restrict__ rkey, double* __restrict__ rval) {
-  __shared__ int64_t s_epos[kEdgeTile + 1];
-  __shared__ int64_t s_off[kEdgeTile];
-  __shared__ double s_share[kEdgeTile];
-  __shared__ int32_t s_v[kEdgeTile];
-  __shared__ int64_t s_i0, s_i1;
-  const int64_t ntiles = (R + kEdgeTile - 1) / kEdgeTile;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t e0 = tile * kEdgeTile;
-    const int64_t e1 = min(R, e0 + kEdgeTile);
-    const int cntsrc = stage_sources(epos, nf, R, e0, e1, &s_i0, &s_i1, s_epos);
-    const int64_t i0 = s_i0;
-    for (int j = threadIdx.x; j < cntsrc; j += kBlock) {
-      s_off[j] = foff[i0 + j];
-      s_share[j] = share[i0 + j];
-      s_v[j] = fv[i0 + j];
-    }
-    __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  int64_t e0 = warp * 32 * kEdgeItems;  // the tile's first record
+  warp_edges<kEdgeItems>(epos, foff, nf, R, warp, nwarps, [&](const int32_t* src,
+                                                              const int64_t* at) {
+#pragma unroll
     for (int k = 0; k < kEdgeItems; k++) {
-      const int64_t e = e0 + k * kBlock + threadIdx.x;
-      int64_t q = 0;
-      const int j = e < e1 ? find_source(s_epos, cntsrc, e, &q) : -1;
-      if (j >= 0) {
-        if (self_rec && q == 0) {
-          rkey[e] = (uint32_t)s_v[j];
-          rval[e] = 0.0;
-        } else {
-          if (self_rec) q -= 1;
-          rkey[e] = (uint32_t)col[s_off[j] + q];
-          rval[e] = s_share[j];
-        }
+      if (src[k] < 0) continue;
+      const int64_t e = e0 + 32 * k + lane;
+      if (self_rec && at[k] == foff[src[k]]) {
+        rkey[e] = (uint32_t)fv[src[k]];
+        rval[e] = 0.0;
+      } else {
+        rkey[e] = (uint32_t)col[at[k] - (self_rec ? 1 : 0)];
+        rval[e] = share[src[k]];
       }
     }
-    __syncthreads();
-  }
+    e0 += nwarps * 32 * kEdgeItems;
+  });
 }
 
 __global__ void head_flags_kernel(const uint32_t* __restrict__ rkey, int64_t R,
@@ -1719,6 +1618,7 @@ struct PushWork {
   DBuf<Counters> xcn;
   DBuf<RoundsState> xst;
   RoundsMem rmem;
+  DBuf<Recip> recip;  // HK-PR pull rounds: 1 / ((j + 1) d) by degree
   lgc_stats st{};
   explicit PushWork(lgc_ctx* c, lgc_graph* gr) : ctx(c), g(gr) {}
   ~PushWork() {
@@ -1742,6 +1642,7 @@ struct PushWork {
     xcn.release(ctx);
     xst.release(ctx);
     rmem.release(ctx);
+    recip.release(ctx);
     share.release(ctx);
     cnt.release(ctx);
     epos.release(ctx);
@@ -1842,16 +1743,8 @@ struct PushWork {
       }
       if (fmode != kFmNone) {  // the qualifying keys in ascending id, with their degrees
         const int64_t words = (g->n + 31) / 32;
-        const int64_t ntiles = ceil_div(words, kCmpTileWords);
-        uint32_t epoch;
-        unsigned long long *ticket, t0;
-        LGC_TRY(lb_begin(ctx, ntiles, &epoch, &ticket, &t0));
-        compact_words_kernel<DenseQualWord><<<(unsigned)ntiles, kBlock, 0, s>>>(
-            DenseQualWord{D, g->deg, g->n, c, fmode}, words, ntiles, g->deg, G.v.ptr, G.s.ptr,
-            ncap, ticket, t0, ctx->sort_status, epoch, ctx->d_sort_err, ctx->d_counters);
-        LGC_COUNT_LAUNCH(ctx);
-        LGC_CUDA_TRY(cudaGetLastError());
-        lb_commit(ctx, ntiles);
+        LGC_TRY(words_compact(ctx, DenseQualWord{D, g->deg, g->n, lite_thr(c), fmode}, nullptr, words,
+                              FrontierOut{g->deg, G.v.ptr, G.s.ptr, ncap, ctx->d_counters}));
       }
       int st = read_counters(out);
       if (ctx->profile && nrec > 0 && !ctx->prof_pending.empty())
@@ -2418,7 +2311,7 @@ int finish_svec(lgc_ctx* ctx, lgc_graph* g, const Table& T, const double* vals, 
   int32_t* d_idx = nullptr;
   double* d_val = nullptr;
   int64_t nnz = 0;
-  LGC_TRY(table_extract_sorted(ctx, T, vals, g->n, &d_idx, &d_val, &nnz));
+  LGC_TRY(table_extract_sorted(ctx, T, vals, g->n, &d_idx, &d_val, &nnz, true, st.touched));
   int s = make_svec(ctx, d_idx, d_val, nnz, ctx->result_on_device, p);
   dfree(ctx, d_idx);
   dfree(ctx, d_val);
@@ -2964,10 +2857,22 @@ int run_hkpr(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_hkpr_params* prm, 
           status = LGC_ECUDA;
           break;
         }
+        // one reciprocal per degree in place of a division per vertex, where
+        // there are more vertices than degrees (b = (j + 1) d is exact and
+        // within div_by's range)
+        const int32_t tab_n =
+            nf >= 4 * (int64_t)g->max_deg && j < (1 << 16) ? std::min(g->max_deg + 1, kRecipMax) : 0;
+        if (tab_n > 0) {
+          if ((status = W.recip.reserve(ctx, tab_n)) != LGC_OK) break;
+          recip_level_kernel<<<std::min(grid_for(tab_n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(
+              W.recip.ptr, tab_n, last ? 1.0 : (double)(j + 1));
+          LGC_COUNT_LAUNCH(ctx);
+        }
         // per vertex: fv, fs 8, r 8, degree 4, p read-modify-write 16, share 8
         ProfScope ps(ctx, LGC_PROF_VERTEXMAP, 44.0 * nf);
         vmap_hkpr_pull_kernel<<<vgrid(ctx, nf), kBlock, 0, ctx->stream>>>(
-            nf, W.F.v.ptr, W.F.s.ptr, Rc, P, g->deg, t, j, last ? 1 : 0, W.psh.ptr,
+            nf, W.F.v.ptr, W.F.s.ptr, Rc, P, g->deg, t, j, last ? 1 : 0, W.recip.ptr, tab_n,
+            W.psh.ptr,
             det ? nullptr : W.prange.ptr, ctx->d_counters);
         LGC_COUNT_LAUNCH(ctx);
       } else {

@@ -1,7 +1,7 @@
 // Decoupled look-back (Merrill and Garland's single-pass prefix scan): the
-// status words the one-launch scans, sorts and compactions publish per tile,
-// the warp-wide look-back over them, and the one-launch ordered compaction
-// of a vertex bitmap (or of one computed word by word).
+// status words the one-launch scans and sorts publish per tile and the
+// warp-wide look-back over them; and the ordered compaction of a vertex
+// bitmap (or of one computed word by word), which does without a look-back.
 //
 // A status word: epoch (24 bits) | state (2 bits: aggregate, inclusive
 // prefix) | value (38 bits).  Every launch (every radix pass) has its own
@@ -64,125 +64,170 @@ __device__ inline int64_t lookback_warp(const unsigned long long* status, int64_
 }
 
 // ---------------------------------------------------------------------------
-// Ordered compaction of a vertex bitmap in one launch.  The bitmap's words
-// come from a functor (word(w): the set bits of word w, for w < words), so
-// that a filter can compute them on the fly.  Tiles of
-// kCmpTileWords words are taken in start order (a counter); warp w of a tile
-// takes 32 * kCmpRounds consecutive words, 32 per round, lane l word l of
-// the round; the tile's count goes to the status array and its offset comes
-// from a decoupled look-back over the earlier tiles (one status word per
-// tile, as in the sort).  A set bit's vertex is written at its position:
-// a round's words are taken in turn, lane l writing bit l, so a warp's
-// stores are consecutive.
+// Ordered compaction of a vertex bitmap in two launches.  The bitmap's words
+// come from a functor called by whole warps (word(w, in): lane l asks for
+// word w = the warp's first + l, `in` saying whether it has one), so that a
+// filter can compute them on the fly, 32 vertices of a word at a time with
+// one lane each.  words_count_kernel keeps the words and counts the set bits
+// of every tile of kCmpTileWords words; words_write_kernel adds up the counts
+// of the tiles before its own (one L2 round trip for a thread's loads) and
+// hands every set bit's vertex v to out.put(position, v), lane l with bit l
+// of one word after another, so a warp's positions are consecutive.  put
+// returns a weight, and out.finish(entries so far, is this the last tile,
+// weight of the block's vertices) is called by one thread per tile.
+//
+// 4.2M vertices, 2.4M of them kept: 3 + 20 us (one launch with a decoupled
+// look-back 27 us); the dense filter over them 21 + 12 us (30-37 us, with the
+// lanes walking their own words' bits and FP64 compares, which alone bound it
+// at 40 us); a look-back by the whole block instead of one warp 45-50 us (its
+// polls crowd out the words it waits for).
 // ---------------------------------------------------------------------------
-constexpr int kCmpRounds = 1;
-constexpr int64_t kCmpTileWords = (int64_t)kBlock * kCmpRounds;  // 256 words
+constexpr int kCmpWarpWords = 8;  // words a warp writes: one batch of loads each
+constexpr int64_t kCmpTileWords = kCmpWarpWords * (kBlock / 32);
 
 template <class WordFn>
 __global__ void __launch_bounds__(kBlock)
-    compact_words_kernel(WordFn word, int64_t words, int64_t ntiles,
-                        const int32_t* __restrict__ deg, int32_t* nfv, int32_t* nfs,
-                        int32_t ncap, unsigned long long* ticket,
-                        unsigned long long ticket0, unsigned long long* status, uint32_t epoch,
-                        int* err, Counters* C) {
-  __shared__ int64_t s_tile, s_base;
-  __shared__ int s_wtot[kBlock / 32];
-  __shared__ int64_t s_deg[kBlock / 32];
+    words_count_kernel(WordFn word, int64_t words, uint32_t* __restrict__ kept,
+                       int32_t* __restrict__ cnt) {
+  __shared__ int s_tot[kBlock / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  if (threadIdx.x == 0) s_tile = (int64_t)(atomicAdd(ticket, 1ull) - ticket0);
+  const int64_t w = (int64_t)blockIdx.x * kCmpTileWords + warp * kCmpWarpWords + lane;
+  const bool in = lane < kCmpWarpWords && w < words;
+  const uint32_t q = word(w, in);
+  if (kept && in) kept[w] = q;
+  const int c = __reduce_add_sync(0xffffffffu, __popc(q));
+  if (lane == 0) s_tot[warp] = c;
   __syncthreads();
-  const int64_t tile = s_tile;
-  if (tile < 0 || tile >= ntiles) {  // a ticket count out of step with the host's: flagged
-    if (threadIdx.x == 0) atomicOr(err, 4);
-    return;
-  }
-  const int64_t wbase = tile * kCmpTileWords + (int64_t)warp * (32 * kCmpRounds);
-  uint32_t q[kCmpRounds];
-  int pre[kCmpRounds];  // set bits before this lane's word in the warp's words
-  int run = 0;
-#pragma unroll
-  for (int k = 0; k < kCmpRounds; k++) {
-    const int64_t w = wbase + 32 * k + lane;
-    q[k] = w < words ? word(w) : 0u;
-    const int c = __popc(q[k]);
-    int inc = c;
-    for (int o = 1; o < 32; o <<= 1) {
-      const int y = __shfl_up_sync(0xffffffffu, inc, o);
-      if (lane >= o) inc += y;
-    }
-    pre[k] = run + inc - c;
-    run += __shfl_sync(0xffffffffu, inc, 31);
-  }
-  if (lane == 0) s_wtot[warp] = run;
-  __syncthreads();
-  if (threadIdx.x < 32) {
-    int64_t tot = 0;  // every lane of warp 0 sums the warps' counts
-    for (int w = 0; w < kBlock / 32; w++) tot += s_wtot[w];
-    __syncwarp();
-    volatile unsigned long long* st = status + tile;
-    if (threadIdx.x == 0) {
-      int64_t run = 0;
-      for (int w = 0; w < kBlock / 32; w++) {  // exclusive over warps
-        const int c = s_wtot[w];
-        s_wtot[w] = (int)run;
-        run += c;
-      }
-      *st = lb_word(epoch, tile == 0 ? kLbInclusive : kLbAggregate, (uint64_t)tot);
-    }
-    const int64_t excl = lookback_warp(status, tile, epoch, err);
-    if (threadIdx.x == 0) {
-      if (tile > 0) *st = lb_word(epoch, kLbInclusive, (uint64_t)(excl + tot));
-      s_base = excl;
-      if (tile == ntiles - 1) C->next_size = (int32_t)(excl + tot);
-    }
-  }
-  __syncthreads();
-  const int64_t wb = s_base + s_wtot[warp];
-  const uint32_t below = (1u << lane) - 1u;
-  int64_t dsum = 0;
-#pragma unroll
-  for (int k = 0; k < kCmpRounds; k++) {
-    if (!__any_sync(0xffffffffu, q[k] != 0u)) continue;
-    for (int j0 = 0; j0 < 32; j0 += 8) {
-      int32_t dk[8];
-#pragma unroll
-      for (int j = 0; j < 8; j++) {
-        const uint32_t qj = __shfl_sync(0xffffffffu, q[k], j0 + j);
-        const int pj = __shfl_sync(0xffffffffu, pre[k], j0 + j);
-        dk[j] = 0;
-        if ((qj >> lane) & 1u) {
-          const int64_t v = (wbase + 32 * k + j0 + j) * 32 + lane;
-          const int64_t at = wb + pj + __popc(qj & below);
-          if (at < ncap) {
-            nfv[at] = (int32_t)v;
-            nfs[at] = (int32_t)v;
-          } else {
-            atomicOr(&C->err, kErrFrontierOverflow);
-          }
-          if (deg) dk[j] = deg[v];
-        }
-      }
-#pragma unroll
-      for (int j = 0; j < 8; j++) dsum += dk[j];
-    }
-  }
-  if (deg) {
-    for (int o = 16; o > 0; o >>= 1) dsum += __shfl_xor_sync(0xffffffffu, dsum, o);
-    if (lane == 0) s_deg[warp] = dsum;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int64_t t = 0;
-      for (int w = 0; w < kBlock / 32; w++) t += s_deg[w];
-      if (t) atomicAdd((unsigned long long*)&C->next_edges, (unsigned long long)t);
-    }
+  if (threadIdx.x == 0) {
+    int t = 0;
+    for (int k = 0; k < kBlock / 32; k++) t += s_tot[k];
+    cnt[blockIdx.x] = t;
   }
 }
 
-// The host side of a look-back launch over `ntiles` tiles: room in the
-// context's status array, a fresh epoch, and the first ticket of the launch
-// (lb_commit after a successful launch takes its tickets).
-int lb_begin(lgc_ctx* ctx, int64_t ntiles, uint32_t* epoch, unsigned long long** ticket,
-             unsigned long long* ticket0);
-inline void lb_commit(lgc_ctx* ctx, int64_t ntiles) { ctx->lb_ticket += (uint64_t)ntiles; }
+template <class Out>
+__global__ void __launch_bounds__(kBlock)
+    words_write_kernel(const uint32_t* __restrict__ kept, int64_t words,
+                       const int32_t* __restrict__ cnt, Out out) {
+  __shared__ int64_t s_pre[kBlock / 32];
+  __shared__ int s_wtot[kBlock / 32];
+  __shared__ int64_t s_sum[kBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t tile = blockIdx.x;
+  const int64_t wbase = tile * kCmpTileWords + warp * kCmpWarpWords;
+  const uint32_t q = lane < kCmpWarpWords && wbase + lane < words ? kept[wbase + lane] : 0u;
+  int64_t p = 0;
+  for (int64_t i = threadIdx.x; i < tile; i += kBlock) p += cnt[i];
+  for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
+  const int c = __popc(q);
+  int pre = c;  // set bits of the warp's words before this lane's
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, pre, o);
+    if (lane >= o) pre += y;
+  }
+  if (lane == 31) s_wtot[warp] = pre;
+  if (lane == 0) s_pre[warp] = p;
+  pre -= c;
+  __syncthreads();
+  int64_t at = 0, tot = 0;
+  for (int w = 0; w < kBlock / 32; w++) {
+    at += s_pre[w];
+    tot += s_wtot[w];
+  }
+  tot += at;  // entries through this tile
+  for (int w = 0; w < warp; w++) at += s_wtot[w];
+  const uint32_t below = (1u << lane) - 1u;
+  int64_t sum = 0;
+  if (__any_sync(0xffffffffu, q != 0u)) {
+    int64_t x[kCmpWarpWords];
+#pragma unroll
+    for (int j = 0; j < kCmpWarpWords; j++) {
+      const uint32_t qj = __shfl_sync(0xffffffffu, q, j);
+      const int pj = __shfl_sync(0xffffffffu, pre, j);
+      x[j] = (qj >> lane) & 1u ? out.put(at + pj + __popc(qj & below), (wbase + j) * 32 + lane)
+                               : 0;
+    }
+#pragma unroll
+    for (int j = 0; j < kCmpWarpWords; j++) sum += x[j];
+  }
+  for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (lane == 0) s_sum[warp] = sum;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    int64_t t = 0;
+    for (int w = 0; w < kBlock / 32; w++) t += s_sum[w];
+    out.finish(tot, tile == gridDim.x - 1, t);
+  }
+}
+
+// The bits of word w of a bitmap whose vertices v (< n) pass keep(v, x), by a
+// whole warp: the words of its first kCmpWarpWords lanes, the lanes taking a
+// word's vertices side by side.  x = load(v); all words' loads in flight.
+template <class Load, class Keep>
+__device__ inline uint32_t filter_words(uint32_t m, int64_t w, int64_t n, Load&& load,
+                                        Keep&& keep) {
+  const int lane = threadIdx.x & 31;
+  const int64_t wb = w - lane;
+  uint32_t q = 0;
+  if (!__any_sync(0xffffffffu, m != 0u)) return 0;
+  double x[kCmpWarpWords];
+  bool p[kCmpWarpWords];
+#pragma unroll
+  for (int j = 0; j < kCmpWarpWords; j++) {
+    const int64_t v = (wb + j) * 32 + lane;
+    p[j] = ((__shfl_sync(0xffffffffu, m, j) >> lane) & 1u) && v < n;
+    x[j] = p[j] ? load(v) : 0.0;
+  }
+#pragma unroll
+  for (int j = 0; j < kCmpWarpWords; j++) p[j] = p[j] && keep((wb + j) * 32 + lane, x[j]);
+#pragma unroll
+  for (int j = 0; j < kCmpWarpWords; j++) {
+    const uint32_t b = __ballot_sync(0xffffffffu, p[j]);
+    if (lane == j) q = b;
+  }
+  return q;
+}
+
+// Compaction into a frontier: vertex ids (twice: dense slots are vertices),
+// their number and the sum of their degrees.
+struct FrontierOut {
+  const int32_t* deg;
+  int32_t *v, *s;
+  int32_t cap;
+  Counters* C;
+  __device__ int64_t put(int64_t at, int64_t u) const {
+    if (at < cap) {
+      v[at] = (int32_t)u;
+      s[at] = (int32_t)u;
+    } else {
+      atomicOr(&C->err, kErrFrontierOverflow);
+    }
+    return deg ? deg[u] : 0;
+  }
+  __device__ void finish(int64_t n, bool last, int64_t weight) const {
+    if (last) C->next_size = (int32_t)n;
+    if (weight) atomicAdd((unsigned long long*)&C->next_edges, (unsigned long long)weight);
+  }
+};
+
+// The two launches on the context's scratch; bits: the words themselves where
+// word only reads them (nothing is kept then), else nullptr.
+int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt);
+
+template <class WordFn, class Out>
+int words_compact(lgc_ctx* ctx, const WordFn& word, const uint32_t* bits, int64_t words,
+                  const Out& out) {
+  if (words <= 0) return LGC_OK;
+  const unsigned ntiles = (unsigned)((words + kCmpTileWords - 1) / kCmpTileWords);
+  uint32_t* kept;
+  int32_t* cnt;
+  LGC_TRY(cmp_reserve(ctx, words, &kept, &cnt));
+  words_count_kernel<WordFn><<<ntiles, kBlock, 0, ctx->stream>>>(word, words,
+                                                                 bits ? nullptr : kept, cnt);
+  LGC_COUNT_LAUNCH(ctx);
+  words_write_kernel<Out><<<ntiles, kBlock, 0, ctx->stream>>>(bits ? bits : kept, words, cnt, out);
+  LGC_COUNT_LAUNCH(ctx);
+  return cudaGetLastError() == cudaSuccess ? LGC_OK : LGC_ECUDA;
+}
 
 }  // namespace lgc

@@ -581,7 +581,7 @@ int status_reserve(lgc_ctx* ctx, int64_t words, int epochs) {
   return LGC_OK;
 }
 
-// The running ticket counter of the one-launch scans and compactions: every
+// The running ticket counter of the one-launch scans: every
 // block of such a launch takes one ticket, so the launch's tiles are the
 // tickets [ctx->lb_ticket, ctx->lb_ticket + blocks), in the order the blocks
 // start (no clearing between launches).
@@ -691,36 +691,30 @@ int radix_sort_u32(lgc_ctx* ctx, uint32_t* keys, uint32_t* keys_tmp, int64_t n, 
                                             (int32_t*)nullptr, n, bits);
 }
 
-int lb_begin(lgc_ctx* ctx, int64_t ntiles, uint32_t* epoch, unsigned long long** ticket,
-             unsigned long long* ticket0) {
-  LGC_TRY(status_reserve(ctx, ntiles, 1));
-  *epoch = ++ctx->sort_epoch;
-  *ticket = lb_counter(ctx);
-  *ticket0 = ctx->lb_ticket;
+int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt) {
+  const int64_t ntiles = ceil_div(words, kCmpTileWords);
+  if (words + ntiles > ctx->cmp_cap) {
+    dfree(ctx, ctx->cmp);
+    ctx->cmp = nullptr;
+    ctx->cmp_cap = 0;
+    LGC_TRY(dalloc_t(ctx, &ctx->cmp, (size_t)(words + ntiles)));
+    ctx->cmp_cap = words + ntiles;
+  }
+  *kept = ctx->cmp;
+  *cnt = reinterpret_cast<int32_t*>(ctx->cmp + words);
   return LGC_OK;
 }
 
 namespace {
 struct BitsWord {
   const uint32_t* bits;
-  __device__ uint32_t operator()(int64_t w) const { return bits[w]; }
+  __device__ uint32_t operator()(int64_t w, bool in) const { return in ? bits[w] : 0u; }
 };
 }  // namespace
 
 int bits_compact(lgc_ctx* ctx, const uint32_t* bits, int64_t words, const int32_t* deg,
                  int32_t* out_v, int32_t* out_s, int32_t cap, Counters* C) {
-  if (words <= 0) return LGC_OK;
-  const int64_t ntiles = ceil_div(words, kCmpTileWords);
-  uint32_t epoch;
-  unsigned long long *ticket, t0;
-  LGC_TRY(lb_begin(ctx, ntiles, &epoch, &ticket, &t0));
-  compact_words_kernel<BitsWord><<<(unsigned)ntiles, kBlock, 0, ctx->stream>>>(
-      BitsWord{bits}, words, ntiles, deg, out_v, out_s, cap, ticket, t0, ctx->sort_status, epoch,
-      ctx->d_sort_err, C);
-  LGC_COUNT_LAUNCH(ctx);
-  if (cudaGetLastError() != cudaSuccess) return LGC_ECUDA;  // not launched: no tickets taken
-  lb_commit(ctx, ntiles);
-  return LGC_OK;
+  return words_compact(ctx, BitsWord{bits}, bits, words, FrontierOut{deg, out_v, out_s, cap, C});
 }
 
 // The multi-tile prefix sum in one launch (scan_lb_kernel).

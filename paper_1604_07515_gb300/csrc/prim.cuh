@@ -38,7 +38,7 @@ int radix_sort_u64_i32_with(lgc_ctx* ctx, uint64_t* keys, int32_t* vals, uint64_
 int radix_sort_u32(lgc_ctx* ctx, uint32_t* keys, uint32_t* keys_tmp, int64_t n, int bits);
 
 // Ordered compaction of the n-bit vertex bitmap bits (words = ceil(n / 32))
-// into out_v = out_s = the set vertices in ascending id, one launch: C's
+// into out_v = out_s = the set vertices in ascending id, two launches: C's
 // next_size becomes their number, and with deg their degrees are added to
 // C's next_edges; positions past cap are not written and flag
 // kErrFrontierOverflow in C's err.  C is device memory, zeroed by the caller

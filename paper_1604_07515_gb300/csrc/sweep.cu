@@ -37,6 +37,7 @@ constexpr int kTile = kBlock * kTileItems;
 // Also flags (bad != 0) entries that are not vertices of degree >= 1.
 __global__ void sweep_keys_kernel(const int32_t* __restrict__ idx, const double* __restrict__ val,
                                   int64_t n0, const int32_t* __restrict__ deg, int64_t n,
+                                  const Recip* __restrict__ recip, int32_t recip_n,
                                   uint64_t* __restrict__ key, int32_t* __restrict__ id,
                                   unsigned long long* npos, int* bad) {
   unsigned long long c = 0;
@@ -51,7 +52,8 @@ __global__ void sweep_keys_kernel(const int32_t* __restrict__ idx, const double*
     }
     uint64_t k = ~0ull;
     if (pv > 0.0) {
-      const double r = pv / (double)deg[v];
+      const int32_t d = deg[v];
+      const double r = d < recip_n ? div_by(pv, recip[d], (double)d) : pv / (double)d;
       k = 0x7FFFFFFFFFFFFFFFull - (uint64_t)__double_as_longlong(r);
       c++;
     }
@@ -364,6 +366,7 @@ __device__ inline int64_t seg_of(const int64_t* __restrict__ beg, int64_t B, int
 __global__ void bsweep_keys_kernel(const SweepIn* __restrict__ in,
                                    const int64_t* __restrict__ inoff,
                                    int64_t B, int64_t M, const int32_t* __restrict__ deg, int64_t n,
+                                   const Recip* __restrict__ recip, int32_t recip_n,
                                    uint64_t* __restrict__ key, int32_t* __restrict__ id,
                                    int32_t* __restrict__ seg, int64_t* __restrict__ keep,
                                    int* bad) {
@@ -379,9 +382,13 @@ __global__ void bsweep_keys_kernel(const SweepIn* __restrict__ in,
       pv = 0.0;
     }
     const bool pos = pv > 0.0;
-    key[i] = pos ? 0x7FFFFFFFFFFFFFFFull -
-                       (uint64_t)__double_as_longlong(pv / (double)deg[v])
-                 : ~0ull;
+    uint64_t k = ~0ull;
+    if (pos) {
+      const int32_t d = deg[v];
+      const double r = d < recip_n ? div_by(pv, recip[d], (double)d) : pv / (double)d;
+      k = 0x7FFFFFFFFFFFFFFFull - (uint64_t)__double_as_longlong(r);
+    }
+    key[i] = k;
     id[i] = v;
     seg[i] = (int32_t)b;
     keep[i] = pos ? 1 : 0;
@@ -557,7 +564,7 @@ int run_sweep(lgc_ctx* ctx, lgc_graph* g, const lgc_svec* p, lgc_cluster** out) 
     int grid = grid_for(n0);
     if (grid > (ctx->sms * 32)) grid = (ctx->sms * 32);
     // S1
-    sweep_keys_kernel<<<grid, kBlock, 0, s>>>(idx, val, n0, g->deg, g->n, key, id,
+    sweep_keys_kernel<<<grid, kBlock, 0, s>>>(idx, val, n0, g->deg, g->n, g->recip, g->recip_n, key, id,
                                                (unsigned long long*)misc, (int*)(misc + 3));
     LGC_COUNT_LAUNCH(ctx);
     LGC_CUDA_TRY(cudaGetLastError());
@@ -774,7 +781,8 @@ int run_sweep_batch(lgc_ctx* ctx, lgc_graph* g, int64_t B, const lgc_svec* const
       }
       const int grid = (int)std::min<int64_t>(ceil_div(M, kBlock), (ctx->sms * 32));
       // S1: keys of the positive entries, seed-major, ids ascending per seed
-      bsweep_keys_kernel<<<grid, kBlock, 0, s>>>(d_in, d_inoff, B, M, g->deg, g->n, key, id, seg,
+      bsweep_keys_kernel<<<grid, kBlock, 0, s>>>(d_in, d_inoff, B, M, g->deg, g->n, g->recip,
+                                                 g->recip_n, key, id, seg,
                                                  keep, d_err);
       LGC_COUNT_LAUNCH(ctx);
       if ((st = scan_i64(ctx, keep, pos, M, false, tot)) != LGC_OK) break;
