@@ -294,6 +294,44 @@ int build_heavy_list(lgc_ctx* ctx, lgc_graph* g) {
   return st;
 }
 
+// The largest (degree, lowest id first) below `below` into *top, packed
+// degree << 32 | ~id.
+__global__ void hot_kernel(const int32_t* __restrict__ deg, int64_t n, unsigned long long below,
+                           unsigned long long* __restrict__ top) {
+  unsigned long long m = 0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const unsigned long long k =
+        ((unsigned long long)(uint32_t)deg[v] << 32) | (uint32_t)~(uint32_t)v;
+    if (k < below && k > m) m = k;
+  }
+  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(top, m);
+}
+
+int build_hot(lgc_ctx* ctx, lgc_graph* g) {
+  if (g->max_deg < kHotDeg) return LGC_OK;
+  unsigned long long* top = nullptr;
+  unsigned long long last = ~0ull;
+  LGC_TRY(dalloc_t(ctx, &top, 1));
+  int st = LGC_OK;
+  for (int h = 0; h < kHot && st == LGC_OK; h++) {
+    if (cudaMemsetAsync(top, 0, 8, ctx->stream)) st = LGC_ECUDA;
+    hot_kernel<<<std::min(grid_for(g->n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(g->deg, g->n,
+                                                                                   last, top);
+    LGC_COUNT_LAUNCH(ctx);
+    if (cudaMemcpyAsync(ctx->h_scratch, top, 8, cudaMemcpyDeviceToHost, ctx->stream) ||
+        cudaStreamSynchronize(ctx->stream))
+      st = LGC_ECUDA;
+    if (st != LGC_OK) break;
+    last = (unsigned long long)ctx->h_scratch[0];
+    if ((int32_t)(last >> 32) < kHotDeg) break;
+    g->hot.v[h] = (int32_t)~(uint32_t)last;
+  }
+  dfree(ctx, top);
+  return st;
+}
+
 // 1 / d by degree (fp64lite.cuh), 16 bytes a degree.
 __global__ void recip_kernel(Recip* __restrict__ recip, int32_t n) {
   for (int32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < n; d += gridDim.x * blockDim.x)
@@ -897,6 +935,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     if (st == LGC_OK) st = build_big_segments(ctx, g);
     if (st == LGC_OK) st = build_light_items(ctx, g);
     if (st == LGC_OK) st = build_recip(ctx, g);
+    if (st == LGC_OK) st = build_hot(ctx, g);
   } while (0);
   if (st != LGC_OK) {
     dfree(ctx, g->off);

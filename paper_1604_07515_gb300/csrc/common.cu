@@ -45,7 +45,7 @@ int ctx_init(lgc_ctx* ctx, int device, cudaStream_t stream) {
     cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &thr);
   }
   LGC_CUDA_TRY(cudaHostAlloc((void**)&ctx->h_counters, sizeof(Counters), cudaHostAllocDefault));
-  LGC_CUDA_TRY(cudaHostAlloc((void**)&ctx->h_scratch, 8 * sizeof(int64_t), cudaHostAllocDefault));
+  LGC_CUDA_TRY(cudaHostAlloc((void**)&ctx->h_scratch, 16 * sizeof(int64_t), cudaHostAllocDefault));
   LGC_CUDA_TRY(cudaMalloc((void**)&ctx->d_counters, sizeof(Counters)));
   LGC_CUDA_TRY(cudaMemsetAsync(ctx->d_counters, 0, sizeof(Counters), ctx->stream));
   LGC_CUDA_TRY(cudaHostAlloc((void**)&ctx->h_sort_err, sizeof(int), cudaHostAllocMapped));

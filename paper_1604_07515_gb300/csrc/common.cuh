@@ -224,7 +224,7 @@ struct lgc_ctx {
   // small pinned host block for per-round read-back
   lgc::Counters* h_counters = nullptr;
   lgc::Counters* d_counters = nullptr;
-  int64_t* h_scratch = nullptr;  // pinned, 8 int64
+  int64_t* h_scratch = nullptr;  // pinned, 16 int64
   // residual of the last PR-Nibble call (host svec), kept under LGC_OPT_TRACE
   lgc_svec* last_residual = nullptr;
   // trace of the last call
@@ -246,6 +246,16 @@ struct lgc_ctx {
   std::vector<cudaEvent_t> event_pool;
   lgc_kernel_profile prof[LGC_PROF_COUNT] = {};
 };
+
+namespace lgc {
+// The vertices of highest degree (of kHotDeg or more; -2: none), whose adds the
+// push kernels combine (edges.cuh).
+constexpr int kHot = 4;
+constexpr int32_t kHotDeg = 1024;
+struct HotSet {
+  int32_t v[kHot] = {-2, -2, -2, -2};
+};
+}  // namespace lgc
 
 // Work item of a pull round: edges [beg, beg + len) of heavy vertex w, the
 // item's vertex being heavy[h] and having nparts items in all.
@@ -281,6 +291,7 @@ struct lgc_graph {
   int32_t max_deg = 0;
   lgc::Recip* recip = nullptr;  // 1 / d by degree d < recip_n (device)
   int32_t recip_n = 0;
+  lgc::HotSet hot;
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
   int pull_batch = 8;          // edges per lane per batch in heavy pull gathers (tuned)
   int pull_group = 32;         // lanes per work item in heavy pull gathers (tuned)

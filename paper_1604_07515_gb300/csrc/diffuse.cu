@@ -228,8 +228,9 @@ __global__ void vmap_hkpr_kernel(int64_t nf, const int32_t* __restrict__ fv,
 __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
                                         const int32_t* __restrict__ deg, const double* share,
                                         const int64_t* epos, const int64_t* foff, int64_t nf,
-                                        int64_t E, Table D, double c, int fmode, int32_t* nfv,
-                                        int32_t* nfs, int32_t ncap, Counters* C) {
+                                        int64_t E, const HotSet& H, Table D, double c, int fmode,
+                                        int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
+  HotSum S;
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;  // counted once per block
@@ -246,6 +247,7 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
         sh[k] = share[src[k]];
       }
     }
+    hot_take(H, S, w, sh);
     // Resolve every item's slot before any atomic, so the first-probe loads
     // (or bitmap loads) of all items are in flight together.
     int32_t slot[kEdgeItems];
@@ -304,6 +306,29 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
       frontier_append(pred[k], w[k], slot[k], dw[k], nfv, nfs, C, ncap);
     }
   });
+  // the hot vertices' sums, each as one add: the one that takes the vertex
+  // across its threshold appends it
+  hot_flush<kBlock / 32>(S, [&](int h, double sh) {
+    const int32_t w = H.v[h];
+    int ins = 0;
+    const int64_t s = tb_find_or_insert(D, w, &ins, &C->err);
+    if (s < 0) return;
+    nins += ins;
+    const double old = atomicAdd(tb_val(D, s), sh);
+    const int64_t d = deg[w];
+    const double thr = c * (double)d;
+    const bool pred = fmode == kFmThreshold ? old < thr && old + sh >= thr
+                                            : fmode == kFmInserted && ins != 0;
+    if (!pred) return;
+    const int32_t pos = atomicAdd(&C->next_size, 1);
+    atomicAdd((unsigned long long*)&C->next_edges, (unsigned long long)d);
+    if (pos < ncap) {
+      nfv[pos] = w;
+      nfs[pos] = (int32_t)s;
+    } else {
+      atomicOr(&C->err, kErrFrontierOverflow);
+    }
+  });
   flush_count(nins, &C->inserted);
 }
 
@@ -311,10 +336,10 @@ __global__ void __launch_bounds__(kBlock)
     emap_atomic_kernel(const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
                        const double* __restrict__ share, const int64_t* __restrict__ epos,
                        const int64_t* __restrict__ foff, int64_t nf, int64_t E_host,
-                       const int64_t* __restrict__ E_dev, Table D, double c, int fmode,
+                       const int64_t* __restrict__ E_dev, HotSet H, Table D, double c, int fmode,
                        int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
   // the device-computed total bounds every edge index, whatever the host passed
-  emap_atomic_body(col, deg, share, epos, foff, nf, min(E_host, *E_dev), D, c, fmode, nfv, nfs,
+  emap_atomic_body(col, deg, share, epos, foff, nf, min(E_host, *E_dev), H, D, c, fmode, nfv, nfs,
                    ncap, C);
 }
 
@@ -330,8 +355,9 @@ constexpr int kRedItems = 8;
 __global__ void __launch_bounds__(kBlock)
     emap_red_kernel(const int32_t* __restrict__ col, const double* __restrict__ share,
                     const int64_t* __restrict__ epos, const int64_t* __restrict__ foff,
-                    int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev, Table D,
-                    Counters* C) {
+                    int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev, HotSet H,
+                    Table D, Counters* C) {
+  HotSum S;
   const int64_t E = min(E_host, *E_dev);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -349,6 +375,7 @@ __global__ void __launch_bounds__(kBlock)
         sh[k] = share[src[k]];
       }
     }
+    hot_take(H, S, w, sh);
     if (D.dense) {
       // nothing waits for a result here: the add and the presence bit are both
       // reductions; the keys this round inserted are counted by the caller
@@ -377,199 +404,13 @@ __global__ void __launch_bounds__(kBlock)
       }
     }
   });
+  hot_flush<kBlock / 32>(S, [&](int h, double sh) {
+    int ins = 0;
+    const int64_t s = tb_find_or_insert(D, H.v[h], &ins, &C->err);
+    if (s >= 0) atomicAdd(tb_val(D, s), sh);
+    nins += D.dense ? 0 : ins;  // a dense set's keys are counted from its bitmap
+  });
   flush_count(nins, &C->inserted);
-}
-
-// ---------------------------------------------------------------------------
-// Consecutive small Nibble rounds in one cooperative launch (rounds_nibble_kernel;
-// PR-Nibble's are in rounds.cu).
-// ---------------------------------------------------------------------------
-struct RoundsState {
-  int32_t cur;   // frontier buffer of the current round (0 or 1)
-  int32_t stop;  // 1 empty frontier, 2 round limit, 3 round not small, 4 error flagged
-  int64_t count, rounds, pushes, pushed_edges;
-  int32_t ptab;  // Nibble: the table holding p (0 the initial one, 1 A, 2 B)
-};
-
-__device__ inline int64_t block_sum_i64(int64_t x, int64_t* s_red) {
-  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
-  if ((threadIdx.x & 31) == 0) s_red[threadIdx.x >> 5] = x;
-  __syncthreads();
-  int64_t t = 0;
-  for (int k = 0; k < (int)(blockDim.x >> 5); k++) t += s_red[k];
-  __syncthreads();
-  return t;
-}
-
-// The grid-wide exclusive prefix sum of cnt[0, nf) into epos: block b owns
-// the chunk [c0, c1) of grid_chunk, writes the sum of cnt over it into
-// bsum[b], and after a grid barrier grid_scan_tail scans its chunk from the
-// sums of the chunks before it and returns the total (every thread of the
-// grid calls it).
-__device__ inline void grid_chunk(int64_t nf, int64_t* c0, int64_t* c1) {
-  const int64_t chunk = (nf + gridDim.x - 1) / gridDim.x;
-  *c0 = min(nf, (int64_t)blockIdx.x * chunk);
-  *c1 = min(nf, *c0 + chunk);
-}
-
-__device__ inline int64_t grid_scan_tail(const int64_t* cnt, int64_t nf, int64_t* epos,
-                                         const int64_t* bsum) {
-  __shared__ int64_t s_red[kBlock / 32];
-  __shared__ int64_t s_scan[kBlock / 32];
-  const int G = gridDim.x;
-  int64_t c0, c1;
-  grid_chunk(nf, &c0, &c1);
-  int64_t pre = 0, tot = 0;
-  for (int b = threadIdx.x; b < G; b += blockDim.x) {
-    const int64_t x = __ldcg(&bsum[b]);
-    tot += x;
-    if (b < (int)blockIdx.x) pre += x;
-  }
-  pre = block_sum_i64(pre, s_red);
-  tot = block_sum_i64(tot, s_red);
-  for (int64_t base = c0; base < c1; base += blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    const int64_t x = i < c1 ? cnt[i] : 0;
-    int64_t inc = x;  // inclusive scan within the warp, then across warps
-    for (int o = 1; o < 32; o <<= 1) {
-      const int64_t y = __shfl_up_sync(0xffffffffu, inc, o);
-      if ((threadIdx.x & 31) >= o) inc += y;
-    }
-    if ((threadIdx.x & 31) == 31) s_scan[threadIdx.x >> 5] = inc;
-    __syncthreads();
-    int64_t wpre = 0, btot = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); k++) {
-      if (k < (int)(threadIdx.x >> 5)) wpre += s_scan[k];
-      btot += s_scan[k];
-    }
-    if (i < c1) epos[i] = pre + wpre + inc - x;
-    pre += btot;
-    __syncthreads();
-  }
-  return tot;
-}
-
-// Every thread keeps the round state (frontier buffer, rounds, pushes,
-// keys) in registers, updated alike from the counters each round wrote once
-// the grid has synchronised; the state goes to S when the kernel stops.  A
-// round: the vertexMap over each block's chunk of the frontier with the
-// chunk's record count | barrier | the scan | barrier | the edge push |
-// barrier.  The current round's counters are cleared after the first
-// barrier (nothing reads them after it), for their reuse as the next
-// round's "next".  The kernel stops (leaving the state for the host, which
-// continues with the same rounds one launch per step) when the frontier is
-// empty, the round limit is reached, or the next round is not small: more
-// than e_max edges, a next frontier that might not fit the buffers, or a
-// table that might pass its load limit.
-//
-// Nibble (Fig. alg:nibble, atomic mode): each round fills a
-// fresh p' from p, so two hashed tables of capacity cap alternate as p'
-// (A in device round 0, 2, ..., B in 1, 3, ...; both clear at launch) and p
-// starts in T0 (any form), the table the host's rounds left.  A round runs
-// the vertexMap (p'[v] = p[v]/2, appending v if that reaches the threshold),
-// the scan and the edge push into p'.  When the new frontier is empty the
-// run is over and p stays where it was (the method returns the previous p);
-// otherwise p' becomes p and the old p, when it is A or B, is cleared in a
-// fourth phase to serve as the next round's p'.  key_limit is cap / 2: a
-// round whose keys (at most |F| + its edges) could pass it stops the kernel
-// first.
-__global__ void __launch_bounds__(kBlock)
-    rounds_nibble_kernel(Table T0, Table A, Table B, const int64_t* __restrict__ off,
-                         const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
-                         double eps, int fmode, int32_t* fv0, int32_t* fs0, int32_t* fv1,
-                         int32_t* fs1, int32_t fcap, double* share, int64_t* cnt, int64_t* epos,
-                         int64_t* foff, int64_t* bsum, Counters* Cn, RoundsState* S,
-                         int64_t max_rounds, int64_t e_max, int64_t key_limit) {
-  cg::grid_group grid = cg::this_grid();
-  __shared__ int64_t s_red[kBlock / 32];
-  int cur = __ldcg(&S->cur), ptab = __ldcg(&S->ptab);
-  int64_t count = __ldcg(&S->count), k = __ldcg(&S->rounds);
-  int64_t pushes = __ldcg(&S->pushes), pushed = __ldcg(&S->pushed_edges);
-  auto finish = [&](int stop) {
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-      S->cur = cur;
-      S->ptab = ptab;
-      S->stop = stop;
-      S->count = count;
-      S->rounds = k;
-      S->pushes = pushes;
-      S->pushed_edges = pushed;
-    }
-  };
-  for (;;) {
-    const int nxt = cur ^ 1;
-    const int64_t nf = __ldcg(&Cn[cur].next_size);
-    const int64_t E = __ldcg(&Cn[cur].next_edges);
-    const int err = __ldcg(&Cn[cur].err) | __ldcg(&Cn[nxt].err);
-    int stop = 0;
-    if (err) stop = 4;
-    else if (nf == 0) stop = 1;
-    else if (k >= max_rounds) stop = 2;
-    else if (E > e_max || nf + E > fcap || nf + E > key_limit) stop = 3;
-    if (stop) {  // the same decision in every thread: no barrier is left waiting
-      finish(stop);
-      return;
-    }
-    const Table P = ptab == 0 ? T0 : ptab == 1 ? A : B;
-    const Table Q = (k & 1) ? B : A;  // never P: P is T0 or the other one
-    int32_t* fv = cur ? fv1 : fv0;
-    int32_t* fs = cur ? fs1 : fs0;
-    int32_t* nfv = cur ? fv0 : fv1;
-    int32_t* nfs = cur ? fs0 : fs1;
-    int64_t c0, c1;
-    grid_chunk(nf, &c0, &c1);
-    int64_t part = nibble_vmap_body(c0, c1, blockDim.x, fv, fs, P, Q, off, eps, fmode, 0, 1,
-                                    share, cnt, foff, nfv, nfs, fcap, &Cn[nxt]);
-    part = block_sum_i64(part, s_red);
-    if (threadIdx.x == 0) bsum[blockIdx.x] = part;
-    grid.sync();
-    if (blockIdx.x == 0 && threadIdx.x == 0) Cn[cur] = Counters{};
-    const int64_t tot = grid_scan_tail(cnt, nf, epos, bsum);
-    grid.sync();
-    emap_atomic_body(col, deg, share, epos, foff, nf, min(E, tot), Q, eps, fmode, nfv, nfs, fcap,
-                     &Cn[nxt]);
-    grid.sync();
-    k += 1;
-    pushes += nf;
-    pushed += E;
-    if (__ldcg(&Cn[nxt].next_size) == 0) {  // the previous p is the result
-      finish(1);
-      return;
-    }
-    count = __ldcg(&Cn[nxt].aux) + __ldcg(&Cn[nxt].inserted);
-    if (ptab != 0) {  // the old p (A or B) becomes the next round's p'
-      for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < P.cap;
-           i += (int64_t)gridDim.x * blockDim.x)
-        P.s[i] = Slot{};
-    }
-    ptab = ((k - 1) & 1) ? 2 : 1;
-    cur = nxt;
-    grid.sync();
-  }
-}
-
-__global__ void rounds_init_kernel(Counters* Cn, RoundsState* S, int64_t nf, int64_t E,
-                                   int64_t count) {
-  Cn[0] = Counters{};
-  Cn[1] = Counters{};
-  Cn[0].next_size = (int32_t)nf;
-  Cn[0].next_edges = E;
-  *S = RoundsState{};
-  S->count = count;
-}
-
-// out: stop | err << 8 | ptab << 16, cur, frontier size, its edges, keys,
-// rounds, pushes, pushed edges
-__global__ void rounds_pack_kernel(const Counters* Cn, const RoundsState* S, int64_t* out) {
-  const int cur = S->cur;
-  out[0] = (int64_t)S->stop | ((int64_t)(Cn[0].err | Cn[1].err) << 8) | ((int64_t)S->ptab << 16);
-  out[1] = cur;
-  out[2] = Cn[cur].next_size;
-  out[3] = Cn[cur].next_edges;
-  out[4] = S->count;
-  out[5] = S->rounds;
-  out[6] = S->pushes;
-  out[7] = S->pushed_edges;
 }
 
 // sign * (set bits of the bitmap) added into *out, one atomic per block.
@@ -1571,6 +1412,19 @@ HeavyKernel<SH> heavy_kernel(int batch, int group) {
 // ---------------------------------------------------------------------------
 namespace {
 
+int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
+
+// Sets of a graph of up to kDenseSmall vertices are dense from the start
+// (automatic form): clearing 16 bytes a vertex costs 4 us at that size,
+// growing and converting a table on the way 40 us and more.
+constexpr int64_t kDenseSmall = int64_t{1} << 20;
+// Keys a table has room for ahead of the device-driven rounds.
+constexpr int64_t kRoomKeys = 16384;
+
+bool dense_small(const lgc_ctx* ctx, int64_t n) {
+  return ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
+}
+
 struct Frontier {
   DBuf<int32_t> v, s;
   int64_t size = 0, edges = 0;
@@ -1612,11 +1466,7 @@ struct PushWork {
   DBuf<uint32_t> selv, selv2;
   DBuf<int32_t> seli, seli2;
   DBuf<unsigned long long> selcnt;
-  // device-driven rounds: two frontier buffers, block sums, counters, state
-  Frontier X[2];
-  DBuf<int64_t> xbsum;
-  DBuf<Counters> xcn;
-  DBuf<RoundsState> xst;
+  // device-driven rounds
   RoundsMem rmem;
   DBuf<Recip> recip;  // HK-PR pull rounds: 1 / ((j + 1) d) by degree
   lgc_stats st{};
@@ -1624,8 +1474,6 @@ struct PushWork {
   ~PushWork() {
     F.release(ctx);
     G.release(ctx);
-    X[0].release(ctx);
-    X[1].release(ctx);
     U.release(ctx);
     selk.release(ctx);
     selk2.release(ctx);
@@ -1638,9 +1486,6 @@ struct PushWork {
     dany.release(ctx);
     dpred.release(ctx);
     dstep.release(ctx);
-    xbsum.release(ctx);
-    xcn.release(ctx);
-    xst.release(ctx);
     rmem.release(ctx);
     recip.release(ctx);
     share.release(ctx);
@@ -1732,7 +1577,7 @@ struct PushWork {
         {
           ProfScope ps(ctx, LGC_PROF_EDGEMAP, alg_bytes);
           emap_red_kernel<<<grid, kBlock, 0, s>>>(g->col, share.ptr, epos.ptr, foff.ptr, nf, nrec,
-                                                   total.ptr, D, ctx->d_counters);
+                                                   total.ptr, g->hot, D, ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
         if (D.dense) {
@@ -1757,7 +1602,7 @@ struct PushWork {
         int grid = (int)(tiles < (ctx->sms * 16) ? tiles : (ctx->sms * 16));
         ProfScope ps(ctx, LGC_PROF_EDGEMAP, alg_bytes);
         emap_atomic_kernel<<<grid, kBlock, 0, s>>>(g->col, g->deg, share.ptr, epos.ptr, foff.ptr,
-                                                    nf, nrec, total.ptr, D, c, fmode, G.v.ptr,
+                                                    nf, nrec, total.ptr, g->hot, D, c, fmode, G.v.ptr,
                                                     G.s.ptr, ncap, ctx->d_counters);
         LGC_COUNT_LAUNCH(ctx);
         LGC_CUDA_TRY(cudaGetLastError());
@@ -1985,18 +1830,9 @@ struct PushWork {
     return read_counters(out);
   }
 
-  // Nibble's small rounds on the device (rounds_nibble_kernel).
-  static constexpr int64_t kRoundsEmax = int64_t{1} << 20;
-  static constexpr int64_t kRoundsPerLaunch = 1024;
-  int64_t rounds_emax() const { return std::min<int64_t>(kRoundsEmax, g->nnz / 16); }
-  int64_t rounds_fcap() const { return std::min<int64_t>(g->n, 2 * kRoundsEmax); }
   // keys T takes within load 1/2 (no set has more than n)
   int64_t key_limit(const Table& T) const {
     return T.dense || T.cap >= 2 * g->n ? INT64_MAX : T.cap / 2;
-  }
-  bool small_round_nibble() const {
-    return ctx->device_rounds && !ctx->trace && F.size > 0 && F.edges <= rounds_emax() &&
-           F.size + F.edges <= rounds_fcap();
   }
   // The edges from which a round is a pull round (use_pull), automatic policy.
   int64_t pull_min() const {
@@ -2027,111 +1863,59 @@ struct PushWork {
     return LGC_OK;
   }
 
-  // Nibble's rounds on the device (rounds_nibble_kernel) from the host's p
-  // table P and frontier F, at most rounds_left of them.  Afterwards P holds
-  // p (a table of the kernel's, or the same one), Pn is a spare, F and the
-  // counters are the host's again, *done counts the rounds run and *over is
-  // set when a round's frontier came out empty (the run is over).
-  int device_rounds_nibble(Table& P, Table& Pn, int64_t* count, double eps, int fmode,
-                           int64_t rounds_left, int64_t* done, bool* over) {
+  // Small rounds into fresh sets on the device (rounds.cu): Nibble's (c
+  // null) from the vector in S, or HK-PR's from level *j with residuals in S
+  // and p in P.  *done counts the rounds run (0: no room for them); S is the
+  // set reached (Nibble with *over: the vector returned), F and st follow.
+  int device_rounds_fresh(Table& S, Table& Sn, Table* P, int64_t* pcount, int64_t* count,
+                          const RoundsFresh& q, bool det, int64_t rounds_left, int64_t* done,
+                          bool* over) {
     cudaStream_t s = ctx->stream;
     *done = 0;
     *over = false;
-    static int blocks_per_sm = -1;  // the same for every device of this build
-    if (blocks_per_sm < 0) {
-      int nb = 0;
-      if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, rounds_nibble_kernel, kBlock, 0) !=
-          cudaSuccess)
-        nb = 0;
-      blocks_per_sm = nb;
-    }
-    int sms = 0;
-    LGC_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, ctx->device));
-    // one block per SM: the rounds are small, and fewer blocks wait at each
-    // grid barrier (two per SM measured 0.3% slower on the bench step)
-    const int G = sms * std::min(blocks_per_sm, 1);
-    if (G < 1) {  // no co-resident grid possible: rounds stay on the host
-      ctx->device_rounds = false;
-      return LGC_OK;
-    }
-    const int64_t fcap = rounds_fcap();
-    // p' tables with room for 8 times this round's keys (a round that
-    // would not fit returns to the host, which comes back with bigger ones)
-    const int64_t keys8 = std::min<int64_t>(g->n, 8 * (F.size + F.edges));
-    const int64_t cap = pow2_at_least(2 * std::max<int64_t>(1024, keys8));
-    Table A, B;
-    int st_ = table_create(ctx, &A, cap, false);
-    if (st_ == LGC_OK) st_ = table_create(ctx, &B, cap, false);
-    if (st_ != LGC_OK) {
-      table_destroy(ctx, &A);
-      table_destroy(ctx, &B);
+    // fresh sets with room for 8 times this round's keys, in the smaller form
+    // (a round that would not fit returns to the host, which comes back with
+    // bigger ones); dense ones where they are cheap to clear
+    const int64_t n = g->n, need = std::min<int64_t>(n, F.size + F.edges);
+    const int64_t cap = pow2_at_least(2 * std::min<int64_t>(n, std::max<int64_t>(kRoomKeys, 8 * need)));
+    const bool dense = want_dense(ctx, need, n) || dense_small(ctx, n) ||
+                       (ctx->table_form == 0 && n >= 1024 && 16 * cap >= 8 * n + n / 8);
+    Table T[4];
+    T[3] = S;
+    int st_ = LGC_OK;
+    for (int k = 0; k < 3 && st_ == LGC_OK; k++)
+      st_ = dense ? table_create_dense(ctx, &T[k], n, false) : table_create(ctx, &T[k], cap, false);
+    RoundsOut o;
+    if (st_ == LGC_OK)
+      st_ = rounds_fresh(ctx, g, rmem, q, T, P, pcount ? *pcount : 0, F.v.ptr, F.s.ptr, F.size,
+                         F.edges, det, pull_min(), rounds_left, key_limit(T[0]),
+                         P ? key_limit(*P) : 0, &o);
+    if (st_ != LGC_OK || o.rounds == 0) {
+      for (int k = 0; k < 3; k++) table_destroy(ctx, &T[k]);
       return st_;
     }
-    auto fail = [&](int code) {
-      table_destroy(ctx, &A);
-      table_destroy(ctx, &B);
-      return code;
-    };
-    for (int k = 0; k < 2; k++) {
-      if (X[k].v.reserve(ctx, fcap) || X[k].s.reserve(ctx, fcap)) return fail(LGC_ENOMEM);
+    *done = o.rounds;
+    *over = o.nf == 0;
+    for (int k = 0; k < 3; k++)
+      if (k != o.tab) table_destroy(ctx, &T[k]);
+    if (o.tab != 3) {
+      table_destroy(ctx, &S);
+      table_destroy(ctx, &Sn);
+      S = T[o.tab];
     }
-    if (reserve_frontier_scratch(fcap) || xbsum.reserve(ctx, G) || xcn.reserve(ctx, 2) ||
-        xst.reserve(ctx, 1) || total.reserve(ctx, 8))
-      return fail(LGC_ENOMEM);
-    if (cudaMemcpyAsync(X[0].v.ptr, F.v.ptr, 4 * F.size, cudaMemcpyDeviceToDevice, s) ||
-        cudaMemcpyAsync(X[0].s.ptr, F.s.ptr, 4 * F.size, cudaMemcpyDeviceToDevice, s))
-      return fail(LGC_ECUDA);
-    rounds_init_kernel<<<1, 1, 0, s>>>(xcn.ptr, xst.ptr, F.size, F.edges, *count);
-    LGC_COUNT_LAUNCH(ctx);
-    int32_t fc = (int32_t)fcap;
-    int64_t mr = std::min<int64_t>(rounds_left, kRoundsPerLaunch), em = rounds_emax(),
-            kl = cap / 2;
-    void* args[] = {&P, &A, &B, &g->off, &g->col, &g->deg, &eps, &fmode, &X[0].v.ptr,
-                    &X[0].s.ptr, &X[1].v.ptr, &X[1].s.ptr, &fc, &share.ptr, &cnt.ptr, &epos.ptr,
-                    &foff.ptr, &xbsum.ptr, &xcn.ptr, &xst.ptr, &mr, &em, &kl};
-    {
-      ProfScope ps(ctx, LGC_PROF_EDGEMAP, 0.0);
-      if (cudaLaunchCooperativeKernel((const void*)rounds_nibble_kernel, G, kBlock, args, 0, s))
-        return fail(LGC_ECUDA);
-      LGC_COUNT_LAUNCH(ctx);
+    *count = o.count;
+    if (pcount) *pcount = o.pcount;
+    st.rounds += o.rounds;
+    st.pushes += o.pushes;
+    st.pushed_edges += o.pushed;
+    LGC_TRY(F.v.reserve(ctx, std::max<int64_t>(o.nf, 1024)));
+    LGC_TRY(F.s.reserve(ctx, std::max<int64_t>(o.nf, 1024)));
+    if (o.nf > 0) {
+      LGC_CUDA_TRY(cudaMemcpyAsync(F.v.ptr, o.v, 4 * o.nf, cudaMemcpyDeviceToDevice, s));
+      LGC_CUDA_TRY(cudaMemcpyAsync(F.s.ptr, o.s, 4 * o.nf, cudaMemcpyDeviceToDevice, s));
     }
-    rounds_pack_kernel<<<1, 1, 0, s>>>(xcn.ptr, xst.ptr, total.ptr);
-    LGC_COUNT_LAUNCH(ctx);
-    if (cudaMemcpyAsync(ctx->h_scratch, total.ptr, 64, cudaMemcpyDeviceToHost, s) ||
-        cudaStreamSynchronize(s))
-      return fail(LGC_ECUDA);
-    const int64_t* o = ctx->h_scratch;
-    const int64_t stop = o[0] & 0xff, err = (o[0] >> 8) & 0xff, ptab = (o[0] >> 16) & 0xff;
-    const int64_t cur = o[1], nf = o[2], E = o[3], rounds = o[5];
-    if (ctx->profile && !ctx->prof_pending.empty())
-      ctx->prof_pending.back().bytes += 24.0 * (double)o[7] + 88.0 * (double)o[6];
-    if (err != 0) return fail(LGC_ETABLEFULL);
-    if (rounds < 1) return fail(LGC_ECUDA);  // the host checked that the first round is small
-    st.rounds += rounds;
-    st.pushes += o[6];
-    st.pushed_edges += o[7];
-    *done = rounds;
-    // p: where the kernel left it; the other tables are spares or freed
-    if (ptab != 0) {
-      table_destroy(ctx, &P);
-      table_destroy(ctx, &Pn);
-      P = ptab == 1 ? A : B;
-      Pn = ptab == 1 ? B : A;
-    } else {
-      table_destroy(ctx, &A);
-      table_destroy(ctx, &B);
-    }
-    if (stop == 1) {
-      *over = true;
-      return LGC_OK;
-    }
-    LGC_TRY(F.v.reserve(ctx, std::max<int64_t>(nf, 1024)));
-    LGC_TRY(F.s.reserve(ctx, std::max<int64_t>(nf, 1024)));
-    LGC_CUDA_TRY(cudaMemcpyAsync(F.v.ptr, X[cur].v.ptr, 4 * nf, cudaMemcpyDeviceToDevice, s));
-    LGC_CUDA_TRY(cudaMemcpyAsync(F.s.ptr, X[cur].s.ptr, 4 * nf, cudaMemcpyDeviceToDevice, s));
-    F.size = nf;
-    F.edges = E;
-    *count = o[4];
+    F.size = o.nf;
+    F.edges = o.E;
     return LGC_OK;
   }
 
@@ -2228,7 +2012,6 @@ int vgrid(const lgc_ctx* ctx, int64_t nf) {
   return (int)(g < 1 ? 1 : g);
 }
 
-int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 
 // Bulk rounds (atomic mode): the destination is dense and the round pushes at
 // least n/32 edges, so a filter pass over the n-bit presence bitmap costs no
@@ -2277,17 +2060,6 @@ int ensure_capacity(lgc_ctx* ctx, Table* T, int64_t count, int64_t add, int64_t 
   if (want_dense(ctx, need, n)) return table_to_dense(ctx, T, n, fv, fs, nf);
   if (2 * need > T->cap) return table_grow(ctx, T, 2 * need, fv, fs, nf);
   return LGC_OK;
-}
-
-// Sets of a graph of up to kDenseSmall vertices are dense from the start
-// (automatic form): clearing 16 bytes a vertex costs 4 us at that size,
-// growing and converting a table on the way 40 us and more.
-constexpr int64_t kDenseSmall = int64_t{1} << 20;
-// Keys a table has room for ahead of the device-driven rounds.
-constexpr int64_t kRoomKeys = 16384;
-
-bool dense_small(const lgc_ctx* ctx, int64_t n) {
-  return ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
 }
 
 // Before device-driven rounds: as ensure_capacity for the next round, with
@@ -2733,13 +2505,19 @@ int run_nibble(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_nibble_params* p
     W.F.edges = dx;
     lgc_stats& st = W.st;
     for (int t = 1; t <= prm->T; t++) {
-      if (!det && W.small_round_nibble()) {
+      if (rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, false) && (!det || eps > 0.0)) {
         int64_t done = 0;
         bool over = false;
-        status = W.device_rounds_nibble(Pc, Pn, &count, eps, fmode, prm->T - t + 1, &done, &over);
+        RoundsFresh q;
+        q.eps = eps;
+        q.count = count;
+        status = W.device_rounds_fresh(Pc, Pn, nullptr, nullptr, &count, q, det, prm->T - t + 1,
+                                       &done, &over);
         if (status != LGC_OK || over) break;
-        t += (int)done - 1;  // the loop adds the last one
-        continue;
+        if (done > 0) {
+          t += (int)done - 1;  // the loop adds the last one
+          continue;
+        }
       }
       W.record_trace();
       const int64_t nf = W.F.size;
@@ -2836,6 +2614,24 @@ int run_hkpr(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_hkpr_params* prm, 
     lgc_stats& st = W.st;
     int j = 0;
     while (W.F.size > 0) {
+      if (j + 1 < N && rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, false) &&
+          (!det || eps > 0.0)) {
+        if ((status = ensure_room_ahead(ctx, &P, pcount, W.F.size, g->n, nullptr, nullptr, 0)) !=
+            LGC_OK)
+          break;
+        int64_t done = 0, rcount = 0;
+        bool over = false;
+        RoundsFresh q;
+        q.t = t;
+        q.c = c.data();
+        q.N = N;
+        q.j = j;
+        status = W.device_rounds_fresh(Rc, Rn, &P, &pcount, &rcount, q, det, N - 1 - j, &done,
+                                       &over);
+        if (status != LGC_OK) break;
+        j += (int)done;
+        if (done > 0) continue;
+      }
       W.record_trace();
       const int64_t nf = W.F.size;
       const bool last = j + 1 >= N;

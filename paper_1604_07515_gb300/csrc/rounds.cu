@@ -1,6 +1,6 @@
-// Consecutive small PR-Nibble rounds (Sec. 3.3) in one cooperative launch,
-// in atomic and in deterministic mode, with and without beta-fraction
-// selection.
+// Consecutive small rounds in one cooperative launch: PR-Nibble's (Sec. 3.3),
+// with and without beta-fraction selection, Nibble's (Sec. 3.2) and HK-PR's
+// (Sec. 3.4), in atomic and in deterministic mode.
 //
 // A host-driven round costs its launches and a read-back whatever its size:
 // 16 launches and two synchronisations in deterministic mode (records,
@@ -58,6 +58,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "edges.cuh"
 #include "foldwarp.cuh"
 #include "prim.cuh"
 #include "rounds.cuh"
@@ -92,6 +93,8 @@ struct RdCnt {
   unsigned long long next;      // the round's frontier: size << 40 | degree sum
   unsigned long long push;      // beta rounds: pushing entries, packed alike
   unsigned long long inserted;  // keys created by the round
+  unsigned long long pinserted; // HK-PR: keys of p created by it
+  int nkeys;                    // fresh sets: entries of the round's key list
   int touched;                  // destinations of the round
   int emin, emax;               // wide rounds: the shares' exponent range, as pull rounds keep it
   int err;
@@ -182,6 +185,24 @@ __device__ inline int64_t rd_append(const RdBuf& B, const RdFront& F, RdCnt* C, 
   return pos;
 }
 
+// The same by one thread.
+__device__ inline void rd_append_one(const RdBuf& B, const RdFront& F, RdCnt* C, int32_t v,
+                                     int32_t s, int64_t d) {
+  const unsigned long long base = atomicAdd(&C->next, rd_pack(1, d));
+  const int64_t pos = rd_size(base);
+  const uint32_t e = (uint32_t)rd_edges(base);
+  if (pos >= B.fcap) {
+    atomicOr(&C->err, kErrFrontierOverflow);
+    return;
+  }
+  F.v[pos] = v;
+  F.s[pos] = s;
+  F.e[pos] = e;
+  F.rank[pos] = 0;
+  F.brank[pos] = 0;
+  rd_tiles(F.tile, B.tiles, pos, e, d);
+}
+
 // Lists the destinations q[k] with k0[k] == 0 (IT per lane, one atomic per
 // warp).
 template <int IT, class Q>
@@ -249,15 +270,31 @@ __device__ inline void rd_edges_of(const RdEdges& R, int64_t warp, int64_t nwarp
   }
 }
 
+// Where a push's destinations go: a set, the list of the keys a round creates
+// in it (fresh sets; null otherwise), and what makes a vertex a candidate: its
+// value reaching c * d (thr) or its insertion.
+struct RdDest {
+  Table T;
+  int32_t* keys;
+  double c;
+  bool thr;
+};
+
+// Hot destinations are summed apart (edges.cuh) where the frontier is large
+// enough for their adds to queue.
+constexpr int64_t kRdHotMin = 2048;
+
 // Atomic push of IT edges a lane: all columns, first probes, slots, adds and
 // crossings of a lane's edges side by side.
 template <int IT>
-__device__ inline void rd_push(const RdBuf& B, const Table& T, const int32_t* __restrict__ col,
-                               const int32_t* __restrict__ deg, const RdEdges& R, double eps,
+__device__ inline void rd_push(const RdBuf& B, const RdDest& D, const HotSet& H, bool hot,
+                               HotSum& S, const int32_t* __restrict__ col,
+                               const int32_t* __restrict__ deg, const RdEdges& R,
                                const RdFront& N, RdCnt* Cc, RdCnt* C, int64_t warp,
                                int64_t nwarps, int64_t* nins) {
+  const Table& T = D.T;
   rd_edges_of<IT>(R, warp, nwarps, [&](int64_t, const int32_t* src, const int64_t* at) {
-    int32_t w[IT], slot[IT];
+    int32_t w[IT], slot[IT], old_key[IT];
     double sh[IT], old[IT];
     uint32_t probe[IT];
     int ins[IT];
@@ -270,6 +307,7 @@ __device__ inline void rd_push(const RdBuf& B, const Table& T, const int32_t* __
         sh[k] = B.share[src[k]];
       }
     }
+    if (hot) hot_take(H, S, w, sh);
 #pragma unroll
     for (int k = 0; k < IT; k++) {
       probe[k] = 0;
@@ -301,27 +339,62 @@ __device__ inline void rd_push(const RdBuf& B, const Table& T, const int32_t* __
       int64_t dw = 0;
       if (slot[k] >= 0) {
         const double nv = old[k] + sh[k];
-        if (nv >= eps) {  // eps * d(w) >= eps for d(w) >= 1: cheap pre-test
+        if (D.thr ? nv >= D.c : ins[k] != 0) {  // c * d(w) >= c for d(w) >= 1: cheap pre-test
           dw = deg[w[k]];
-          const double thr = eps * (double)dw;
-          pred = old[k] < thr && nv >= thr;
+          const double thr = D.c * (double)dw;
+          pred = !D.thr || (old[k] < thr && nv >= thr);
         }
         *nins += ins[k];
       }
+      old_key[k] = ins[k] ? 0 : 1;
       uint32_t e;
       rd_append(B, N, C, pred, w[k], slot[k], dw, &e);
     }
+    if (D.keys) rd_touch<IT>(D.keys, &Cc->nkeys, slot, old_key);
+  });
+}
+
+// The hot vertices' sums after a push, each as one add.
+__device__ inline void rd_push_hot(const RdBuf& B, const RdDest& D, const HotSet& H,
+                                   const HotSum& S, const int32_t* __restrict__ deg,
+                                   const RdFront& N, RdCnt* Cc, RdCnt* C, int64_t* nins) {
+  hot_flush<kRdWarps>(S, [&](int h, double sh) {
+    const int32_t w = H.v[h];
+    int ins = 0;
+    const int64_t s = tb_find_or_insert(D.T, w, &ins, &Cc->err);
+    if (s < 0) return;
+    *nins += ins;
+    if (ins && D.keys) D.keys[atomicAdd(&Cc->nkeys, 1)] = (int32_t)s;
+    const double old = atomicAdd(tb_val(D.T, s), sh);
+    const int64_t d = deg[w];
+    const double thr = D.c * (double)d;
+    if (D.thr ? old < thr && old + sh >= thr : ins != 0) rd_append_one(B, N, C, w, (int32_t)s, d);
   });
 }
 
 // Wide push: every edge's share added to its destination's fixed-point sum;
-// a destination's first edge lists it.
+// a destination's first edge lists it.  Hot destinations are summed apart, as
+// in rd_push.
+struct RdHotFx {
+  Fx a[kHot] = {};
+  unsigned any = 0;
+};
+
+__device__ inline unsigned long long rd_fx_add(Fx* acc, const Fx& x) {
+  unsigned long long old = 0;
+  if (x.lo) old = atomicAdd((unsigned long long*)&acc->lo, (unsigned long long)x.lo);
+  const uint64_t hi = x.hi + (old + x.lo < old ? 1 : 0);
+  if (hi) atomicAdd((unsigned long long*)&acc->hi, (unsigned long long)hi);
+  return old;
+}
+
 template <int IT>
-__device__ inline void rd_push_exact(const RdBuf& B, const Table& T,
-                                     const int32_t* __restrict__ col, const RdEdges& R, int L,
-                                     RdCnt* C, int64_t warp, int64_t nwarps, int64_t* nins) {
+__device__ inline void rd_push_exact(const RdBuf& B, const RdDest& D, const HotSet& H, bool hot,
+                                     RdHotFx& S, const int32_t* __restrict__ col,
+                                     const RdEdges& R, int L, RdCnt* C, int64_t warp,
+                                     int64_t nwarps, int64_t* nins) {
   rd_edges_of<IT>(R, warp, nwarps, [&](int64_t, const int32_t* src, const int64_t* at) {
-    int32_t w[IT], slot[IT], k0[IT];
+    int32_t w[IT], slot[IT], k0[IT], old_key[IT];
     Fx x[IT];
     unsigned long long old[IT];
 #pragma unroll
@@ -333,12 +406,27 @@ __device__ inline void rd_push_exact(const RdBuf& B, const Table& T,
         x[k] = fx_from_bits(fx_bits(B.share[src[k]]), L);
       }
     }
+    if (hot) {
+#pragma unroll
+      for (int k = 0; k < IT; k++) {
+        bool hit = false;
+#pragma unroll
+        for (int h = 0; h < kHot; h++)
+          if (w[k] == H.v[h]) {
+            fx_add(S.a[h], x[k]);
+            S.any |= 1u << h;
+            hit = true;
+          }
+        if (hit) w[k] = -1;
+      }
+    }
 #pragma unroll
     for (int k = 0; k < IT; k++) {
       slot[k] = -1;
       int ins = 0;
-      if (w[k] >= 0) slot[k] = (int32_t)tb_find_or_insert(T, w[k], &ins, &C->err);
+      if (w[k] >= 0) slot[k] = (int32_t)tb_find_or_insert(D.T, w[k], &ins, &C->err);
       *nins += ins;
+      old_key[k] = ins ? 0 : 1;
     }
 #pragma unroll
     for (int k = 0; k < IT; k++) {
@@ -359,7 +447,76 @@ __device__ inline void rd_push_exact(const RdBuf& B, const Table& T,
 #pragma unroll
     for (int k = 0; k < IT; k++) q[k] = make_int2(w[k], slot[k]);
     rd_touch<IT>(B.touched, &C->touched, q, k0);
+    if (D.keys) rd_touch<IT>(D.keys, &C->nkeys, slot, old_key);
   });
+}
+
+__device__ inline void rd_push_exact_hot(const RdBuf& B, const RdDest& D, const HotSet& H,
+                                         const RdHotFx& S, RdCnt* C, int64_t* nins) {
+  __shared__ Fx s_fx[kRdWarps][kHot];
+  __shared__ unsigned s_met;
+  if (!__syncthreads_or(S.any != 0)) return;
+  if (threadIdx.x == 0) s_met = 0;
+  __syncthreads();
+  const int lane = threadIdx.x & 31;
+  const unsigned met = __reduce_or_sync(0xffffffffu, S.any);
+#pragma unroll
+  for (int h = 0; h < kHot; h++) {
+    Fx x = S.a[h];
+    for (int o = 16; o > 0; o >>= 1) {
+      Fx y;
+      y.lo = __shfl_xor_sync(0xffffffffu, x.lo, o);
+      y.hi = __shfl_xor_sync(0xffffffffu, x.hi, o);
+      fx_add(x, y);
+    }
+    if (lane == 0) s_fx[threadIdx.x >> 5][h] = x;
+  }
+  if (lane == 0 && met) atomicOr(&s_met, met);
+  __syncthreads();
+  if (threadIdx.x < kHot && ((s_met >> threadIdx.x) & 1u)) {
+    const int32_t w = H.v[threadIdx.x];
+    Fx x = {0, 0};
+    for (int k = 0; k < kRdWarps; k++) fx_add(x, s_fx[k][threadIdx.x]);
+    int ins = 0;
+    const int64_t s = tb_find_or_insert(D.T, w, &ins, &C->err);
+    if (s >= 0) {
+      *nins += ins;
+      if (ins && D.keys) D.keys[atomicAdd(&C->nkeys, 1)] = (int32_t)s;
+      rd_fx_add(&B.xacc[s], x);
+      if (atomicAdd(&B.cnt[s], 1) == 0)
+        B.touched[atomicAdd(&C->touched, 1)] = make_int2(w, (int32_t)s);
+    }
+  }
+}
+
+// After the barrier: every listed destination's sum joins its value, rounded
+// once, as a pull round adds it.
+__device__ inline void rd_settle_exact(const RdBuf& B, const RdDest& D,
+                                       const int32_t* __restrict__ deg, int L, const RdFront& N,
+                                       RdCnt* Cc, RdCnt* C, int64_t warp, int64_t nwarps) {
+  const int lane = threadIdx.x & 31;
+  const int nt = __ldcg(&Cc->touched);
+  for (int64_t b = warp * 32; b < nt; b += nwarps * 32) {
+    const int64_t i = b + lane;
+    bool pred = false;
+    int2 ts = make_int2(0, 0);
+    int64_t d = 0;
+    if (i < nt) {
+      ts = B.touched[i];
+      const Fx X = B.xacc[ts.y];
+      B.xacc[ts.y] = Fx{0, 0};
+      B.cnt[ts.y] = 0;
+      double* at = tb_val(D.T, ts.y);
+      const double old = *at;
+      const double v = old + fx_to_double(X, L);
+      *at = v;
+      d = deg[ts.x];
+      const double thr = D.c * (double)d;
+      pred = old < thr && v >= thr;
+    }
+    uint32_t e;
+    rd_append(B, N, C, pred, ts.x, ts.y, d, &e);
+  }
 }
 
 // Deterministic filing: every edge's pushing entry into its destination's
@@ -367,9 +524,10 @@ __device__ inline void rd_push_exact(const RdBuf& B, const Table& T,
 template <int IT>
 __device__ inline void rd_file(const RdBuf& B, const Table& T, const int64_t* __restrict__ off,
                                const int32_t* __restrict__ col, const RdEdges& R, int4* touched,
-                               RdCnt* C, int64_t warp, int64_t nwarps, int64_t* nins) {
+                               int32_t* keys, RdCnt* C, int64_t warp, int64_t nwarps,
+                               int64_t* nins) {
   rd_edges_of<IT>(R, warp, nwarps, [&](int64_t, const int32_t* src, const int64_t* at) {
-    int32_t slot[IT], k0[IT];
+    int32_t slot[IT], k0[IT], old_key[IT];
     int4 q[IT];
 #pragma unroll
     for (int k = 0; k < IT; k++) q[k].x = src[k] >= 0 ? col[at[k]] : -1;
@@ -384,6 +542,7 @@ __device__ inline void rd_file(const RdBuf& B, const Table& T, const int64_t* __
       int ins = 0;
       if (q[k].x >= 0) slot[k] = (int32_t)tb_find_or_insert(T, q[k].x, &ins, &C->err);
       *nins += ins;
+      old_key[k] = ins ? 0 : 1;
       q[k].y = slot[k];
       q[k].w -= q[k].z;
     }
@@ -393,6 +552,7 @@ __device__ inline void rd_file(const RdBuf& B, const Table& T, const int64_t* __
     for (int k = 0; k < IT; k++)
       if (slot[k] >= 0) B.bucket[q[k].z + (k0[k] & (kRdSelf - 1))] = src[k];
     rd_touch<IT>(touched, &C->touched, q, k0);
+    if (keys) rd_touch<IT>(keys, &C->nkeys, slot, old_key);
   });
 }
 
@@ -657,6 +817,7 @@ struct RdArgs {
   int gbits;      // sums of fewer than 2^gbits shares
   int keep_room;  // the buffers do not hold every vertex
   int64_t x_min, count, max_rounds, e_max, f_max, key_limit;
+  HotSet hot;
 };
 
 // The vertexMap's arithmetic for residual r and degree d: the share an edge
@@ -792,6 +953,34 @@ __device__ inline void rd_count_inserted(int64_t nins, RdCnt* C) {
     atomicAdd(&C->inserted, (unsigned long long)nins);
 }
 
+// The edge phase of an atomic round over the edges R: the push, and for a
+// wide round (exact) the barrier and the sums' settling.
+__device__ inline void rd_push_round(const RdBuf& B, const RdDest& D, const HotSet& H,
+                                     const int32_t* __restrict__ col,
+                                     const int32_t* __restrict__ deg, const RdEdges& R, bool exact,
+                                     int gbits, const RdFront& N, RdCnt* Cc, RdCnt* C,
+                                     int64_t warp, int64_t nwarps, cg::grid_group& grid) {
+  int64_t nins = 0;
+  const bool wide = R.E > nwarps * 64;  // several edges a lane once every warp has work
+  const bool hot = R.np >= kRdHotMin;
+  if (exact) {
+    RdHotFx S;
+    const int L = fx_scale(2047 - __ldcg(&Cc->emin), __ldcg(&Cc->emax), gbits);
+    if (wide) rd_push_exact<4>(B, D, H, hot, S, col, R, L, Cc, warp, nwarps, &nins);
+    else rd_push_exact<1>(B, D, H, hot, S, col, R, L, Cc, warp, nwarps, &nins);
+    if (hot) rd_push_exact_hot(B, D, H, S, Cc, &nins);
+    rd_count_inserted(nins, Cc);
+    grid.sync();
+    rd_settle_exact(B, D, deg, L, N, Cc, C, warp, nwarps);
+  } else {
+    HotSum S;
+    if (wide) rd_push<4>(B, D, H, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
+    else rd_push<1>(B, D, H, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
+    if (hot) rd_push_hot(B, D, H, S, deg, N, Cc, C, &nins);
+    rd_count_inserted(nins, Cc);
+  }
+}
+
 // Atomic mode.
 template <bool BETA>
 __global__ void __launch_bounds__(kRdBlock, 1) rounds_kernel(RdArgs A, RdBuf B, Table T) {
@@ -831,49 +1020,83 @@ __global__ void __launch_bounds__(kRdBlock, 1) rounds_kernel(RdArgs A, RdBuf B, 
     const unsigned long long pp = BETA ? __ldcg(&Cc->push) : fr;
     const int64_t np = rd_size(pp), Ep = rd_edges(pp);
     const RdEdges R = {BETA ? B.pe : F.e, B.base, BETA ? B.ptile : F.tile, np, Ep};
-    int64_t nins = 0;
-    const bool wide = Ep > nwarps * 64;  // several edges a lane once every warp has work
-    if (exact) {
-      const int L = fx_scale(2047 - __ldcg(&Cc->emin), __ldcg(&Cc->emax), A.gbits);
-      if (wide) rd_push_exact<4>(B, T, A.col, R, L, Cc, warp, nwarps, &nins);
-      else rd_push_exact<1>(B, T, A.col, R, L, Cc, warp, nwarps, &nins);
-      rd_count_inserted(nins, Cc);
-      grid.sync();
-      const int nt = __ldcg(&Cc->touched);
-      for (int64_t b = warp * 32; b < nt; b += nwarps * 32) {
-        const int64_t i = b + lane;
-        bool pred = false;
-        int2 ts = make_int2(0, 0);
-        int64_t d = 0;
-        if (i < nt) {
-          ts = B.touched[i];
-          const Fx X = B.xacc[ts.y];
-          B.xacc[ts.y] = Fx{0, 0};
-          B.cnt[ts.y] = 0;
-          double* at = tb_val(T, ts.y);
-          const double old = *at;
-          const double v = old + fx_to_double(X, L);
-          *at = v;
-          d = A.deg[ts.x];
-          const double thr = A.eps * (double)d;
-          pred = old < thr && v >= thr;
-        }
-        uint32_t e;
-        rd_append(B, N, C, pred, ts.x, ts.y, d, &e);
-      }
-    } else {
-      if (wide)
-        rd_push<4>(B, T, A.col, A.deg, R, A.eps, N, Cc, C, warp, nwarps, &nins);
-      else
-        rd_push<1>(B, T, A.col, A.deg, R, A.eps, N, Cc, C, warp, nwarps, &nins);
-      rd_count_inserted(nins, Cc);
-    }
+    const RdDest D = {T, nullptr, A.eps, true};
+    rd_push_round(B, D, A.hot, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps, grid);
     grid.sync();
     rounds += 1;
     pushes += np;
     pushed += Ep;
     count += (int64_t)__ldcg(&Cc->inserted);
     err |= __ldcg(&Cc->err);
+  }
+}
+
+// The fold phase of a deterministic round: every listed destination's bucket
+// folded into its value; settle(ok, destination, value before, value after, p)
+// is then called by whole warps.  Block b takes destinations b, b + gridDim.x,
+// ... (the first ones listed are the hubs), a thread each; longer buckets are
+// left to the warps, the longest to the block.
+template <class Settle>
+__device__ inline void rd_fold(const RdBuf& B, const Table& T, const RdSrc& S, const int4* touched,
+                               int64_t nf, RdCnt* Cc, uint32_t* s_mem, bool want_p,
+                               Settle&& settle) {
+  // the block's buckets for a warp and for the block: thread and count; per
+  // thread the bucket's place, the value before and the one after
+  __shared__ int2 s_mid[kRdBlock], s_big[kRdBlock];
+  __shared__ int s_n[2];
+  __shared__ int32_t s_o[kRdBlock];
+  __shared__ double s_val[kRdBlock];
+  const int lane = threadIdx.x & 31;
+  uint32_t* sm = s_mem + (threadIdx.x >> 5) * kRdMidWords;
+  const int nt = __ldcg(&Cc->touched);
+  const int64_t mine = (nt - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x;  // <= 0: none
+  for (int64_t j0 = 0; j0 < mine; j0 += kRdBlock) {
+    if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
+    __syncthreads();
+    const int64_t j = j0 + threadIdx.x;
+    const bool ok = j < mine;
+    int4 ts = make_int4(0, 0, 0, 0);
+    int c = 0;
+    double old = 0.0, acc = 0.0, p = 0.0;
+    if (ok) {
+      // everything a destination needs next, at once: its count, its values
+      // and the first entries of its bucket
+      ts = touched[j * gridDim.x + blockIdx.x];
+      c = B.cnt[ts.y] & (kRdSelf - 1);
+      old = *tb_val(T, ts.y);
+      if (want_p) p = T.p[ts.y];
+      int32_t q[kRdShort];
+#pragma unroll
+      for (int k = 0; k < kRdShort; k++) q[k] = k < ts.w ? B.bucket[ts.z + k] : 0;
+      B.cnt[ts.y] = 0;
+      if (c > kRdShort) {
+        const int big = c > kRdMid ? 1 : 0;
+        (big ? s_big : s_mid)[atomicAdd(&s_n[big], 1)] = make_int2(threadIdx.x, c);
+        s_o[threadIdx.x] = ts.z;
+        s_val[threadIdx.x] = old;
+      } else {
+        acc = rd_fold_short(q, S, c, old);
+      }
+    }
+    __syncthreads();
+    const int nmid = s_n[0], nbig = s_n[1];
+    for (int k = threadIdx.x >> 5; k < nmid; k += kRdWarps) {
+      const int2 q = s_mid[k];
+      const double x = rd_fold_mid(B.bucket + s_o[q.x], S, q.y, nf, s_val[q.x], sm);
+      if (lane == 0) s_val[q.x] = x;
+    }
+    for (int k = 0; k < nbig; k++) {
+      __syncthreads();  // the shared memory of the buckets before
+      const int2 q = s_big[k];
+      const double x = rd_fold_block(B.bucket + s_o[q.x], S, q.y, nf, s_val[q.x], s_mem);
+      if (threadIdx.x == 0) s_val[q.x] = x;
+    }
+    __syncthreads();
+    if (j - lane < mine) {  // uniform in the warp
+      if (c > kRdShort) acc = s_val[threadIdx.x];
+      if (ok) *tb_val(T, ts.y) = acc;
+      settle(ok, ts, old, acc, p);
+    }
   }
 }
 
@@ -885,13 +1108,6 @@ __global__ void __launch_bounds__(kRdBlock, 1) rounds_det_kernel(RdArgs A, RdBuf
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nwarps = (int64_t)gridDim.x * kRdWarps;
-  uint32_t* sm = s_mem + (threadIdx.x >> 5) * kRdMidWords;
-  // the block's buckets for a warp and for the block: thread and count; per
-  // thread the bucket's place, the value before and the one after
-  __shared__ int2 s_mid[kRdBlock], s_big[kRdBlock];
-  __shared__ int s_n[2];
-  __shared__ int32_t s_o[kRdBlock];
-  __shared__ double s_val[kRdBlock];
   int64_t rounds = 0, pushes = 0, pushed = 0, count = A.count;
   int err = 0;
   // The vertices with pred (residual r, p, adjacency [o, o + d)) join frontier
@@ -965,73 +1181,207 @@ __global__ void __launch_bounds__(kRdBlock, 1) rounds_det_kernel(RdArgs A, RdBuf
     const RdEdges R = {BETA ? B.pe : F.e, BETA ? B.base : F.base, BETA ? B.ptile : F.tile, np, Ep};
     int64_t nins = 0;
     if (Ep > nwarps * 64)  // several edges a lane once every warp has work
-      rd_file<4>(B, T, A.off, A.col, R, F.touched, Cc, warp, nwarps, &nins);
+      rd_file<4>(B, T, A.off, A.col, R, F.touched, nullptr, Cc, warp, nwarps, &nins);
     else
-      rd_file<1>(B, T, A.off, A.col, R, F.touched, Cc, warp, nwarps, &nins);
+      rd_file<1>(B, T, A.off, A.col, R, F.touched, nullptr, Cc, warp, nwarps, &nins);
     rd_count_inserted(nins, Cc);
     grid.sync();
     if (blockIdx.x == 0 && threadIdx.x == 0) *Cz = RdCnt{};
-    // fold: block b takes destinations b, b + gridDim.x, ... (the first ones
-    // listed are the hubs), a thread each; longer buckets are left to the
-    // warps, the longest to the block
-    const int nt = __ldcg(&Cc->touched);
     const RdSrc S = BETA ? RdSrc{B.pv, B.pr, B.share} : RdSrc{F.v, F.rank, F.share};
-    const int64_t mine = (nt - (int64_t)blockIdx.x + gridDim.x - 1) / gridDim.x;  // <= 0: none
-    for (int64_t j0 = 0; j0 < mine; j0 += kRdBlock) {
-      if (threadIdx.x < 2) s_n[threadIdx.x] = 0;
-      __syncthreads();
-      const int64_t j = j0 + threadIdx.x;
-      const bool ok = j < mine;
-      int4 ts = make_int4(0, 0, 0, 0);
-      int c = 0;
-      double old = 0.0, acc = 0.0, p = 0.0;
-      if (ok) {
-        // everything a destination needs next, at once: its count, its values
-        // and the first entries of its bucket
-        ts = F.touched[j * gridDim.x + blockIdx.x];
-        c = B.cnt[ts.y] & (kRdSelf - 1);
-        old = *tb_val(T, ts.y);
-        if (!BETA) p = T.p[ts.y];
-        int32_t q[kRdShort];
-#pragma unroll
-        for (int k = 0; k < kRdShort; k++) q[k] = k < ts.w ? B.bucket[ts.z + k] : 0;
-        B.cnt[ts.y] = 0;
-        if (c > kRdShort) {
-          const int big = c > kRdMid ? 1 : 0;
-          (big ? s_big : s_mid)[atomicAdd(&s_n[big], 1)] = make_int2(threadIdx.x, c);
-          s_o[threadIdx.x] = ts.z;
-          s_val[threadIdx.x] = old;
-        } else {
-          acc = rd_fold_short(q, S, c, old);
-        }
-      }
-      __syncthreads();
-      const int nmid = s_n[0], nbig = s_n[1];
-      for (int k = threadIdx.x >> 5; k < nmid; k += kRdWarps) {
-        const int2 q = s_mid[k];
-        const double x = rd_fold_mid(B.bucket + s_o[q.x], S, q.y, nf, s_val[q.x], sm);
-        if (lane == 0) s_val[q.x] = x;
-      }
-      for (int k = 0; k < nbig; k++) {
-        __syncthreads();  // the shared memory of the buckets before
-        const int2 q = s_big[k];
-        const double x = rd_fold_block(B.bucket + s_o[q.x], S, q.y, nf, s_val[q.x], s_mem);
-        if (threadIdx.x == 0) s_val[q.x] = x;
-      }
-      __syncthreads();
-      if (j - lane < mine) {  // uniform in the warp
-        if (c > kRdShort) acc = s_val[threadIdx.x];
-        if (ok) *tb_val(T, ts.y) = acc;
-        const double thr = A.eps * (double)ts.w;
-        // with a selection the waiting and kept candidates are listed already
-        enter(N, C, ok && acc >= thr && (!BETA || old < thr), ts.x, ts.y, ts.z, ts.w, acc, p);
-      }
-    }
+    // p of the destinations, for those that enter
+    rd_fold(B, T, S, F.touched, nf, Cc, s_mem, !BETA, [&](bool ok, int4 ts, double old, double acc,
+                                                         double p) {
+      const double thr = A.eps * (double)ts.w;
+      // with a selection the waiting and kept candidates are listed already
+      enter(N, C, ok && acc >= thr && (!BETA || old < thr), ts.x, ts.y, ts.z, ts.w, acc, p);
+    });
     grid.sync();
     rounds += 1;
     pushes += np;
     pushed += Ep;
     count += (int64_t)__ldcg(&Cc->inserted);
+    err |= __ldcg(&Cc->err);
+  }
+}
+
+// Rounds into fresh sets: Nibble (KIND 0: p'[v] = p[v]/2 on the frontier and
+// share p[v]/(2 d)) and HK-PR (KIND 1: p[v] += r[v] and share
+// t r[v]/((j+1) d), r' fresh).  The new set of round k is T[k mod 3], its
+// source T[(k-1) mod 3] (T[3] in the first round); the third one, the source
+// of the round before (still the result where a Nibble round's frontier comes
+// out empty), is cleared by its list of keys, so a round costs what it
+// touches.  V | push | (wide rounds: settle |), or V | file | fold |: what a
+// round takes is a dozen us; with prefix sums for the edges, tables cleared
+// in full and every hub's adds queueing it was 52 (13 rounds of a scale-22
+// Nibble).
+struct RfArgs {
+  double t;
+  const double* c;  // thresholds by level (device)
+  int N, j0;
+  int64_t pcount, p_limit;
+};
+struct RfTabs {
+  Table T[4], P;
+  int32_t* keys[3];
+};
+
+template <bool DET, int KIND>
+__global__ void __launch_bounds__(kRdBlock, 1)
+    rounds_fresh_kernel(RdArgs A, RfArgs X, RdBuf B, RfTabs Q) {
+  extern __shared__ uint32_t s_mem[];
+  cg::grid_group grid = cg::this_grid();
+  const int lane = threadIdx.x & 31;
+  const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int64_t nwarps = (int64_t)gridDim.x * kRdWarps;
+  int64_t rounds = 0, pushes = 0, pushed = 0, pcount = X.pcount;
+  int64_t count = A.count, before = A.count;  // keys of the newest set, of its source
+  int nk[3] = {0, 0, 0};                      // keys listed per table
+  int err = 0;
+  for (int64_t b = warp * 32; b < A.in_nf; b += nwarps * 32) {
+    const int64_t i = b + lane;
+    const bool ok = i < A.in_nf;
+    const int32_t v = ok ? A.in_v[i] : 0;
+    uint32_t e;
+    rd_append(B, B.F[0], &B.cn[0], ok, v, ok ? A.in_s[i] : 0, ok ? A.deg[v] : 0, &e);
+  }
+  grid.sync();
+  for (int set = 0;; set = set == 2 ? 0 : set + 1) {
+    const int cur = (int)(rounds & 1);
+    RdCnt *Cc = &B.cn[set], *C = &B.cn[set == 2 ? 0 : set + 1];
+    RdCnt* Cz = &B.cn[set == 0 ? 2 : set - 1];
+    const RdFront &F = B.F[cur], &N = B.F[cur ^ 1];
+    // round k uses set k mod 3 and table k mod 3: the same index
+    const int src = rounds == 0 ? 3 : (set == 0 ? 2 : set - 1), old = set == 2 ? 0 : set + 1;
+    const unsigned long long fr = __ldcg(&Cc->next);
+    err |= __ldcg(&Cc->err);
+    const int64_t nf = rd_size(fr), E = rd_edges(fr);
+    const int j = X.j0 + (int)rounds;
+    int stop = 0;
+    if (err) stop = 4;
+    else if (nf == 0) stop = 1;
+    else if (rounds >= A.max_rounds || (KIND == 1 && j + 1 >= X.N)) stop = 2;
+    else if (E > A.e_max || nf > A.f_max || (A.keep_room && nf + E > B.fcap) ||
+             nf + E > A.key_limit || (KIND == 1 && pcount + nf > X.p_limit))
+      stop = 3;
+    if (stop) {  // the same decision in every thread: no barrier is left waiting
+      rd_finish(B, stop, err, cur, fr, count, rounds, pushes, pushed);
+      if (blockIdx.x == 0 && threadIdx.x == 0) {
+        // an empty Nibble frontier: the vector before the round that made it
+        const bool back = KIND == 0 && stop == 1;
+        B.out[4] = back ? before : count;
+        B.out[8] = !back ? src : rounds <= 1 ? 3 : old;
+        B.out[9] = pcount;
+      }
+      return;
+    }
+    const Table S = Q.T[src], D = Q.T[set];
+    const double c = KIND == 0 ? A.eps : X.c[j + 1];
+    const bool thr = c > 0.0;
+    const bool exact = !DET && thr && E >= A.x_min;
+    // the ranks of the frontier's ids, for buckets too long for shuffles
+    if (DET && A.need_rank)
+      rd_rank<RdIdKey>(
+          nf, F.rank, warp, nwarps, [&](int64_t i) { return RdIdKey{F.v[i]}; },
+          [](const RdIdKey& a, const RdIdKey& b) { return a.v < b.v; });
+    // V
+    int64_t nins = 0, pins = 0;
+    int emin = 0, emax = 0;
+    for (int64_t b = warp * 32; b < nf; b += nwarps * 32) {
+      const int64_t i = b + lane;
+      bool self = false;
+      int32_t v = 0, ds = 0, k0 = 1;
+      int64_t d = 0;
+      if (i < nf) {
+        v = F.v[i];
+        const int32_t s = F.s[i];
+        const double r = s >= 0 ? *tb_val(S, s) : 0.0;
+        const int64_t o0 = A.off[v];
+        d = A.off[v + 1] - o0;
+        double sh;
+        if (KIND == 0) {
+          int ins = 0;
+          ds = (int32_t)tb_find_or_insert(D, v, &ins, &Cc->err);
+          const double half = r / 2.0;
+          if (ds >= 0) *tb_val(D, ds) = half;
+          nins += ins;
+          k0 = ins ? 0 : 1;
+          sh = r / (2.0 * (double)d);
+          self = ds >= 0 && (!thr || half >= c * (double)d);
+        } else {
+          int ins = 0;
+          const int64_t ps = tb_find_or_insert(Q.P, v, &ins, &Cc->err);
+          if (ps >= 0) *tb_val(Q.P, ps) = *tb_val(Q.P, ps) + r;
+          pins += ins;
+          sh = (X.t * r) / ((double)(j + 1) * (double)d);
+        }
+        if (exact && sh > 0.0) {
+          const int be = fx_bexp(fx_bits(sh));
+          emin = max(emin, 2047 - be);
+          emax = max(emax, be);
+        }
+        B.share[i] = sh;
+        B.base[i] = o0 - (int64_t)F.e[i];
+      }
+      if (KIND == 0) {
+        rd_touch<1>(Q.keys[set], &Cc->nkeys, &ds, &k0);
+        uint32_t e;
+        rd_append(B, N, C, self, v, ds, d, &e);
+      }
+    }
+    if (exact) {
+      emin = __reduce_max_sync(0xffffffffu, emin);
+      emax = __reduce_max_sync(0xffffffffu, emax);
+      if (lane == 0 && (emin | emax)) {
+        atomicMax(&Cc->emin, emin);
+        atomicMax(&Cc->emax, emax);
+      }
+    }
+    if (KIND == 1) {
+      for (int o = 16; o > 0; o >>= 1) pins += __shfl_xor_sync(0xffffffffu, pins, o);
+      if (lane == 0 && pins) atomicAdd(&Cc->pinserted, (unsigned long long)pins);
+    }
+    // the table after next, by its keys
+    for (int64_t i = warp * 32 + lane; i < nk[old]; i += nwarps * 32) {
+      const int32_t k = Q.keys[old][i];
+      const Table& Z = Q.T[old];
+      if (Z.dense) {
+        Z.dval[k] = 0.0;
+        Z.bits[k >> 5] = 0;  // every key of the word goes
+      } else {
+        Z.s[k] = Slot{};
+      }
+    }
+    rd_count_inserted(nins, Cc);
+    grid.sync();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *Cz = RdCnt{};
+    const RdEdges R = {F.e, B.base, F.tile, nf, E};
+    if (DET) {
+      int64_t fins = 0;
+      if (E > nwarps * 64)
+        rd_file<4>(B, D, A.off, A.col, R, F.touched, Q.keys[set], Cc, warp, nwarps, &fins);
+      else
+        rd_file<1>(B, D, A.off, A.col, R, F.touched, Q.keys[set], Cc, warp, nwarps, &fins);
+      rd_count_inserted(fins, Cc);
+      grid.sync();
+      rd_fold(B, D, RdSrc{F.v, F.rank, B.share}, F.touched, nf, Cc, s_mem, false,
+              [&](bool ok, int4 ts, double old_v, double acc, double) {
+                const double th = c * (double)ts.w;
+                uint32_t e;
+                rd_append(B, N, C, ok && old_v < th && acc >= th, ts.x, ts.y, ts.w, &e);
+              });
+    } else {
+      const RdDest dest = {D, Q.keys[set], c, thr};
+      rd_push_round(B, dest, A.hot, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps, grid);
+    }
+    grid.sync();
+    rounds += 1;
+    pushes += nf;
+    pushed += E;
+    before = count;
+    nk[set] = __ldcg(&Cc->nkeys);
+    nk[old] = 0;
+    count = nk[set];
+    pcount += (int64_t)__ldcg(&Cc->pinserted);
     err |= __ldcg(&Cc->err);
   }
 }
@@ -1056,18 +1406,25 @@ bool rounds_take(const lgc_ctx* ctx, const lgc_graph* g, const RoundsMem& M, int
   return !beta || nf <= kRdFront;
 }
 
-int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, const int32_t* fv,
-                    const int32_t* fs, int64_t nf, int64_t E, int64_t count, double alpha,
-                    double cs, double cn, double eps, int rule, bool det, double beta,
-                    int64_t x_min, int64_t max_rounds, int64_t key_limit, RoundsOut* out) {
+namespace {
+
+// What a launch is given: limits, buffers carved from M's slab, arguments.
+struct RdLaunch {
+  RdArgs A{};
+  RdBuf B{};
+};
+
+// fresh_keys: room for the key lists of fresh sets (else null); levels: room
+// for that many thresholds (device) in *levels.  no_room set: M.no_det is.
+int rd_prepare(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, int64_t slots, const int32_t* fv,
+               const int32_t* fs, int64_t nf, bool det, bool sel, bool staged, int64_t x_min,
+               int64_t max_rounds, int64_t key_limit, int32_t** fresh_keys, int64_t levels,
+               double** level_c, RdLaunch* L, bool* no_room) {
   cudaStream_t s = ctx->stream;
-  const bool sel = beta < 1.0;
+  RdBuf& B = L->B;
+  RdArgs& A = L->A;
+  *no_room = false;
   const bool wide = !det && x_min <= rd_emax(g);  // wide rounds may occur
-  RdKernel kern = det ? (sel ? rounds_det_kernel<true> : rounds_det_kernel<false>)
-                      : (sel ? rounds_kernel<true> : rounds_kernel<false>);
-  const size_t smem = det ? (size_t)kRdSmemWords * 4 : 0;
-  LGC_CUDA_TRY(cudaFuncSetAttribute((const void*)kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                    (int)smem));
   const int64_t e_max = rd_emax(g);
   // a next frontier has at most nf + E entries, all distinct
   const int64_t fcap = std::min<int64_t>(g->n, 2 * kRdEdges);
@@ -1077,12 +1434,12 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
     if (dalloc_t(ctx, &M.bucket, (size_t)g->nnz) != LGC_OK) {
       M.bucket = nullptr;
       M.no_det = true;
+      *no_room = true;
       return LGC_OK;
     }
   }
   const int64_t tiles = e_max / 32 + 1;
-  // carve one slab
-  RdBuf B{};
+  // carve one slab; staged: a V phase writes the shares (else the entries' owners)
   size_t at = 0;
   char* base = nullptr;
   auto carve = [&](auto** p, int64_t n, bool want) {
@@ -1093,7 +1450,7 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
   auto lay = [&] {
     at = 0;
     carve(&B.cn, 3, true);
-    carve(&B.out, 8, true);
+    carve(&B.out, 16, true);
     for (RdFront& F : B.F) {
       carve(&F.v, fcap, true);
       carve(&F.s, fcap, true);
@@ -1101,20 +1458,23 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
       carve(&F.tile, tiles, true);
       carve(&F.rank, fcap, true);
       carve(&F.brank, fcap, true);
-      carve(&F.share, fcap, det && !sel);
-      carve(&F.base, fcap, det && !sel);
-      carve(&F.r0, fcap, det && !sel);
-      carve(&F.p0, fcap, det && !sel);
+      carve(&F.share, fcap, !staged);
+      carve(&F.base, fcap, !staged);
+      carve(&F.r0, fcap, !staged);
+      carve(&F.p0, fcap, !staged);
       carve(&F.touched, std::min<int64_t>(g->n, e_max + fcap), det);
     }
-    carve(&B.share, f_max, !det || sel);
-    carve(&B.base, f_max, !det || sel);
+    carve(&B.share, f_max, staged);
+    carve(&B.base, f_max, staged);
     carve(&B.key, f_max, sel);
     carve(&B.pe, f_max, sel);
     carve(&B.ptile, tiles, sel);
     carve(&B.pv, f_max, sel && det);
     carve(&B.pr, f_max, sel && det);
     carve(&B.touched, std::min<int64_t>(g->n, e_max), wide);
+    if (fresh_keys)
+      for (int k = 0; k < 3; k++) carve(&fresh_keys[k], std::min<int64_t>(g->n, e_max + fcap), true);
+    if (level_c) carve(level_c, levels, levels > 0);
   };
   lay();
   if (at > M.slab_bytes) {
@@ -1130,53 +1490,54 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
   B.tiles = (int32_t)tiles;
   B.bucket = M.bucket;
   if (det || wide) {
-    if (M.slots != T.cap) {
+    if (M.slots != slots) {
       dfree(ctx, M.per_slot);
       M.per_slot = nullptr;
       M.slots = 0;
-      const size_t bytes = (4 + (wide ? sizeof(Fx) : 0)) * (size_t)T.cap;
+      const size_t bytes = (4 + (wide ? sizeof(Fx) : 0)) * (size_t)slots;
       LGC_TRY(dalloc_t(ctx, &M.per_slot, bytes));
-      M.slots = T.cap;
+      M.slots = slots;
       LGC_CUDA_TRY(cudaMemsetAsync(M.per_slot, 0, bytes, s));
     }
     // the sums first: they need 16-byte alignment
     B.xacc = wide ? reinterpret_cast<Fx*>(M.per_slot) : nullptr;
-    B.cnt = reinterpret_cast<int32_t*>(M.per_slot + (wide ? sizeof(Fx) * T.cap : 0));
+    B.cnt = reinterpret_cast<int32_t*>(M.per_slot + (wide ? sizeof(Fx) * slots : 0));
   }
   LGC_CUDA_TRY(cudaMemsetAsync(B.cn, 0, 3 * sizeof(RdCnt), s));
-  RdArgs A{};
   A.off = g->off;
   A.col = g->col;
   A.deg = g->deg;
   A.in_v = fv;
   A.in_s = fs;
   A.in_nf = nf;
-  A.alpha = alpha;
-  A.cs = cs;
-  A.cn = cn;
-  A.eps = eps;
-  A.beta = beta;
-  A.rule = rule;
   A.need_rank = rd_ranks(g) ? 1 : 0;
   A.gbits = 1;  // sums of at most max_deg terms: max_deg < 2^gbits
   while (A.gbits < 62 && (int64_t{1} << A.gbits) <= g->max_deg) A.gbits++;
   A.keep_room = fcap < g->n ? 1 : 0;
   A.x_min = det ? INT64_MAX : x_min;
-  A.count = count;
   A.max_rounds = std::min<int64_t>(max_rounds, kRdRounds);
   A.e_max = e_max;
   A.f_max = f_max;
   A.key_limit = key_limit;
-  Table Tk = T;
-  void* args[] = {&A, &B, &Tk};
+  A.hot = g->hot;
+  return LGC_OK;
+}
+
+// Launches kern with args and reads the state it ended in.
+int rd_run(lgc_ctx* ctx, lgc_graph* g, const void* kern, void** args, const RdBuf& B, bool det,
+           RoundsOut* out) {
+  cudaStream_t s = ctx->stream;
+  const size_t smem = det ? (size_t)kRdSmemWords * 4 : 0;
+  LGC_CUDA_TRY(
+      cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
   {
     ProfScope ps(ctx, det ? LGC_PROF_DET_EDGE : LGC_PROF_EDGEMAP, 0.0);
     // one block per SM: the rounds are small, and fewer blocks wait at each
     // grid barrier
-    LGC_CUDA_TRY(cudaLaunchCooperativeKernel((const void*)kern, ctx->sms, kRdBlock, args, smem, s));
+    LGC_CUDA_TRY(cudaLaunchCooperativeKernel(kern, ctx->sms, kRdBlock, args, smem, s));
     LGC_COUNT_LAUNCH(ctx);
   }
-  LGC_CUDA_TRY(cudaMemcpyAsync(ctx->h_scratch, B.out, 64, cudaMemcpyDeviceToHost, s));
+  LGC_CUDA_TRY(cudaMemcpyAsync(ctx->h_scratch, B.out, 80, cudaMemcpyDeviceToHost, s));
   LGC_CUDA_TRY(cudaStreamSynchronize(s));
   const int64_t* o = ctx->h_scratch;
   if (o[0] != 0) return LGC_ETABLEFULL;
@@ -1190,6 +1551,8 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
   out->rounds = o[5];
   out->pushes = o[6];
   out->pushed = o[7];
+  out->tab = (int)o[8];
+  out->pcount = o[9];
   if (ctx->profile && !ctx->prof_pending.empty())
     ctx->prof_pending.back().bytes += 24.0 * (double)out->pushed + 88.0 * (double)out->pushes;
   // host-driven deterministic rounds take the frontier in ascending id
@@ -1197,6 +1560,69 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
     LGC_TRY(radix_sort_u32_i32(ctx, (uint32_t*)out->v, out->s, (uint32_t*)B.F[cur ^ 1].v,
                                B.F[cur ^ 1].s, out->nf, bits_for(g->n)));
   return LGC_OK;
+}
+
+}  // namespace
+
+int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, const int32_t* fv,
+                    const int32_t* fs, int64_t nf, int64_t E, int64_t count, double alpha,
+                    double cs, double cn, double eps, int rule, bool det, double beta,
+                    int64_t x_min, int64_t max_rounds, int64_t key_limit, RoundsOut* out) {
+  (void)E;
+  const bool sel = beta < 1.0;
+  RdKernel kern = det ? (sel ? rounds_det_kernel<true> : rounds_det_kernel<false>)
+                      : (sel ? rounds_kernel<true> : rounds_kernel<false>);
+  RdLaunch L;
+  bool no_room;
+  LGC_TRY(rd_prepare(ctx, g, M, T.cap, fv, fs, nf, det, sel, !det || sel, x_min, max_rounds,
+                     key_limit, nullptr, 0, nullptr, &L, &no_room));
+  if (no_room) return LGC_OK;
+  L.A.alpha = alpha;
+  L.A.cs = cs;
+  L.A.cn = cn;
+  L.A.eps = eps;
+  L.A.beta = beta;
+  L.A.rule = rule;
+  L.A.count = count;
+  Table Tk = T;
+  void* args[] = {&L.A, &L.B, &Tk};
+  return rd_run(ctx, g, (const void*)kern, args, L.B, det, out);
+}
+
+int rounds_fresh(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const RoundsFresh& q, const Table* T,
+                 const Table* P, int64_t pcount, const int32_t* fv, const int32_t* fs, int64_t nf,
+                 int64_t E, bool det, int64_t x_min, int64_t max_rounds, int64_t key_limit,
+                 int64_t p_limit, RoundsOut* out) {
+  (void)E;
+  const bool hk = q.c != nullptr;
+  RdLaunch L;
+  RfArgs X{};
+  RfTabs Q{};
+  bool no_room;
+  double* c = nullptr;
+  LGC_TRY(rd_prepare(ctx, g, M, T[0].cap, fv, fs, nf, det, false, true, x_min, max_rounds,
+                     key_limit, Q.keys, hk ? q.N + 1 : 0, &c, &L, &no_room));
+  if (no_room) return LGC_OK;
+  if (hk) {
+    LGC_CUDA_TRY(cudaMemcpyAsync(c, q.c, sizeof(double) * (q.N + 1), cudaMemcpyHostToDevice,
+                                 ctx->stream));
+    X.t = q.t;
+    X.c = c;
+    X.N = q.N;
+    X.j0 = q.j;
+    X.pcount = pcount;
+    X.p_limit = p_limit;
+    Q.P = *P;
+  }
+  L.A.eps = q.eps;
+  L.A.count = q.count;
+  for (int k = 0; k < 4; k++) Q.T[k] = T[k];
+  const void* kern = det ? (hk ? (const void*)rounds_fresh_kernel<true, 1>
+                               : (const void*)rounds_fresh_kernel<true, 0>)
+                         : (hk ? (const void*)rounds_fresh_kernel<false, 1>
+                               : (const void*)rounds_fresh_kernel<false, 0>);
+  void* args[] = {&L.A, &X, &L.B, &Q};
+  return rd_run(ctx, g, kern, args, L.B, det, out);
 }
 
 }  // namespace lgc

@@ -1,4 +1,4 @@
-// Consecutive small PR-Nibble rounds in one cooperative launch (rounds.cu).
+// Consecutive small rounds in one cooperative launch (rounds.cu).
 #pragma once
 
 #include "common.cuh"
@@ -31,6 +31,8 @@ struct RoundsMem {
 struct RoundsOut {
   int32_t *v = nullptr, *s = nullptr;
   int64_t nf = 0, E = 0, count = 0, rounds = 0, pushes = 0, pushed = 0;
+  int tab = 3;         // fresh sets: which table holds the set reached (3: the first)
+  int64_t pcount = 0;  // HK-PR: keys of p
 };
 
 // Whether the rounds kernel takes a frontier of nf vertices and E edges
@@ -48,5 +50,25 @@ int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, co
                     const int32_t* fs, int64_t nf, int64_t E, int64_t count, double alpha,
                     double cs, double cn, double eps, int rule, bool det, double beta,
                     int64_t x_min, int64_t max_rounds, int64_t key_limit, RoundsOut* out);
+
+// Rounds that fill a fresh set from the frontier: Nibble (c null; threshold
+// eps, 0: every inserted vertex goes on) or HK-PR from level j of N (t, and
+// the levels' threshold factors c[0..N]).
+struct RoundsFresh {
+  double eps = 0.0, t = 0.0;
+  const double* c = nullptr;
+  int N = 0, j = 0;
+  int64_t count = 0;  // keys of the first set
+};
+
+// Runs such rounds: the first reads the set T[3], the others T[0..2] in turn
+// (cleared, of one form; key_limit keys each).  HK-PR adds into P (pcount
+// keys, at most p_limit) and stops before its last level.  Nibble stops with
+// an empty frontier at the round that made it, T[tab] being the vector before
+// that round, as the method returns it.  rounds 0 in *out: as above.
+int rounds_fresh(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const RoundsFresh& q, const Table* T,
+                 const Table* P, int64_t pcount, const int32_t* fv, const int32_t* fs, int64_t nf,
+                 int64_t E, bool det, int64_t x_min, int64_t max_rounds, int64_t key_limit,
+                 int64_t p_limit, RoundsOut* out);
 
 }  // namespace lgc

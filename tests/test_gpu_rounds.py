@@ -91,6 +91,68 @@ def test_beta_rounds(ctx, beta, rule, mode):
     g.close()
 
 
+@pytest.mark.parametrize("pull", [0, 1], ids=["wide", "plain"])
+@pytest.mark.parametrize("c", [1100, 5000])
+def test_hot_destinations(ctx, c, pull):
+    """Frontiers of more than 2048 vertices that all push into the two hubs
+    (degree 1024 and more): the hubs' adds are combined."""
+    off, col = fan(c, 3)
+    g = lgc.Graph(ctx, off, col)
+    ctx.set_option(lgc.OPT_PULL, pull)
+    try:
+        for x in (0, 5):
+            for ref, (p, st) in (
+                    (oracle.prnibble(off, col, x, 0.05, 1e-8),
+                     lgc.prnibble(g, x, 0.05, 1e-8, mode="atomic")),
+                    (oracle.nibble(off, col, x, 9, 1e-9), lgc.nibble(g, x, 9, 1e-9)),
+                    (oracle.hkpr(off, col, x, 4.0, 9, 1e-9), lgc.hkpr(g, x, 4.0, 9, 1e-9))):
+                assert (st.rounds, st.pushes, st.pushed_edges) == (ref.rounds, ref.pushes,
+                                                                   ref.pushed_edges)
+                assert np.array_equal(p.idx, ref.idx)
+                assert np.abs(p.val - ref.val).sum() <= 1e-12 * ref.val.sum()
+    finally:
+        ctx.set_option(lgc.OPT_PULL, 0)
+        g.close()
+
+
+FRESH = {"star1500": (lambda: inputs.star(1500), 1e-6),
+         "path40": (lambda: inputs.path(40), 1e-3),
+         "grid17": (lambda: inputs.grid3d(17), 1e-7),
+         "rmat12": (lambda: inputs.rmat(12, seed=1), 1e-6),
+         "rmat16": (lambda: inputs.rmat(16, seed=1), 1e-7)}
+
+
+@pytest.mark.parametrize("mode", ["atomic", "det"])
+@pytest.mark.parametrize("form", [0, 1, 2], ids=["auto", "hashed", "dense"])
+@pytest.mark.parametrize("name", list(FRESH))
+def test_fresh_set_rounds(ctx, name, form, mode):
+    """Nibble (its early exit too) and HK-PR rounds into fresh sets."""
+    make, eps = FRESH[name]
+    off, col = make()
+    g = lgc.Graph(ctx, off, col)
+    ctx.set_option(lgc.OPT_TABLE_FORM, form)
+    try:
+        x = inputs.config1_seed(off, col)
+        runs = []
+        for T, e in ((1, eps), (2, eps), (17, eps), (25, 300 * eps), (6, 0.3), (4, 0.0)):
+            runs.append((oracle.nibble(off, col, x, T, e), lgc.nibble(g, x, T, e, mode=mode)))
+        for t, N, e in ((5.0, 12, eps), (5.0, 2, eps), (1.0, 1, eps), (8.0, 20, 100 * eps),
+                        (2.0, 4, 0.0)):
+            runs.append((oracle.hkpr(off, col, x, t, N, e), lgc.hkpr(g, x, t, N, e, mode=mode)))
+        for ref, (p, st) in runs:
+            assert (st.rounds, st.pushes, st.pushed_edges) == (ref.rounds, ref.pushes,
+                                                               ref.pushed_edges)
+            assert st.touched == ref.touched
+            assert np.array_equal(p.idx, ref.idx)
+            if mode == "det":
+                assert np.array_equal(p.val, ref.val)
+            else:
+                assert np.abs(p.val - ref.val).sum() <= 1e-12 * ref.val.sum()
+    finally:
+        ctx.set_option(lgc.OPT_TABLE_FORM, 0)
+        g.close()
+
+
 def test_wide_atomic_rounds_sum_as_pull_rounds(ctx):
     """Every round of this diffusion is one that the host would run as a pull
     round: the exact sums give the same bits either way."""
