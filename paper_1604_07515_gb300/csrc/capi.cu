@@ -294,41 +294,104 @@ int build_heavy_list(lgc_ctx* ctx, lgc_graph* g) {
   return st;
 }
 
-// The largest (degree, lowest id first) below `below` into *top, packed
-// degree << 32 | ~id.
-__global__ void hot_kernel(const int32_t* __restrict__ deg, int64_t n, unsigned long long below,
-                           unsigned long long* __restrict__ top) {
-  unsigned long long m = 0;
+// How many degrees have each bit length.
+__global__ void degree_bits_kernel(const int32_t* __restrict__ deg, int64_t n,
+                                   unsigned long long* __restrict__ len) {
+  __shared__ unsigned s_len[33];
+  for (int i = threadIdx.x; i < 33; i += blockDim.x) s_len[i] = 0;
+  __syncthreads();
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
-    const unsigned long long k =
-        ((unsigned long long)(uint32_t)deg[v] << 32) | (uint32_t)~(uint32_t)v;
-    if (k < below && k > m) m = k;
+    const int b = 32 - __clz(deg[v]);
+    if (b > 10) atomicAdd(&s_len[b], 1u);  // degrees of kHotDeg or more
   }
-  for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
-  if ((threadIdx.x & 31) == 0 && m) atomicMax(top, m);
+  __syncthreads();
+  for (int i = threadIdx.x; i < 33; i += blockDim.x)
+    if (s_len[i]) atomicAdd(&len[i], (unsigned long long)s_len[i]);
 }
 
+__global__ void degree_list_kernel(const int32_t* __restrict__ deg, int64_t n, int32_t least,
+                                   int2* __restrict__ list, int cap, int* __restrict__ count) {
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x)
+    if (deg[v] >= least) {
+      const int at = atomicAdd(count, 1);
+      if (at < cap) list[at] = make_int2(deg[v], (int32_t)v);
+    }
+}
+
+// The graph's hot vertices: the degrees' bit lengths give a threshold that at
+// least kHot vertices reach (fewer where the next would pass kMostHot), whose
+// list the host sorts.
 int build_hot(lgc_ctx* ctx, lgc_graph* g) {
+  constexpr int kMostHot = 16384;
+  static_assert(kHotDeg == 1024, "bit lengths above 10");
   if (g->max_deg < kHotDeg) return LGC_OK;
-  unsigned long long* top = nullptr;
-  unsigned long long last = ~0ull;
-  LGC_TRY(dalloc_t(ctx, &top, 1));
+  cudaStream_t s = ctx->stream;
+  const int grid = std::min(grid_for(g->n), 4 * ctx->sms);
+  char* buf = nullptr;
+  LGC_TRY(dalloc_t(ctx, &buf, 512 + sizeof(int2) * kMostHot));
   int st = LGC_OK;
-  for (int h = 0; h < kHot && st == LGC_OK; h++) {
-    if (cudaMemsetAsync(top, 0, 8, ctx->stream)) st = LGC_ECUDA;
-    hot_kernel<<<std::min(grid_for(g->n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(g->deg, g->n,
-                                                                                   last, top);
+  do {
+    unsigned long long len[33];
+    if (cudaMemsetAsync(buf, 0, 512, s)) { st = LGC_ECUDA; break; }
+    degree_bits_kernel<<<grid, kBlock, 0, s>>>(g->deg, g->n, (unsigned long long*)buf);
     LGC_COUNT_LAUNCH(ctx);
-    if (cudaMemcpyAsync(ctx->h_scratch, top, 8, cudaMemcpyDeviceToHost, ctx->stream) ||
-        cudaStreamSynchronize(ctx->stream))
+    if (cudaMemcpyAsync(len, buf, sizeof len, cudaMemcpyDeviceToHost, s) ||
+        cudaStreamSynchronize(s)) {
       st = LGC_ECUDA;
-    if (st != LGC_OK) break;
-    last = (unsigned long long)ctx->h_scratch[0];
-    if ((int32_t)(last >> 32) < kHotDeg) break;
-    g->hot.v[h] = (int32_t)~(uint32_t)last;
-  }
-  dfree(ctx, top);
+      break;
+    }
+    int b = 32;
+    unsigned long long many = len[32];
+    while (b > 11 && many < kHot && many + len[b - 1] <= kMostHot) many += len[--b];
+    if (many == 0 || many > kMostHot) break;
+    int* count = (int*)(buf + 33 * 8);
+    int2* list = (int2*)(buf + 512);
+    degree_list_kernel<<<grid, kBlock, 0, s>>>(g->deg, g->n, (int32_t)1 << (b - 1), list, kMostHot,
+                                               count);
+    LGC_COUNT_LAUNCH(ctx);
+    std::vector<int2> h((size_t)many);
+    if (cudaMemcpyAsync(h.data(), list, sizeof(int2) * many, cudaMemcpyDeviceToHost, s) ||
+        cudaStreamSynchronize(s)) {
+      st = LGC_ECUDA;
+      break;
+    }
+    const size_t k = std::min<size_t>(h.size(), kHot);
+    std::partial_sort(h.begin(), h.begin() + k, h.end(), [](const int2& x, const int2& y) {
+      return x.x > y.x || (x.x == y.x && x.y < y.y);
+    });
+    // a multiplier under which no two of them share an entry: one in eight
+    // does for 32 of 256
+    int2 tab[kHotTab];
+    int32_t ids[kHot];
+    uint32_t mult = 0x9E3779B1u;
+    bool ok = false;
+    for (int tries = 0; tries < 4096 && !ok; tries++, mult = mult * 1664525u + 1013904223u) {
+      mult |= 1u;
+      ok = true;
+      for (int2& e : tab) e = make_int2(-1, 0);
+      for (size_t i = 0; i < k && ok; i++) {
+        int2& e = tab[(uint32_t)h[i].y * mult >> (32 - kHotBits)];
+        ok = e.x < 0;
+        e = make_int2(h[i].y, (int)i);
+      }
+      if (ok) break;
+    }
+    if (!ok) break;  // no combining: speed only
+    for (int i = 0; i < kHot; i++) ids[i] = i < (int)k ? h[i].y : -1;
+    if ((st = dalloc_t(ctx, &g->hot_mem, kHotTab + kHot)) != LGC_OK) break;
+    if (cudaMemcpyAsync(g->hot_mem, tab, sizeof tab, cudaMemcpyHostToDevice, s) ||
+        cudaMemcpyAsync(g->hot_mem + kHotTab, ids, sizeof ids, cudaMemcpyHostToDevice, s) ||
+        cudaStreamSynchronize(s)) {
+      st = LGC_ECUDA;
+      break;
+    }
+    g->hot.tab = g->hot_mem;
+    g->hot.ids = (const int32_t*)(g->hot_mem + kHotTab);
+    g->hot.mult = mult;
+  } while (0);
+  dfree(ctx, buf);
   return st;
 }
 
@@ -950,6 +1013,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     if (g->light_det != g->light) dfree(ctx, g->light_det);
     dfree(ctx, g->light);
     dfree(ctx, g->recip);
+    dfree(ctx, g->hot_mem);
     cudaStreamSynchronize(s);
     delete g;
     return st;
@@ -990,6 +1054,7 @@ void lgc_graph_destroy(lgc_graph* g) {
   if (g->light_det != g->light) dfree(ctx, g->light_det);
   dfree(ctx, g->light);
   dfree(ctx, g->recip);
+  dfree(ctx, g->hot_mem);
   cudaStreamSynchronize(ctx->stream);
   delete g;
 }

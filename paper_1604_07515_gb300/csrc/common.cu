@@ -287,7 +287,8 @@ struct DenseKeptWord {
   const double* src;
   int64_t n;
   int positive_only;
-  __device__ uint32_t operator()(int64_t w, bool in) const {
+  __device__ void marked(int) const {}
+  __device__ uint32_t operator()(int64_t w, bool in, int*) const {
     const uint32_t m = in ? T.bits[w] : 0u;
     if (!positive_only) return m;
     return filter_words(

@@ -248,12 +248,18 @@ struct lgc_ctx {
 };
 
 namespace lgc {
-// The vertices of highest degree (of kHotDeg or more; -2: none), whose adds the
-// push kernels combine (edges.cuh).
-constexpr int kHot = 4;
+// The vertices of highest degree (kHot at most, of degree kHotDeg or more),
+// whose adds the push kernels combine (edges.cuh): their ids, and a table
+// {vertex, index} in which vertex v stands at (v * mult) >> (32 - kHotBits)
+// (device memory; tab null: none).
+constexpr int kHot = 32;
+constexpr int kHotBits = 8;
+constexpr int kHotTab = 1 << kHotBits;
 constexpr int32_t kHotDeg = 1024;
 struct HotSet {
-  int32_t v[kHot] = {-2, -2, -2, -2};
+  const int2* tab = nullptr;
+  const int32_t* ids = nullptr;
+  uint32_t mult = 1;
 };
 }  // namespace lgc
 
@@ -292,6 +298,7 @@ struct lgc_graph {
   lgc::Recip* recip = nullptr;  // 1 / d by degree d < recip_n (device)
   int32_t recip_n = 0;
   lgc::HotSet hot;
+  int2* hot_mem = nullptr;  // its table and ids
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
   int pull_batch = 8;          // edges per lane per batch in heavy pull gathers (tuned)
   int pull_group = 32;         // lanes per work item in heavy pull gathers (tuned)

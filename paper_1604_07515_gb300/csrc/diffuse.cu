@@ -230,7 +230,9 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
                                         const int64_t* epos, const int64_t* foff, int64_t nf,
                                         int64_t E, const HotSet& H, Table D, double c, int fmode,
                                         int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
-  HotSum S;
+  __shared__ HotShared s_tab;
+  HotLane<double> S;
+  hot_load(H, s_tab);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;  // counted once per block
@@ -247,7 +249,7 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
         sh[k] = share[src[k]];
       }
     }
-    hot_take(H, S, w, sh);
+    if (H.tab) hot_take(H, s_tab, S, w, sh);
     // Resolve every item's slot before any atomic, so the first-probe loads
     // (or bitmap loads) of all items are in flight together.
     int32_t slot[kEdgeItems];
@@ -308,8 +310,8 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
   });
   // the hot vertices' sums, each as one add: the one that takes the vertex
   // across its threshold appends it
-  hot_flush<kBlock / 32>(S, [&](int h, double sh) {
-    const int32_t w = H.v[h];
+  const auto join = [](double& a, double x) { a = a + x; };
+  hot_flush<kBlock / 32>(H, S, join, [&](int32_t w, double sh) {
     int ins = 0;
     const int64_t s = tb_find_or_insert(D, w, &ins, &C->err);
     if (s < 0) return;
@@ -356,8 +358,10 @@ __global__ void __launch_bounds__(kBlock)
     emap_red_kernel(const int32_t* __restrict__ col, const double* __restrict__ share,
                     const int64_t* __restrict__ epos, const int64_t* __restrict__ foff,
                     int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev, HotSet H,
-                    Table D, Counters* C) {
-  HotSum S;
+                    Table D, int mark, Counters* C) {
+  __shared__ HotShared s_tab;
+  HotLane<double> S;
+  hot_load(H, s_tab);
   const int64_t E = min(E_host, *E_dev);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -375,23 +379,20 @@ __global__ void __launch_bounds__(kBlock)
         sh[k] = share[src[k]];
       }
     }
-    hot_take(H, S, w, sh);
+    if (H.tab) hot_take(H, s_tab, S, w, sh);
     if (D.dense) {
-      // nothing waits for a result here: the add and the presence bit are both
-      // reductions; the keys this round inserted are counted by the caller
-      // from the bitmap's population before and after.  A bit that is set
-      // already is not set again (a read that may be served from L1: stale, it
-      // only misses bits)
-      uint32_t b[kRedItems];
+      // nothing waits for a result here: the adds are reductions, and the keys
+      // they create are marked by the filter pass that follows (DenseQualWord)
+      // or, without one (mark) or where the share is zero, by another reduction
+      // unless they are marked already
 #pragma unroll
-      for (int k = 0; k < kRedItems; k++) {
-        b[k] = w[k] >= 0 ? D.bits[w[k] >> 5] : ~0u;
+      for (int k = 0; k < kRedItems; k++)
         if (w[k] >= 0) atomicAdd(&D.dval[w[k]], sh[k]);
-      }
 #pragma unroll
       for (int k = 0; k < kRedItems; k++) {
+        if (w[k] < 0 || (!mark && sh[k] > 0.0)) continue;
         const uint32_t m = 1u << (w[k] & 31);
-        if (!(b[k] & m)) atomicOr(&D.bits[w[k] >> 5], m);
+        if (!(__ldcg(&D.bits[w[k] >> 5]) & m)) nins += !(atomicOr(&D.bits[w[k] >> 5], m) & m);
       }
     } else {
 #pragma unroll
@@ -404,48 +405,62 @@ __global__ void __launch_bounds__(kBlock)
       }
     }
   });
-  hot_flush<kBlock / 32>(S, [&](int h, double sh) {
+  const auto join = [](double& a, double x) { a = a + x; };
+  hot_flush<kBlock / 32>(H, S, join, [&](int32_t w, double sh) {
     int ins = 0;
-    const int64_t s = tb_find_or_insert(D, H.v[h], &ins, &C->err);
+    const int64_t s = tb_find_or_insert(D, w, &ins, &C->err);
     if (s >= 0) atomicAdd(tb_val(D, s), sh);
-    nins += D.dense ? 0 : ins;  // a dense set's keys are counted from its bitmap
+    nins += ins;
   });
   flush_count(nins, &C->inserted);
 }
 
-// sign * (set bits of the bitmap) added into *out, one atomic per block.
-__global__ void bits_pop_kernel(const uint32_t* __restrict__ bits, int64_t words, int sign,
-                                int64_t* out) {
-  __shared__ unsigned long long s_pop;
-  if (threadIdx.x == 0) s_pop = 0;
-  __syncthreads();
-  unsigned long long c = 0;
-  for (int64_t w = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; w < words;
-       w += (int64_t)gridDim.x * blockDim.x)
-    c += __popc(bits[w]);
-  for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
-  if ((threadIdx.x & 31) == 0 && c) atomicAdd(&s_pop, c);
-  __syncthreads();
-  if (threadIdx.x == 0 && s_pop)
-    atomicAdd((unsigned long long*)out, (unsigned long long)((int64_t)sign * (int64_t)s_pop));
-}
-
-// Filter of a dense set, in ascending vertex order: vertex v qualifies when it
-// is a key and its value reaches c*d(v) (kFmThreshold) or always
+// Filter of a dense set after a bulk push, in ascending vertex order.  The
+// push leaves the presence bits of the keys it created to this pass, which
+// reads the values anyway: a vertex with a value that is not zero is a key
+// (the push marks the destinations of zero shares itself).  Vertex v qualifies
+// when it is a key and its value reaches c*d(v) (kFmThreshold) or always
 // (kFmInserted); the qualifying vertices are compacted (words_compact), their
-// degrees summed.
+// degrees summed, and the new keys counted.
 struct DenseQualWord {
   Table D;
   const int32_t* deg;
   int64_t n;
   LiteThr c;
   int fmode;
-  __device__ uint32_t operator()(int64_t w, bool in) const {
+  int64_t* inserted;
+  __device__ void marked(int k) const {
+    atomicAdd((unsigned long long*)inserted, (unsigned long long)k);
+  }
+  __device__ uint32_t operator()(int64_t w, bool in, int* fresh) const {
+    const int lane = threadIdx.x & 31;
+    const int64_t wb = w - lane;
     const uint32_t m = in ? D.bits[w] : 0u;
-    if (fmode != kFmThreshold) return m;
-    return filter_words(
-        m, w, n, [&](int64_t v) { return D.dval[v]; },
-        [&](int64_t v, double x) { return lite_reaches(x, c, deg[v]); });
+    double x[kCmpWarpWords];
+#pragma unroll
+    for (int j = 0; j < kCmpWarpWords; j++) {
+      const int64_t v = (wb + j) * 32 + lane;
+      x[j] = v < n ? D.dval[v] : 0.0;
+    }
+    uint32_t q = 0;
+#pragma unroll
+    for (int j = 0; j < kCmpWarpWords; j++) {
+      const int64_t v = (wb + j) * 32 + lane;
+      const uint32_t mj = __shfl_sync(0xffffffffu, m, j);
+      const bool nz = __double_as_longlong(x[j]) != 0;  // no value is -0.0
+      const uint32_t key = mj | __ballot_sync(0xffffffffu, nz);
+      const uint32_t b = fmode == kFmThreshold
+                             ? __ballot_sync(0xffffffffu, nz && lite_reaches(x[j], c, deg[v]))
+                             : key;
+      if (lane == j) {
+        q = b;
+        if (key != m) {
+          D.bits[w] = key;
+          *fresh = __popc(key & ~m);
+        }
+      }
+    }
+    return q;
   }
 };
 
@@ -1567,28 +1582,19 @@ struct PushWork {
       if (nrec > 0) {
         int64_t tiles = ceil_div(nrec, kEdgeTile);
         int grid = (int)(tiles < (ctx->sms * 16) ? tiles : (ctx->sms * 16));
-        // a dense destination's inserted keys: population after - before
-        const int64_t words = (g->n + 31) / 32;
-        const int pg = std::min(grid_for(words), ctx->sms * 8);
-        if (D.dense) {
-          bits_pop_kernel<<<pg, kBlock, 0, s>>>(D.bits, words, -1, &ctx->d_counters->inserted);
-          LGC_COUNT_LAUNCH(ctx);
-        }
         {
           ProfScope ps(ctx, LGC_PROF_EDGEMAP, alg_bytes);
           emap_red_kernel<<<grid, kBlock, 0, s>>>(g->col, share.ptr, epos.ptr, foff.ptr, nf, nrec,
-                                                   total.ptr, g->hot, D, ctx->d_counters);
-          LGC_COUNT_LAUNCH(ctx);
-        }
-        if (D.dense) {
-          bits_pop_kernel<<<pg, kBlock, 0, s>>>(D.bits, words, 1, &ctx->d_counters->inserted);
+                                                   total.ptr, g->hot, D, fmode == kFmNone ? 1 : 0,
+                                                   ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
         LGC_CUDA_TRY(cudaGetLastError());
       }
       if (fmode != kFmNone) {  // the qualifying keys in ascending id, with their degrees
         const int64_t words = (g->n + 31) / 32;
-        LGC_TRY(words_compact(ctx, DenseQualWord{D, g->deg, g->n, lite_thr(c), fmode}, nullptr, words,
+        LGC_TRY(words_compact(ctx, DenseQualWord{D, g->deg, g->n, lite_thr(c), fmode,
+                                                 &ctx->d_counters->inserted}, nullptr, words,
                               FrontierOut{g->deg, G.v.ptr, G.s.ptr, ncap, ctx->d_counters}));
       }
       int st = read_counters(out);

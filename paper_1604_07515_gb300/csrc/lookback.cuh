@@ -89,19 +89,28 @@ template <class WordFn>
 __global__ void __launch_bounds__(kBlock)
     words_count_kernel(WordFn word, int64_t words, uint32_t* __restrict__ kept,
                        int32_t* __restrict__ cnt) {
-  __shared__ int s_tot[kBlock / 32];
+  __shared__ int s_tot[kBlock / 32], s_new[kBlock / 32];
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int64_t w = (int64_t)blockIdx.x * kCmpTileWords + warp * kCmpWarpWords + lane;
   const bool in = lane < kCmpWarpWords && w < words;
-  const uint32_t q = word(w, in);
+  int fresh = 0;  // keys the functor found and marked
+  const uint32_t q = word(w, in, &fresh);
   if (kept && in) kept[w] = q;
   const int c = __reduce_add_sync(0xffffffffu, __popc(q));
-  if (lane == 0) s_tot[warp] = c;
+  fresh = __reduce_add_sync(0xffffffffu, fresh);
+  if (lane == 0) {
+    s_tot[warp] = c;
+    s_new[warp] = fresh;
+  }
   __syncthreads();
   if (threadIdx.x == 0) {
-    int t = 0;
-    for (int k = 0; k < kBlock / 32; k++) t += s_tot[k];
+    int t = 0, f = 0;
+    for (int k = 0; k < kBlock / 32; k++) {
+      t += s_tot[k];
+      f += s_new[k];
+    }
     cnt[blockIdx.x] = t;
+    if (f) word.marked(f);
   }
 }
 

@@ -708,7 +708,8 @@ int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt) {
 namespace {
 struct BitsWord {
   const uint32_t* bits;
-  __device__ uint32_t operator()(int64_t w, bool in) const { return in ? bits[w] : 0u; }
+  __device__ uint32_t operator()(int64_t w, bool in, int*) const { return in ? bits[w] : 0u; }
+  __device__ void marked(int) const {}
 };
 }  // namespace
 

@@ -238,33 +238,24 @@ struct RdEdges {
 // Every warp takes 32 * IT consecutive edges at a time and calls
 // fn(e0, src, at) with each lane's IT edges e0 + 32 k + lane, their pushing
 // entries src[k] (-1 past the end) and their places at[k] in the adjacency.
-// The first edge's entry comes from the tile array; from there on the
-// entries that start within the next 32 edges are one load and one
-// OR-reduction away.
+// The first edge's entry comes from the tile array, the others from a window
+// of the entries that follow it (edges.cuh).
 template <int IT, class Fn>
 __device__ inline void rd_edges_of(const RdEdges& R, int64_t warp, int64_t nwarps, Fn&& fn) {
   const int lane = threadIdx.x & 31;
   for (int64_t e0 = warp * 32 * IT; e0 < R.E; e0 += nwarps * 32 * IT) {
-    int64_t j = R.tile[e0 / 32];
-    int64_t bj = R.base[j];
+    EdgeWindow W(
+        R.tile[e0 / 32], R.np, [&](int64_t i) { return (int64_t)R.e[i]; },
+        [&](int64_t i) { return R.base[i]; });
     int32_t src[IT];
     int64_t at[IT];
 #pragma unroll
     for (int k = 0; k < IT; k++) {
-      const uint32_t eb = (uint32_t)(e0 + 32 * k);
-      const bool in = j + 1 + lane < R.np;
-      const uint32_t st = in ? R.e[j + 1 + lane] : 0xFFFFFFFFu;
-      const int64_t bw = in ? R.base[j + 1 + lane] : 0;
-      const uint32_t rel = st - eb;  // 0xFFFFFFFF - eb >= 32: edges stay below 2^31
-      const unsigned m = __reduce_or_sync(0xffffffffu, rel < 32u ? 1u << rel : 0u);
-      const int i = __popc(m & (0xffffffffu >> (31 - lane)));  // entries past j
-      const int64_t bs = __shfl_sync(0xffffffffu, bw, max(i - 1, 0));
-      src[k] = e0 + 32 * k + lane < R.E ? (int32_t)(j + i) : -1;
-      at[k] = (i ? bs : bj) + e0 + 32 * k + lane;
-      const int all = __popc(m);
-      const int64_t bl = __shfl_sync(0xffffffffu, bw, max(all - 1, 0));
-      bj = all ? bl : bj;
-      j += all;
+      const int64_t eb = e0 + 32 * k;
+      int64_t b = 0;
+      const int64_t i = W.find(eb, &b);
+      src[k] = eb + lane < R.E ? (int32_t)i : -1;
+      at[k] = b + eb + lane;
     }
     fn(e0, src, at);
   }
@@ -287,8 +278,9 @@ constexpr int64_t kRdHotMin = 2048;
 // Atomic push of IT edges a lane: all columns, first probes, slots, adds and
 // crossings of a lane's edges side by side.
 template <int IT>
-__device__ inline void rd_push(const RdBuf& B, const RdDest& D, const HotSet& H, bool hot,
-                               HotSum& S, const int32_t* __restrict__ col,
+__device__ inline void rd_push(const RdBuf& B, const RdDest& D, const HotSet& H,
+                               const HotShared& M, bool hot, HotLane<double>& S,
+                               const int32_t* __restrict__ col,
                                const int32_t* __restrict__ deg, const RdEdges& R,
                                const RdFront& N, RdCnt* Cc, RdCnt* C, int64_t warp,
                                int64_t nwarps, int64_t* nins) {
@@ -307,7 +299,7 @@ __device__ inline void rd_push(const RdBuf& B, const RdDest& D, const HotSet& H,
         sh[k] = B.share[src[k]];
       }
     }
-    if (hot) hot_take(H, S, w, sh);
+    if (hot) hot_take(H, M, S, w, sh);
 #pragma unroll
     for (int k = 0; k < IT; k++) {
       probe[k] = 0;
@@ -356,10 +348,10 @@ __device__ inline void rd_push(const RdBuf& B, const RdDest& D, const HotSet& H,
 
 // The hot vertices' sums after a push, each as one add.
 __device__ inline void rd_push_hot(const RdBuf& B, const RdDest& D, const HotSet& H,
-                                   const HotSum& S, const int32_t* __restrict__ deg,
+                                   const HotLane<double>& S, const int32_t* __restrict__ deg,
                                    const RdFront& N, RdCnt* Cc, RdCnt* C, int64_t* nins) {
-  hot_flush<kRdWarps>(S, [&](int h, double sh) {
-    const int32_t w = H.v[h];
+  const auto join = [](double& a, double x) { a = a + x; };
+  hot_flush<kRdWarps>(H, S, join, [&](int32_t w, double sh) {
     int ins = 0;
     const int64_t s = tb_find_or_insert(D.T, w, &ins, &Cc->err);
     if (s < 0) return;
@@ -375,11 +367,6 @@ __device__ inline void rd_push_hot(const RdBuf& B, const RdDest& D, const HotSet
 // Wide push: every edge's share added to its destination's fixed-point sum;
 // a destination's first edge lists it.  Hot destinations are summed apart, as
 // in rd_push.
-struct RdHotFx {
-  Fx a[kHot] = {};
-  unsigned any = 0;
-};
-
 __device__ inline unsigned long long rd_fx_add(Fx* acc, const Fx& x) {
   unsigned long long old = 0;
   if (x.lo) old = atomicAdd((unsigned long long*)&acc->lo, (unsigned long long)x.lo);
@@ -389,8 +376,9 @@ __device__ inline unsigned long long rd_fx_add(Fx* acc, const Fx& x) {
 }
 
 template <int IT>
-__device__ inline void rd_push_exact(const RdBuf& B, const RdDest& D, const HotSet& H, bool hot,
-                                     RdHotFx& S, const int32_t* __restrict__ col,
+__device__ inline void rd_push_exact(const RdBuf& B, const RdDest& D, const HotSet& H,
+                                     const HotShared& M, bool hot, HotLane<Fx>& S,
+                                     const int32_t* __restrict__ col,
                                      const RdEdges& R, int L, RdCnt* C, int64_t warp,
                                      int64_t nwarps, int64_t* nins) {
   rd_edges_of<IT>(R, warp, nwarps, [&](int64_t, const int32_t* src, const int64_t* at) {
@@ -406,20 +394,13 @@ __device__ inline void rd_push_exact(const RdBuf& B, const RdDest& D, const HotS
         x[k] = fx_from_bits(fx_bits(B.share[src[k]]), L);
       }
     }
-    if (hot) {
-#pragma unroll
-      for (int k = 0; k < IT; k++) {
-        bool hit = false;
-#pragma unroll
-        for (int h = 0; h < kHot; h++)
-          if (w[k] == H.v[h]) {
-            fx_add(S.a[h], x[k]);
-            S.any |= 1u << h;
-            hit = true;
-          }
-        if (hit) w[k] = -1;
-      }
-    }
+    if (hot)
+      hot_take(
+          H, M, S, w, x,
+          [](const Fx& y, int l) {
+            return Fx{__shfl_sync(0xffffffffu, y.lo, l), __shfl_sync(0xffffffffu, y.hi, l)};
+          },
+          [](Fx& a, const Fx& y) { fx_add(a, y); });
 #pragma unroll
     for (int k = 0; k < IT; k++) {
       slot[k] = -1;
@@ -452,41 +433,18 @@ __device__ inline void rd_push_exact(const RdBuf& B, const RdDest& D, const HotS
 }
 
 __device__ inline void rd_push_exact_hot(const RdBuf& B, const RdDest& D, const HotSet& H,
-                                         const RdHotFx& S, RdCnt* C, int64_t* nins) {
-  __shared__ Fx s_fx[kRdWarps][kHot];
-  __shared__ unsigned s_met;
-  if (!__syncthreads_or(S.any != 0)) return;
-  if (threadIdx.x == 0) s_met = 0;
-  __syncthreads();
-  const int lane = threadIdx.x & 31;
-  const unsigned met = __reduce_or_sync(0xffffffffu, S.any);
-#pragma unroll
-  for (int h = 0; h < kHot; h++) {
-    Fx x = S.a[h];
-    for (int o = 16; o > 0; o >>= 1) {
-      Fx y;
-      y.lo = __shfl_xor_sync(0xffffffffu, x.lo, o);
-      y.hi = __shfl_xor_sync(0xffffffffu, x.hi, o);
-      fx_add(x, y);
-    }
-    if (lane == 0) s_fx[threadIdx.x >> 5][h] = x;
-  }
-  if (lane == 0 && met) atomicOr(&s_met, met);
-  __syncthreads();
-  if (threadIdx.x < kHot && ((s_met >> threadIdx.x) & 1u)) {
-    const int32_t w = H.v[threadIdx.x];
-    Fx x = {0, 0};
-    for (int k = 0; k < kRdWarps; k++) fx_add(x, s_fx[k][threadIdx.x]);
+                                         const HotLane<Fx>& S, RdCnt* C, int64_t* nins) {
+  const auto join = [](Fx& a, const Fx& x) { fx_add(a, x); };
+  hot_flush<kRdWarps>(H, S, join, [&](int32_t w, const Fx& x) {
     int ins = 0;
     const int64_t s = tb_find_or_insert(D.T, w, &ins, &C->err);
-    if (s >= 0) {
-      *nins += ins;
-      if (ins && D.keys) D.keys[atomicAdd(&C->nkeys, 1)] = (int32_t)s;
-      rd_fx_add(&B.xacc[s], x);
-      if (atomicAdd(&B.cnt[s], 1) == 0)
-        B.touched[atomicAdd(&C->touched, 1)] = make_int2(w, (int32_t)s);
-    }
-  }
+    if (s < 0) return;
+    *nins += ins;
+    if (ins && D.keys) D.keys[atomicAdd(&C->nkeys, 1)] = (int32_t)s;
+    rd_fx_add(&B.xacc[s], x);
+    if (atomicAdd(&B.cnt[s], 1) == 0)
+      B.touched[atomicAdd(&C->touched, 1)] = make_int2(w, (int32_t)s);
+  });
 }
 
 // After the barrier: every listed destination's sum joins its value, rounded
@@ -956,26 +914,27 @@ __device__ inline void rd_count_inserted(int64_t nins, RdCnt* C) {
 // The edge phase of an atomic round over the edges R: the push, and for a
 // wide round (exact) the barrier and the sums' settling.
 __device__ inline void rd_push_round(const RdBuf& B, const RdDest& D, const HotSet& H,
+                                     const HotShared& M,
                                      const int32_t* __restrict__ col,
                                      const int32_t* __restrict__ deg, const RdEdges& R, bool exact,
                                      int gbits, const RdFront& N, RdCnt* Cc, RdCnt* C,
                                      int64_t warp, int64_t nwarps, cg::grid_group& grid) {
   int64_t nins = 0;
   const bool wide = R.E > nwarps * 64;  // several edges a lane once every warp has work
-  const bool hot = R.np >= kRdHotMin;
+  const bool hot = H.tab && R.np >= kRdHotMin;
   if (exact) {
-    RdHotFx S;
+    HotLane<Fx> S;
     const int L = fx_scale(2047 - __ldcg(&Cc->emin), __ldcg(&Cc->emax), gbits);
-    if (wide) rd_push_exact<4>(B, D, H, hot, S, col, R, L, Cc, warp, nwarps, &nins);
-    else rd_push_exact<1>(B, D, H, hot, S, col, R, L, Cc, warp, nwarps, &nins);
+    if (wide) rd_push_exact<4>(B, D, H, M, hot, S, col, R, L, Cc, warp, nwarps, &nins);
+    else rd_push_exact<1>(B, D, H, M, hot, S, col, R, L, Cc, warp, nwarps, &nins);
     if (hot) rd_push_exact_hot(B, D, H, S, Cc, &nins);
     rd_count_inserted(nins, Cc);
     grid.sync();
     rd_settle_exact(B, D, deg, L, N, Cc, C, warp, nwarps);
   } else {
-    HotSum S;
-    if (wide) rd_push<4>(B, D, H, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
-    else rd_push<1>(B, D, H, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
+    HotLane<double> S;
+    if (wide) rd_push<4>(B, D, H, M, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
+    else rd_push<1>(B, D, H, M, hot, S, col, deg, R, N, Cc, C, warp, nwarps, &nins);
     if (hot) rd_push_hot(B, D, H, S, deg, N, Cc, C, &nins);
     rd_count_inserted(nins, Cc);
   }
@@ -984,6 +943,8 @@ __device__ inline void rd_push_round(const RdBuf& B, const RdDest& D, const HotS
 // Atomic mode.
 template <bool BETA>
 __global__ void __launch_bounds__(kRdBlock, 1) rounds_kernel(RdArgs A, RdBuf B, Table T) {
+  __shared__ HotShared s_tab;
+  hot_load(A.hot, s_tab);
   cg::grid_group grid = cg::this_grid();
   const int lane = threadIdx.x & 31;
   // consecutive warps on different SMs: a small phase spreads over the chip
@@ -1021,7 +982,7 @@ __global__ void __launch_bounds__(kRdBlock, 1) rounds_kernel(RdArgs A, RdBuf B, 
     const int64_t np = rd_size(pp), Ep = rd_edges(pp);
     const RdEdges R = {BETA ? B.pe : F.e, B.base, BETA ? B.ptile : F.tile, np, Ep};
     const RdDest D = {T, nullptr, A.eps, true};
-    rd_push_round(B, D, A.hot, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps, grid);
+    rd_push_round(B, D, A.hot, s_tab, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps, grid);
     grid.sync();
     rounds += 1;
     pushes += np;
@@ -1229,6 +1190,8 @@ template <bool DET, int KIND>
 __global__ void __launch_bounds__(kRdBlock, 1)
     rounds_fresh_kernel(RdArgs A, RfArgs X, RdBuf B, RfTabs Q) {
   extern __shared__ uint32_t s_mem[];
+  __shared__ HotShared s_tab;
+  if (!DET) hot_load(A.hot, s_tab);
   cg::grid_group grid = cg::this_grid();
   const int lane = threadIdx.x & 31;
   const int64_t warp = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
@@ -1371,7 +1334,8 @@ __global__ void __launch_bounds__(kRdBlock, 1)
               });
     } else {
       const RdDest dest = {D, Q.keys[set], c, thr};
-      rd_push_round(B, dest, A.hot, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps, grid);
+      rd_push_round(B, dest, A.hot, s_tab, A.col, A.deg, R, exact, A.gbits, N, Cc, C, warp, nwarps,
+                    grid);
     }
     grid.sync();
     rounds += 1;
