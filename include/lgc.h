@@ -234,7 +234,7 @@ void lgc_graph_destroy(lgc_graph *g);
  *    alone, from 2m/64, 2m/16, 2m/4 (each at least 2^20) and never, timing
  *    one batch of 256 seeds of the graph at each (lgc_graph_batch_handoff
  *    reports the choice).
- * Until it is called the graph uses (8, 32, 16) and max(2^20, 2m/64). */
+ * Until it is called the graph uses (8, 16, 8) and max(2^20, 2m/64). */
 int lgc_graph_autotune(lgc_graph *g, int *pull_batch, int *pull_group, int *pull_share);
 /* The hand-off threshold (edges) the graph's batches use while
  * LGC_OPT_BATCH_HANDOFF is 0: the tuned value, else max(2^20, 2m/64);

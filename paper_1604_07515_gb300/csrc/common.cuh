@@ -300,9 +300,13 @@ struct lgc_graph {
   lgc::HotSet hot;
   int2* hot_mem = nullptr;  // its table and ids
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
-  int pull_batch = 8;          // edges per lane per batch in heavy pull gathers (tuned)
-  int pull_group = 32;         // lanes per work item in heavy pull gathers (tuned)
-  int pull_share = 16;         // bytes per gathered share in atomic pull gathers (tuned)
+  // the shape of the atomic pull gathers (tuned): edges per lane per batch,
+  // lanes per work item (heavy), bytes per gathered share.  Until tuned, the
+  // best with light = 32 on a scale-22 R-MAT graph: a HK-PR call there takes
+  // 8.05 ms, 8.15 with (16, 16, 8), 8.38 with (4, 32, 8), 10.5 with (8, 32, 16).
+  int pull_batch = 8;
+  int pull_group = 16;
+  int pull_share = 8;
   int64_t batch_handoff = 0;   // batched PR-Nibble hand-off threshold (tuned; 0: untuned)
   int pull_light = 32;         // atomic pull rounds: degree <= pull_light one thread each (tuned)
   // vertices of degree > pull_light in ascending id, for the atomic pull edge phase

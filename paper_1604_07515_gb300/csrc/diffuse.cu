@@ -496,8 +496,8 @@ __global__ void pull_scatter_kernel(int64_t nf, const int32_t* __restrict__ fv,
   }
 }
 
-__device__ inline bool pull_qualifies(double acc, int64_t d, double c, int fmode) {
-  if (fmode == kFmThreshold) return lite_reaches(acc, lite_thr(c), (int32_t)d);
+__device__ inline bool pull_qualifies(double acc, int64_t d, LiteThr c, int fmode) {
+  if (fmode == kFmThreshold) return lite_reaches(acc, c, (int32_t)d);
   return fmode == kFmInserted;
 }
 
@@ -507,7 +507,7 @@ __device__ inline bool pull_qualifies(double acc, int64_t d, double c, int fmode
 // have one length.  qbits is cleared before; qualifying vertices are ORed in.
 __global__ void pull_light_kernel(const LightItem* __restrict__ items, int64_t nl,
                                   const int32_t* __restrict__ col,
-                                  const double* __restrict__ sh, Table D, double c, int fmode,
+                                  const double* __restrict__ sh, Table D, LiteThr c, int fmode,
                                   uint32_t* __restrict__ qbits, Counters* C) {
   int64_t nins = 0;  // keys inserted here, counted once per block
   for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nl;
@@ -543,7 +543,7 @@ constexpr int kPullBatch = 8;
 // Writes a heavy vertex's gathered value (lane 0 calls it); 1 if the vertex
 // became a key here (the caller counts it).
 __device__ inline int pull_finish(const Table& D, int32_t w, int64_t d, double acc, bool touched,
-                                  bool present, double c, int fmode, uint32_t* qbits) {
+                                  bool present, LiteThr c, int fmode, uint32_t* qbits) {
   if (!touched) return 0;
   const uint32_t m = 1u << (w & 31);
   D.dval[w] = acc;
@@ -561,7 +561,7 @@ __device__ inline int pull_finish(const Table& D, int32_t w, int64_t d, double a
 __global__ void __launch_bounds__(kBlock)
     pull_mid_det_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                         const int32_t* __restrict__ mid, int64_t nmid,
-                        const double* __restrict__ sh, Table D, double c, int fmode,
+                        const double* __restrict__ sh, Table D, LiteThr c, int fmode,
                         uint32_t* __restrict__ qbits, Counters* C) {
   int64_t nins = 0;  // keys inserted here, counted once per block
   for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nmid;
@@ -713,7 +713,7 @@ __global__ void __launch_bounds__(kBlock)
                           const int64_t* __restrict__ seg0, int64_t nbig,
                           const double* __restrict__ sh, const int32_t* __restrict__ pred,
                           const FoldStep* __restrict__ step, const int32_t* __restrict__ segany,
-                          Table D, double c, int fmode, uint32_t* __restrict__ qbits,
+                          Table D, LiteThr c, int fmode, uint32_t* __restrict__ qbits,
                           Counters* C) {
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -920,27 +920,63 @@ __global__ void tune_fill_kernel(SH* __restrict__ shx, int64_t n, int32_t* __res
   }
 }
 
+// A gathered list's sum: W >= 1, 8-byte shares in W windows (FxWindow); W = 0,
+// 16-byte records or 8-byte shares over any range, in 128 bits term by term.
+template <int W, typename SH>
+struct PullSum {
+  FxWindow<W> win;
+  uint32_t any = 0;
+  __device__ void add(double s, int, uint32_t be0) {
+    const uint64_t b = fx_bits(s);
+    any |= (uint32_t)b | (uint32_t)(b >> 32);
+    win.add(b, be0);
+  }
+  __device__ Fx total() const { return win.total(); }
+  __device__ bool member() const { return any != 0; }
+};
+template <typename SH>
+struct PullSum<0, SH> {
+  Fx acc = {0, 0};
+  uint64_t flag = 0;
+  __device__ void add(const SH& s, int L, uint32_t) {
+    const Fx x = to_fx(s, L);
+    flag |= x.hi;
+    fx_add(acc, x);
+  }
+  __device__ Fx total() const { return acc; }
+  __device__ bool member() const { return (flag & kFxFlag) != 0; }
+};
+
+// Calls body<W>() for the windows the round's shares need (the same in every
+// thread of the grid).
+template <typename SH, class Body>
+__device__ inline void pull_windows(const int32_t* range, int L, Body&& body) {
+  if constexpr (sizeof(SH) == 8) {
+    const int w = fx_windows(2047 - range[0], range[1], L);
+    if (w == 1) return body(std::integral_constant<int, 1>());
+    if (w == 2) return body(std::integral_constant<int, 2>());
+  }
+  body(std::integral_constant<int, 0>());
+}
+
 // Vertices of degree 1..kPullLight, one thread each, taken from the graph's
 // list grouped by degree so that the threads of a warp walk lists of one
 // length (in id order most of a warp idled behind its longest list); the
 // edges are read four at a time (all column loads, then all share loads).
 // The bitmap qbits is cleared before this launch; this kernel and the heavy
 // one OR their qualifying vertices in.
-template <typename SH>
-__device__ inline void pull_light_fx_body(int64_t bid, int64_t nblk,
-                                          const LightItem* __restrict__ items, int64_t nl,
-                                          const int32_t* __restrict__ col,
-                                          const SH* __restrict__ shx,
-                                          const int32_t* __restrict__ range, int g, Table D,
-                                          double c, int fmode, uint32_t* __restrict__ qbits,
-                                          Counters* C) {
-  const int L = round_scale(range, g);
+template <int W, typename SH>
+__device__ inline int64_t pull_light_fx_body(const LightItem* __restrict__ items, int64_t nl,
+                                             const int32_t* __restrict__ col,
+                                             const SH* __restrict__ shx, uint32_t be0, int L,
+                                             const Table& D, LiteThr c, int fmode,
+                                             uint32_t* __restrict__ qbits) {
   int64_t nins = 0;  // keys inserted here, counted once per block
-  for (int64_t i = bid * blockDim.x + threadIdx.x; i < nl; i += nblk * blockDim.x) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nl;
+       i += (int64_t)gridDim.x * blockDim.x) {
     const LightItem it = items[i];
     const int32_t w = it.w, d = it.d;
-    Fx acc = {0, 0};
-    uint64_t flag = 0;
+    PullSum<W, SH> sum;
     for (int k = 0; k < d; k += 4) {
       int32_t u[4];
 #pragma unroll
@@ -949,22 +985,18 @@ __device__ inline void pull_light_fx_body(int64_t bid, int64_t nblk,
 #pragma unroll
       for (int j = 0; j < 4; j++) raw[j] = u[j] >= 0 ? shx[u[j]] : no_share<SH>();
 #pragma unroll
-      for (int j = 0; j < 4; j++) {
-        const Fx x = to_fx(raw[j], L);
-        flag |= x.hi;
-        fx_add(acc, x);
-      }
+      for (int j = 0; j < 4; j++) sum.add(raw[j], L, be0);
     }
     const uint32_t m = 1u << (w & 31);
     const bool present = (D.bits[w >> 5] & m) != 0;
-    if (present || (flag & kFxFlag)) {
-      const double v = (present ? D.dval[w] : 0.0) + fx_to_double(acc, L);
+    if (present || sum.member()) {
+      const double v = (present ? D.dval[w] : 0.0) + fx_to_double(sum.total(), L);
       D.dval[w] = v;
       if (!present && !(atomicOr(&D.bits[w >> 5], m) & m)) nins++;
       if (pull_qualifies(v, d, c, fmode)) atomicOr(&qbits[w >> 5], m);
     }
   }
-  flush_count(nins, &C->inserted);
+  return nins;
 }
 
 // Heavy vertices: one warp per work item (at most kPullItem edges of one
@@ -980,22 +1012,20 @@ __device__ inline void pull_light_fx_body(int64_t bid, int64_t nblk,
 // consecutive items.  The loop over items runs the same number of times in
 // every lane of the warp (a group past the end works on nothing), so the
 // group-wide shuffles always find all their lanes.
-template <int BATCH, int GL, typename SH>
-__device__ inline void pull_heavy_fx_body(int64_t bid, int64_t nblk,
-                                          const int64_t* __restrict__ off,
-                                          const int32_t* __restrict__ col,
-                                          const PullItem* __restrict__ items, int64_t nitems,
-                                          const SH* __restrict__ shx,
-                                          const int32_t* __restrict__ range, int g, Table D,
-                                          double c, int fmode, uint32_t* __restrict__ qbits,
-                                          Fx* __restrict__ hacc, int32_t* __restrict__ hcnt,
-                                          int32_t* __restrict__ htouch, Counters* C) {
+template <int W, int BATCH, int GL, typename SH>
+__device__ inline int64_t pull_heavy_fx_body(const int64_t* __restrict__ off,
+                                             const int32_t* __restrict__ col,
+                                             const PullItem* __restrict__ items, int64_t nitems,
+                                             const SH* __restrict__ shx, uint32_t be0, int L,
+                                             const Table& D, LiteThr c, int fmode,
+                                             uint32_t* __restrict__ qbits, Fx* __restrict__ hacc,
+                                             int32_t* __restrict__ hcnt,
+                                             int32_t* __restrict__ htouch) {
   constexpr int kGroups = 32 / GL;
-  const int L = round_scale(range, g);
   int64_t nins = 0;  // vertices that became keys here
   const int lane = threadIdx.x & 31, gl = lane % GL, gid = lane / GL;
-  const int64_t warp0 = (bid * blockDim.x + threadIdx.x) >> 5;
-  const int64_t nwarps = (nblk * blockDim.x) >> 5;
+  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t base = warp0 * kGroups; base < nitems; base += nwarps * kGroups) {
     const int64_t it = base + gid;
     const bool valid = it < nitems;
@@ -1019,8 +1049,7 @@ __device__ inline void pull_heavy_fx_body(int64_t bid, int64_t nblk,
       cur = D.dval[w];
       d = off[w + 1] - off[w];
     }
-    Fx part = {0, 0};
-    uint64_t flag = 0;
+    PullSum<W, SH> sum;
     for (int k0 = 0; k0 < I.len; k0 += GL * BATCH) {
       int32_t u[BATCH];
 #pragma unroll
@@ -1032,13 +1061,10 @@ __device__ inline void pull_heavy_fx_body(int64_t bid, int64_t nblk,
 #pragma unroll
       for (int j = 0; j < BATCH; j++) raw[j] = u[j] >= 0 ? shx[u[j]] : no_share<SH>();
 #pragma unroll
-      for (int j = 0; j < BATCH; j++) {
-        const Fx x = to_fx(raw[j], L);
-        flag |= x.hi;
-        fx_add(part, x);
-      }
+      for (int j = 0; j < BATCH; j++) sum.add(raw[j], L, be0);
     }
-    uint32_t mem = (flag & kFxFlag) ? 1u : 0u;
+    Fx part = sum.total();
+    uint32_t mem = sum.member() ? 1u : 0u;
     for (int o = GL / 2; o > 0; o >>= 1) {  // within the group
       Fx t;
       t.lo = __shfl_xor_sync(0xffffffffu, part.lo, o);
@@ -1057,6 +1083,7 @@ __device__ inline void pull_heavy_fx_body(int64_t bid, int64_t nblk,
     }
     const int32_t h = I.h;
     unsigned long long* acc = reinterpret_cast<unsigned long long*>(&hacc[h]);
+    part.hi &= kFxMask;
     if (part.lo | part.hi) {
       const unsigned long long old = atomicAdd(&acc[0], (unsigned long long)part.lo);
       const unsigned long long carry = old + part.lo < old ? 1ull : 0ull;
@@ -1078,7 +1105,7 @@ __device__ inline void pull_heavy_fx_body(int64_t bid, int64_t nblk,
       htouch[h] = 0;
     }
   }
-  flush_count(nins, &C->inserted);
+  return nins;
 }
 
 template <int BATCH, int GL, typename SH>
@@ -1086,21 +1113,37 @@ __global__ void __launch_bounds__(kBlock)
     pull_heavy_fx_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                          const PullItem* __restrict__ items, int64_t nitems,
                          const SH* __restrict__ shx, const int32_t* __restrict__ range, int g,
-                         Table D, double c, int fmode, uint32_t* __restrict__ qbits,
+                         Table D, LiteThr c, int fmode, uint32_t* __restrict__ qbits,
                          Fx* __restrict__ hacc, int32_t* __restrict__ hcnt,
                          int32_t* __restrict__ htouch, Counters* C) {
-  pull_heavy_fx_body<BATCH, GL, SH>(blockIdx.x, gridDim.x, off, col, items, nitems, shx, range, g,
-                                    D, c, fmode, qbits, hacc, hcnt, htouch, C);
+  const int L = round_scale(range, g);
+  const uint32_t be0 = (uint32_t)(2047 - range[0]);
+  int64_t nins = 0;
+  pull_windows<SH>(range, L, [&](auto w) {
+    constexpr int W = decltype(w)::value;
+    // shares over any range are rare: a short batch keeps the registers of the
+    // others
+    constexpr int B = W == 0 && sizeof(SH) == 8 ? 4 : BATCH;
+    nins = pull_heavy_fx_body<W, B, GL, SH>(off, col, items, nitems, shx, be0, L, D, c, fmode,
+                                            qbits, hacc, hcnt, htouch);
+  });
+  flush_count(nins, &C->inserted);
 }
 
 template <typename SH>
 __global__ void pull_light_fx_kernel(const LightItem* __restrict__ items, int64_t nl,
                                      const int32_t* __restrict__ col,
                                      const SH* __restrict__ shx,
-                                     const int32_t* __restrict__ range, int g, Table D, double c,
+                                     const int32_t* __restrict__ range, int g, Table D, LiteThr c,
                                      int fmode, uint32_t* __restrict__ qbits, Counters* C) {
-  pull_light_fx_body<SH>(blockIdx.x, gridDim.x, items, nl, col, shx, range, g, D, c, fmode,
-                         qbits, C);
+  const int L = round_scale(range, g);
+  const uint32_t be0 = (uint32_t)(2047 - range[0]);
+  int64_t nins = 0;
+  pull_windows<SH>(range, L, [&](auto w) {
+    nins = pull_light_fx_body<decltype(w)::value, SH>(items, nl, col, shx, be0, L, D, c, fmode,
+                                                      qbits);
+  });
+  flush_count(nins, &C->inserted);
 }
 
 // ---------------------------------------------------------------------------
@@ -1407,7 +1450,7 @@ __global__ void uniq_write_kernel(const uint32_t* __restrict__ kv, const int32_t
 
 template <typename SH>
 using HeavyKernel = void (*)(const int64_t*, const int32_t*, const PullItem*, int64_t, const SH*,
-                             const int32_t*, int, Table, double, int, uint32_t*, Fx*, int32_t*,
+                             const int32_t*, int, Table, LiteThr, int, uint32_t*, Fx*, int32_t*,
                              int32_t*, Counters*);
 
 // The heavy-vertex gather compiled for a (batch depth, lanes per item) shape.
@@ -1730,6 +1773,7 @@ struct PushWork {
     const int64_t n = g->n, words = (n + 31) / 32, nf = F.size;
     LGC_TRY(pull_reserve(det));
     const int sb = pull_share_bytes(det);
+    const LiteThr ct = lite_thr(c);
     const int32_t ncap = (int32_t)G.v.cap;
     // sums of at most max_deg terms: max_deg < 2^gb
     int gb = 1;
@@ -1761,13 +1805,13 @@ struct PushWork {
           const int lgl =
               (int)std::min<int64_t>(ceil_div(g->nlight_det, kBlock), (ctx->sms * 32));
           pull_light_kernel<<<lgl, kBlock, 0, s>>>(g->light_det, g->nlight_det, g->col, psh.ptr,
-                                                   D, c, fmode, pq.ptr, ctx->d_counters);
+                                                   D, ct, fmode, pq.ptr, ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
         if (g->ndet_mid > 0) {
           const int mg = (int)std::min<int64_t>(ceil_div(g->ndet_mid, kBlock), (ctx->sms * 32));
           pull_mid_det_kernel<<<mg, kBlock, 0, s>>>(g->off, g->col, g->det_mid, g->ndet_mid,
-                                                    psh.ptr, D, c, fmode, pq.ptr,
+                                                    psh.ptr, D, ct, fmode, pq.ptr,
                                                     ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
@@ -1789,7 +1833,7 @@ struct PushWork {
           const int vg = (int)std::min<int64_t>(ceil_div(g->nbig, kBlock / 32), (ctx->sms * 16));
           det_seg_verify_kernel<<<vg, kBlock, 0, s>>>(g->off, g->col, g->segs, g->big_w,
                                                       g->big_seg0, g->nbig, psh.ptr, dpred.ptr,
-                                                      dstep.ptr, dany.ptr, D, c, fmode, pq.ptr,
+                                                      dstep.ptr, dany.ptr, D, ct, fmode, pq.ptr,
                                                       ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
@@ -1801,7 +1845,7 @@ struct PushWork {
           if (g->nlight > 0) {
             const int lgl = (int)std::min<int64_t>(ceil_div(g->nlight, kBlock), (ctx->sms * 32));
             pull_light_fx_kernel<SH><<<lgl, kBlock, 0, s>>>(g->light, g->nlight, g->col, shv,
-                                                             prange.ptr, gb, D, c, fmode, pq.ptr,
+                                                             prange.ptr, gb, D, ct, fmode, pq.ptr,
                                                              ctx->d_counters);
             LGC_COUNT_LAUNCH(ctx);
           }
@@ -1812,7 +1856,7 @@ struct PushWork {
             const int batch = ctx->pull_batch ? ctx->pull_batch : g->pull_batch;
             HeavyKernel<SH> heavy = heavy_kernel<SH>(batch, gw);
             heavy<<<hg, kBlock, 0, s>>>(g->off, g->col, g->items, g->nitems, shv, prange.ptr, gb,
-                                        D, c, fmode, pq.ptr, phacc.ptr, phcnt.ptr, phtouch.ptr,
+                                        D, ct, fmode, pq.ptr, phacc.ptr, phcnt.ptr, phtouch.ptr,
                                         ctx->d_counters);
             LGC_COUNT_LAUNCH(ctx);
           }
@@ -2151,7 +2195,7 @@ int autotune_pull(lgc_ctx* ctx, lgc_graph* g) {
     const int cand[7][2] = {{4, 32}, {8, 32}, {16, 32}, {8, 16}, {16, 16}, {8, 8}, {16, 8}};
     const int lights[4] = {32, 64, 128, 256};
     float best_ms = 0.f;
-    int best = kPullBatch, best_group = 32, best_share = 16, best_light = g->pull_light;
+    int best = g->pull_batch, best_group = g->pull_group, best_share = g->pull_share, best_light = g->pull_light;
     bool first = true;
     for (int li = 0; li < 4 && st == LGC_OK; li++) {
       if (g->pull_light != lights[li] && (st = rebuild_pull_lists(ctx, g, lights[li])) != LGC_OK)
@@ -2180,8 +2224,8 @@ int autotune_pull(lgc_ctx* ctx, lgc_graph* g) {
               1, std::min<int64_t>(ceil_div(g->nlight, kBlock), (ctx->sms * 32)));
           timed([&] {
             pull_light_fx_kernel<SH><<<lgl, kBlock, 0, s>>>(g->light, g->nlight, g->col, shv,
-                                                           range, gb, D, 1.0, kFmThreshold, q,
-                                                           ctx->d_counters);
+                                                           range, gb, D, lite_thr(1.0),
+                                                           kFmThreshold, q, ctx->d_counters);
           }, &light_ms);
         };
         if (g->nlight > 0) {
@@ -2204,7 +2248,7 @@ int autotune_pull(lgc_ctx* ctx, lgc_graph* g) {
             const int hg = (int)(hb < (ctx->sms * 16) ? hb : (ctx->sms * 16));
             timed([&] {
               heavy<<<hg, kBlock, 0, s>>>(g->off, g->col, g->items, g->nitems, shv, range, gb, D,
-                                          1.0, kFmThreshold, q, hacc, hcnt, htouch,
+                                          lite_thr(1.0), kFmThreshold, q, hacc, hcnt, htouch,
                                           ctx->d_counters);
             }, &med);
           };

@@ -162,6 +162,69 @@ LGC_HD void fx_add(Fx& a, const Fx& b) {
   a.lo = lo;
 }
 
+// Sums of shares whose biased exponents lie in [be0, be0 + 32 W), W = 1 or 2,
+// in units of 2^fx_lsb(be0), with a third of the instructions of converting
+// each to 128 bits and adding it with carries: the significand is cut into 18,
+// 18 and 17 bits, each multiplied by 2^(be - be0) and added to a 64-bit sum of
+// its own by one multiply-add (a product stays below 2^49, so 2^14 terms fit).
+// With W = 2 a share goes to one of two sets of sums, 32 bits apart.  Terms:
+// the bits of a double that is +0.0 or -0.0 (they add nothing) or positive and
+// normal in the range; 1 <= be0 <= 1984.
+LGC_HD uint32_t fx_shl32(uint32_t x, uint32_t s) {
+#if defined(__CUDA_ARCH__)
+  uint32_t r;
+  asm("shl.b32 %0, %1, %2;" : "=r"(r) : "r"(x), "r"(s));  // 0 from 32 on
+  return r;
+#else
+  return s >= 32 ? 0 : x << s;
+#endif
+}
+
+template <int W>
+struct FxWindow {
+  uint64_t a[3 * W] = {};
+
+  LGC_HD void add(uint64_t bits, uint32_t be0) {
+    const uint32_t lo = (uint32_t)bits, hi = (uint32_t)(bits >> 32);
+    const uint32_t m0 = lo & 0x3FFFFu;
+    const uint32_t m1 = (uint32_t)(bits >> 18) & 0x3FFFFu;
+    const uint32_t m2 = (hi >> 4 & 0xFFFFu) | 0x10000u;
+    // +0.0 is below every range (be 0), -0.0 above (be 2048)
+    const uint32_t sh = (hi >> 20) - be0;
+    const uint32_t p = fx_shl32(1u, sh);
+    a[0] += (uint64_t)m0 * p;
+    a[1] += (uint64_t)m1 * p;
+    a[2] += (uint64_t)m2 * p;
+    if (W == 2) {
+      const uint32_t q = fx_shl32(1u, sh - 32u);
+      a[3 * W - 3] += (uint64_t)m0 * q;
+      a[3 * W - 2] += (uint64_t)m1 * q;
+      a[3 * W - 1] += (uint64_t)m2 * q;
+    }
+  }
+
+  LGC_HD static void join(Fx& t, uint64_t x, int s) {
+    Fx y;
+    y.lo = s >= 64 ? 0 : x << s;
+    y.hi = s >= 64 ? x << (s - 64) : s ? x >> (64 - s) : 0;
+    const uint64_t lo = t.lo + y.lo;
+    t.hi += y.hi + (lo < y.lo ? 1ull : 0ull);
+    t.lo = lo;
+  }
+  LGC_HD Fx total() const {
+    Fx t = {0, 0};
+    for (int k = 0; k < 3 * W; k++) join(t, a[k], 18 * (k % 3) + 32 * (k / 3));
+    return t;
+  }
+};
+
+// The windows that take a round's shares: 1 or 2, or 0 where they span more,
+// a share is subnormal, or the scale L leaves bits of the smallest out.
+LGC_HD int fx_windows(int be_min, int be_max, int L) {
+  if (be_min > be_max || be_min < 1 || be_min > 1984 || L != fx_lsb(be_min)) return 0;
+  return be_max - be_min < 32 ? 1 : be_max - be_min < 64 ? 2 : 0;
+}
+
 // RN(X * 2^L) as a double, X < 2^127 (the flag bit is ignored).
 LGC_HD double fx_to_double(Fx X, int L) {
   const uint64_t hi = X.hi & kFxMask, lo = X.lo;
