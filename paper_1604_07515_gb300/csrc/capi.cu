@@ -117,25 +117,11 @@ __global__ void gather_off_kernel(const int32_t* __restrict__ ids, int64_t k,
     out[i] = off[ids[i]];
 }
 
-// The deterministic pull's vertices of degree (kPullLight, kDetBig], and those
-// of degree > kDetBig with their 256-edge segments (built on the host from the
-// degree copy; only their list starts are read back).
+// The deterministic pull's vertices of degree > kDetBig with their 256-edge
+// segments (built on the host from the degree copy; only their list starts are
+// read back).
 int build_big_segments(lgc_ctx* ctx, lgc_graph* g) {
   cudaStream_t s = ctx->stream;
-  {
-    std::vector<int32_t> mid;
-    for (int64_t v = 0; v < g->n; v++)
-      if (g->hdeg[v] > kPullLight && g->hdeg[v] <= kDetBig) mid.push_back((int32_t)v);
-    std::stable_sort(mid.begin(), mid.end(),
-                     [&](int32_t a, int32_t b) { return g->hdeg[a] > g->hdeg[b]; });
-    g->ndet_mid = (int64_t)mid.size();
-    if (g->ndet_mid > 0) {
-      LGC_TRY(dalloc_t(ctx, &g->det_mid, g->ndet_mid));
-      LGC_CUDA_TRY(cudaMemcpyAsync(g->det_mid, mid.data(), 4 * g->ndet_mid,
-                                   cudaMemcpyHostToDevice, s));
-      LGC_CUDA_TRY(cudaStreamSynchronize(s));  // mid goes out of scope
-    }
-  }
   std::vector<int32_t> bw;
   for (int64_t v = 0; v < g->n; v++)
     if (g->hdeg[v] > kDetBig) bw.push_back((int32_t)v);
@@ -186,58 +172,100 @@ __global__ void light_items_kernel(const int32_t* __restrict__ order, int64_t k,
   }
 }
 
-// The vertices of degree 1..L grouped by degree, highest first, ids
-// ascending within a degree (a counting sort of the host degree copy), into
-// *out (*nout entries).
-int build_light_list(lgc_ctx* ctx, lgc_graph* g, int L, LightItem** out, int64_t* nout) {
+// The columns of entries 32 k .. 32 k + 31 side by side (LightView), a warp
+// each.
+__global__ void slice_fill_kernel(const LightItem* __restrict__ items, int64_t k,
+                                  const int64_t* __restrict__ slice,
+                                  const int32_t* __restrict__ col, int32_t* __restrict__ out) {
+  const int lane = threadIdx.x & 31;
+  const int64_t nslices = (k + 31) / 32;
+  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t q = warp0; q < nslices; q += nwarps) {
+    const int64_t i = 32 * q + lane;
+    const LightItem it = i < k ? items[i] : LightItem{0, 0, 0};
+    const int64_t base = slice[q];
+    const int len = (int)((slice[q + 1] - base) / 32);
+    for (int e = 0; e < len; e++) out[base + 32 * e + lane] = e < it.d ? col[it.beg + e] : -1;
+  }
+}
+
+// The interleaved columns of the short lists, unless they would take more than
+// an eighth of the free device memory.
+int build_slices(lgc_ctx* ctx, lgc_graph* g) {
+  const int64_t k = g->short_at[0], nslices = (k + 31) / 32;
+  if (k == 0) return LGC_OK;
+  cudaStream_t s = ctx->stream;
+  std::vector<int64_t> at;
+  try {
+    at.resize(nslices + 1);
+  } catch (...) {
+    return LGC_ENOMEM;
+  }
+  int d = kDetBig;  // a slice is as long as its first entry's list
+  at[0] = 0;
+  for (int64_t q = 0; q < nslices; q++) {
+    while (g->short_at[d - 1] <= 32 * q) d--;
+    at[q + 1] = at[q] + 32 * (int64_t)d;
+  }
+  const size_t bytes = 4 * (size_t)at[nslices] + 8 * (size_t)(nslices + 1);
+  size_t avail = 0, all = 0;
+  LGC_CUDA_TRY(cudaMemGetInfo(&avail, &all));
+  if (bytes > avail / 8) return LGC_OK;
+  LGC_TRY(dalloc_t(ctx, &g->slice_at, nslices + 1));
+  LGC_TRY(dalloc_t(ctx, &g->slice_col, at[nslices]));
+  LGC_CUDA_TRY(cudaMemcpyAsync(g->slice_at, at.data(), 8 * (nslices + 1), cudaMemcpyHostToDevice,
+                               s));
+  slice_fill_kernel<<<std::min(grid_for(k), ctx->sms * 16), kBlock, 0, s>>>(
+      g->shorts, k, g->slice_at, g->col, g->slice_col);
+  LGC_COUNT_LAUNCH(ctx);
+  LGC_CUDA_TRY(cudaGetLastError());
+  LGC_CUDA_TRY(cudaStreamSynchronize(s));  // at goes out of scope
+  return LGC_OK;
+}
+
+// The vertices of degree 1..kDetBig grouped by degree, highest first, ids
+// ascending within a degree (a counting sort of the host degree copy), with
+// their columns interleaved.
+int build_shorts(lgc_ctx* ctx, lgc_graph* g) {
   cudaStream_t s = ctx->stream;
   const int64_t n = g->n;
-  std::vector<int64_t> cnt(L + 2, 0), at(L + 2, 0);
-  int64_t k = 0;
-  for (int64_t v = 0; v < n; v++)
-    if (g->hdeg[v] >= 1 && g->hdeg[v] <= L) cnt[g->hdeg[v]]++;
-  for (int d = L; d >= 1; d--) {
-    at[d] = k;
-    k += cnt[d];
-  }
-  *nout = k;
-  if (k == 0) return LGC_OK;
+  std::vector<int64_t> at(kDetBig + 1, 0);
   std::vector<int32_t> order;
+  int64_t k = 0;
   try {
+    g->short_at.assign(kDetBig + 1, 0);
+    for (int64_t v = 0; v < n; v++)
+      if (g->hdeg[v] >= 1 && g->hdeg[v] <= kDetBig) at[g->hdeg[v]]++;
+    for (int d = kDetBig; d >= 1; d--) {
+      const int64_t c = at[d];
+      g->short_at[d] = at[d] = k;
+      k += c;
+    }
+    g->short_at[0] = k;
     order.resize(k);
   } catch (...) {
     return LGC_ENOMEM;
   }
+  if (k == 0) return LGC_OK;
   for (int64_t v = 0; v < n; v++) {
     const int32_t d = g->hdeg[v];
-    if (d >= 1 && d <= L) order[at[d]++] = (int32_t)v;
+    if (d >= 1 && d <= kDetBig) order[at[d]++] = (int32_t)v;
   }
   int32_t* d_order = nullptr;
   LGC_TRY(dalloc_t(ctx, &d_order, k));
-  int st = dalloc_t(ctx, out, k);
+  int st = dalloc_t(ctx, &g->shorts, k);
   if (st == LGC_OK &&
       cudaMemcpyAsync(d_order, order.data(), 4 * k, cudaMemcpyHostToDevice, s) != cudaSuccess)
     st = LGC_ECUDA;
   if (st == LGC_OK) {
-    light_items_kernel<<<grid_for(k), kBlock, 0, s>>>(d_order, k, g->off, *out);
+    light_items_kernel<<<grid_for(k), kBlock, 0, s>>>(d_order, k, g->off, g->shorts);
     LGC_COUNT_LAUNCH(ctx);
     if (cudaGetLastError() != cudaSuccess || cudaStreamSynchronize(s) != cudaSuccess)
       st = LGC_ECUDA;  // (the host order goes out of scope)
   }
   dfree(ctx, d_order);
-  return st;
-}
-
-// The atomic pull's light list (degree <= pull_light) and the deterministic
-// pull's (degree <= kPullLight), shared while the two bins agree.
-int build_light_items(lgc_ctx* ctx, lgc_graph* g) {
-  LGC_TRY(build_light_list(ctx, g, g->pull_light, &g->light, &g->nlight));
-  if (g->pull_light == kPullLight) {
-    g->light_det = g->light;
-    g->nlight_det = g->nlight;
-    return LGC_OK;
-  }
-  return build_light_list(ctx, g, kPullLight, &g->light_det, &g->nlight_det);
+  return st == LGC_OK ? build_slices(ctx, g) : st;
 }
 
 // The vertices of degree > kPullLight, ascending, for pull rounds, and their
@@ -415,31 +443,16 @@ int build_recip(lgc_ctx* ctx, lgc_graph* g) {
 
 namespace lgc {
 
-// Rebuilds the degree-binned vertex lists of the pull rounds for the atomic
-// light threshold L: vertices of degree 1..L one thread each (grouped by
-// degree), the others in work items.  The deterministic lists keep their own
-// bins whatever L is: degree 1..kPullLight one thread each, (kPullLight,
-// kDetBig] one lane each, longer ones segment-parallel.
+// Moves the bin of the atomic pull rounds to L: vertices of degree 1..L one
+// thread each, the others in work items, which are cut anew.
 int rebuild_pull_lists(lgc_ctx* ctx, lgc_graph* g, int L) {
   if (L < 4 || L > 256) return LGC_EINVAL;
-  if (g->light_det != g->light) dfree(ctx, g->light_det);
-  for (void* p : {(void*)g->heavy, (void*)g->items, (void*)g->big_w, (void*)g->big_seg0,
-                  (void*)g->segs, (void*)g->det_mid, (void*)g->light})
-    dfree(ctx, p);
-  g->light_det = nullptr;
-  g->nlight_det = 0;
+  for (void* p : {(void*)g->heavy, (void*)g->items}) dfree(ctx, p);
   g->heavy = nullptr;
   g->items = nullptr;
-  g->big_w = nullptr;
-  g->big_seg0 = nullptr;
-  g->segs = nullptr;
-  g->det_mid = nullptr;
-  g->light = nullptr;
-  g->nheavy = g->nitems = g->nbig = g->nsegs = g->ndet_mid = g->nlight = 0;
+  g->nheavy = g->nitems = 0;
   g->pull_light = L;
-  LGC_TRY(build_heavy_list(ctx, g));
-  LGC_TRY(build_big_segments(ctx, g));
-  return build_light_items(ctx, g);
+  return build_heavy_list(ctx, g);
 }
 
 }  // namespace lgc
@@ -996,7 +1009,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     }
     st = build_heavy_list(ctx, g);
     if (st == LGC_OK) st = build_big_segments(ctx, g);
-    if (st == LGC_OK) st = build_light_items(ctx, g);
+    if (st == LGC_OK) st = build_shorts(ctx, g);
     if (st == LGC_OK) st = build_recip(ctx, g);
     if (st == LGC_OK) st = build_hot(ctx, g);
   } while (0);
@@ -1009,9 +1022,9 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     dfree(ctx, g->big_w);
     dfree(ctx, g->big_seg0);
     dfree(ctx, g->segs);
-    dfree(ctx, g->det_mid);
-    if (g->light_det != g->light) dfree(ctx, g->light_det);
-    dfree(ctx, g->light);
+    dfree(ctx, g->shorts);
+    dfree(ctx, g->slice_col);
+    dfree(ctx, g->slice_at);
     dfree(ctx, g->recip);
     dfree(ctx, g->hot_mem);
     cudaStreamSynchronize(s);
@@ -1050,9 +1063,9 @@ void lgc_graph_destroy(lgc_graph* g) {
   dfree(ctx, g->big_w);
   dfree(ctx, g->big_seg0);
   dfree(ctx, g->segs);
-  dfree(ctx, g->det_mid);
-  if (g->light_det != g->light) dfree(ctx, g->light_det);
-  dfree(ctx, g->light);
+  dfree(ctx, g->shorts);
+  dfree(ctx, g->slice_col);
+  dfree(ctx, g->slice_at);
   dfree(ctx, g->recip);
   dfree(ctx, g->hot_mem);
   cudaStreamSynchronize(ctx->stream);

@@ -271,12 +271,33 @@ struct __align__(32) PullItem {
   int64_t pad;
 };
 
-// A vertex of degree 1..kPullLight for the atomic pull gather: its list
-// [beg, beg + d).  The graph keeps them grouped by degree (highest first), so
-// the threads of a warp walk lists of one length.
+// A vertex of degree 1..kDetBig for the gathers that give a vertex one
+// thread: its list [beg, beg + d).  The graph keeps them grouped by degree
+// (highest first), so the threads of a warp walk lists of one length.
 struct __align__(16) LightItem {
   int64_t beg;
   int32_t w, d;
+};
+
+// Entries [beg, end) of that list, and their columns: with slices, those of
+// entries 32 k .. 32 k + 31 lie interleaved from col[slice[k]] on (edge e of
+// entry i at slice[i / 32] + 32 e + i % 32), so that a warp's column load
+// reads one line; walking 32 lists side by side touches as many lines as the
+// gather of the shares and took as much of L1 (scale-22 R-MAT, degree 1..256:
+// 166 -> 127 us a gather).  Without slices, entry i's columns are
+// col[items[i].beg + e].
+struct LightView {
+  const LightItem* items;
+  int64_t beg, end;
+  const int32_t* col;
+  const int64_t* slice;
+  // Threads that walk it: thread t takes entry first() + t.
+  __host__ __device__ int64_t first() const { return beg & ~int64_t{31}; }
+  __host__ __device__ int64_t threads() const { return end - first(); }
+  __device__ const int32_t* columns(int64_t i, const LightItem& it) const {
+    return slice ? col + slice[i >> 5] + (i & 31) : col + it.beg;
+  }
+  __device__ int stride() const { return slice ? 32 : 1; }
 };
 
 // A 256-edge segment of a big vertex's list (deterministic pull rounds):
@@ -317,10 +338,6 @@ struct lgc_graph {
   // load)
   PullItem* items = nullptr;
   int64_t nitems = 0;
-  // vertices of degree in (kPullLight, kDetBig], longest lists first (one
-  // lane each folds its list in the deterministic pull)
-  int32_t* det_mid = nullptr;
-  int64_t ndet_mid = 0;
   // vertices of degree > kDetBig, whose deterministic fold runs segment-
   // parallel: their ids, the first of their segments (nbig + 1 prefix), and
   // the 256-edge segments
@@ -329,14 +346,19 @@ struct lgc_graph {
   int64_t nbig = 0;
   DetSeg* segs = nullptr;
   int64_t nsegs = 0;
-  // vertices of degree 1..pull_light grouped by degree (atomic pull rounds)
-  LightItem* light = nullptr;
-  int64_t nlight = 0;
-  // the deterministic pull's own list of vertices of degree 1..kPullLight
-  // (its light lists fold in one thread, so its bin stays at kPullLight);
-  // the atomic list itself while pull_light == kPullLight
-  LightItem* light_det = nullptr;
-  int64_t nlight_det = 0;
+  // vertices of degree 1..kDetBig grouped by degree, highest first; those of
+  // degree d or less start at short_at[d] (short_at[0]: their number).  The
+  // atomic pull takes degree 1..pull_light from it, the deterministic one
+  // 1..kPullLight and the rest apart.  slice_col, slice_at: the interleaved
+  // columns (null where device memory is short; see LightView).
+  LightItem* shorts = nullptr;
+  std::vector<int64_t> short_at;
+  int32_t* slice_col = nullptr;
+  int64_t* slice_at = nullptr;
+  LightView view(int from, int to) const {  // degrees from..to
+    if (!shorts) return {nullptr, 0, 0, nullptr, nullptr};
+    return {shorts, short_at[to], short_at[from - 1], slice_col ? slice_col : col, slice_at};
+  }
 };
 
 namespace lgc {

@@ -505,21 +505,22 @@ __device__ inline bool pull_qualifies(double acc, int64_t d, LiteThr c, int fmod
 // list in order (acc <- RN(acc + s) from the present value), taking the
 // vertices from the graph's list grouped by degree so that a warp's chains
 // have one length.  qbits is cleared before; qualifying vertices are ORed in.
-__global__ void pull_light_kernel(const LightItem* __restrict__ items, int64_t nl,
-                                  const int32_t* __restrict__ col,
-                                  const double* __restrict__ sh, Table D, LiteThr c, int fmode,
-                                  uint32_t* __restrict__ qbits, Counters* C) {
+__global__ void pull_light_kernel(LightView V, const double* __restrict__ sh, Table D, LiteThr c,
+                                  int fmode, uint32_t* __restrict__ qbits, Counters* C) {
+  const int stride = V.stride();
   int64_t nins = 0;  // keys inserted here, counted once per block
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nl;
+  for (int64_t i = V.first() + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V.end;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const LightItem it = items[i];
+    if (i < V.beg) continue;
+    const LightItem it = V.items[i];
+    const int32_t* col = V.columns(i, it);
     const int32_t w = it.w;
     const uint32_t m = 1u << (w & 31);
     const bool present = (D.bits[w >> 5] & m) != 0;
     double acc = present ? D.dval[w] : 0.0;
     bool touched = present;
     for (int k = 0; k < it.d; k++) {
-      const double x = sh[col[it.beg + k]];
+      const double x = sh[col[k * stride]];
       if (pull_member(x)) {
         acc = acc + x;
         touched = true;
@@ -559,18 +560,18 @@ __device__ inline int pull_finish(const Table& D, int32_t w, int64_t d, double a
 // so every add is issued for (nearly) all 32 lanes; each lane loads eight
 // columns, then their eight shares, before folding them.
 __global__ void __launch_bounds__(kBlock)
-    pull_mid_det_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ col,
-                        const int32_t* __restrict__ mid, int64_t nmid,
-                        const double* __restrict__ sh, Table D, LiteThr c, int fmode,
+    pull_mid_det_kernel(LightView V, const double* __restrict__ sh, Table D, LiteThr c, int fmode,
                         uint32_t* __restrict__ qbits, Counters* C) {
+  const int stride = V.stride();
   int64_t nins = 0;  // keys inserted here, counted once per block
-  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nmid;
+  for (int64_t base = V.first() + (int64_t)blockIdx.x * blockDim.x; base < V.end;
        base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = base + threadIdx.x;
     int ins = 0;
-    if (i < nmid) {
-      const int32_t w = mid[i];
-      const int64_t o0 = off[w], d = off[w + 1] - o0;
+    if (i >= V.beg && i < V.end) {
+      const LightItem it = V.items[i];
+      const int32_t* col = V.columns(i, it);
+      const int32_t w = it.w, d = it.d;
       const uint32_t m = 1u << (w & 31);
       const bool present = (D.bits[w >> 5] & m) != 0;
       double acc = present ? D.dval[w] : 0.0;
@@ -581,17 +582,17 @@ __global__ void __launch_bounds__(kBlock)
       int32_t u[16], un[16];
       double x[16];
 #pragma unroll
-      for (int j = 0; j < 16; j++) u[j] = j < d ? col[o0 + j] : -1;
+      for (int j = 0; j < 16; j++) u[j] = j < d ? col[j * stride] : -1;
 #pragma unroll
-      for (int j = 0; j < 16; j++) un[j] = 16 + j < d ? col[o0 + 16 + j] : -1;
+      for (int j = 0; j < 16; j++) un[j] = 16 + j < d ? col[(16 + j) * stride] : -1;
 #pragma unroll
       for (int j = 0; j < 16; j++) x[j] = u[j] >= 0 ? sh[u[j]] : 0.0;
-      for (int64_t k = 0; k < d; k += 16) {
+      for (int k = 0; k < d; k += 16) {
         double xn[16];
 #pragma unroll
         for (int j = 0; j < 16; j++) xn[j] = un[j] >= 0 ? sh[un[j]] : 0.0;
 #pragma unroll
-        for (int j = 0; j < 16; j++) u[j] = k + 32 + j < d ? col[o0 + k + 32 + j] : -1;
+        for (int j = 0; j < 16; j++) u[j] = k + 32 + j < d ? col[(k + 32 + j) * stride] : -1;
 #pragma unroll
         for (int j = 0; j < 16; j++) {
           if (pull_member(x[j])) {  // in order: j ascending is adjacency order
@@ -966,26 +967,28 @@ __device__ inline void pull_windows(const int32_t* range, int L, Body&& body) {
 // The bitmap qbits is cleared before this launch; this kernel and the heavy
 // one OR their qualifying vertices in.
 template <int W, typename SH>
-__device__ inline int64_t pull_light_fx_body(const LightItem* __restrict__ items, int64_t nl,
-                                             const int32_t* __restrict__ col,
-                                             const SH* __restrict__ shx, uint32_t be0, int L,
-                                             const Table& D, LiteThr c, int fmode,
-                                             uint32_t* __restrict__ qbits) {
+__device__ inline int64_t pull_light_fx_body(const LightView& V, const SH* __restrict__ shx,
+                                             uint32_t be0, int L, const Table& D, LiteThr c,
+                                             int fmode, uint32_t* __restrict__ qbits) {
+  constexpr int kB = W == 0 ? 4 : 8;  // edges in flight (128-bit sums: registers)
+  const int stride = V.stride();
   int64_t nins = 0;  // keys inserted here, counted once per block
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nl;
+  for (int64_t i = V.first() + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V.end;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const LightItem it = items[i];
+    if (i < V.beg) continue;
+    const LightItem it = V.items[i];
+    const int32_t* __restrict__ col = V.columns(i, it);
     const int32_t w = it.w, d = it.d;
     PullSum<W, SH> sum;
-    for (int k = 0; k < d; k += 4) {
-      int32_t u[4];
+    for (int k = 0; k < d; k += kB) {
+      int32_t u[kB];
 #pragma unroll
-      for (int j = 0; j < 4; j++) u[j] = k + j < d ? col[it.beg + k + j] : -1;
-      SH raw[4];
+      for (int j = 0; j < kB; j++) u[j] = k + j < d ? col[(k + j) * stride] : -1;
+      SH raw[kB];
 #pragma unroll
-      for (int j = 0; j < 4; j++) raw[j] = u[j] >= 0 ? shx[u[j]] : no_share<SH>();
+      for (int j = 0; j < kB; j++) raw[j] = u[j] >= 0 ? shx[u[j]] : no_share<SH>();
 #pragma unroll
-      for (int j = 0; j < 4; j++) sum.add(raw[j], L, be0);
+      for (int j = 0; j < kB; j++) sum.add(raw[j], L, be0);
     }
     const uint32_t m = 1u << (w & 31);
     const bool present = (D.bits[w >> 5] & m) != 0;
@@ -1131,17 +1134,14 @@ __global__ void __launch_bounds__(kBlock)
 }
 
 template <typename SH>
-__global__ void pull_light_fx_kernel(const LightItem* __restrict__ items, int64_t nl,
-                                     const int32_t* __restrict__ col,
-                                     const SH* __restrict__ shx,
+__global__ void pull_light_fx_kernel(LightView V, const SH* __restrict__ shx,
                                      const int32_t* __restrict__ range, int g, Table D, LiteThr c,
                                      int fmode, uint32_t* __restrict__ qbits, Counters* C) {
   const int L = round_scale(range, g);
   const uint32_t be0 = (uint32_t)(2047 - range[0]);
   int64_t nins = 0;
   pull_windows<SH>(range, L, [&](auto w) {
-    nins = pull_light_fx_body<decltype(w)::value, SH>(items, nl, col, shx, be0, L, D, c, fmode,
-                                                      qbits);
+    nins = pull_light_fx_body<decltype(w)::value, SH>(V, shx, be0, L, D, c, fmode, qbits);
   });
   flush_count(nins, &C->inserted);
 }
@@ -1472,6 +1472,10 @@ namespace {
 
 int64_t min64(int64_t a, int64_t b) { return a < b ? a : b; }
 
+int light_grid(const lgc_ctx* ctx, const LightView& V) {
+  return (int)min64(ceil_div(V.threads(), kBlock), ctx->sms * 32);
+}
+
 // Sets of a graph of up to kDenseSmall vertices are dense from the start
 // (automatic form): clearing 16 bytes a vertex costs 4 us at that size,
 // growing and converting a table on the way 40 us and more.
@@ -1801,18 +1805,15 @@ struct PushWork {
       if (det) {
         // every gather ORs its qualifying vertices into the cleared bitmap
         LGC_CUDA_TRY(cudaMemsetAsync(pq.ptr, 0, 4 * words, s));
-        if (g->nlight_det > 0) {
-          const int lgl =
-              (int)std::min<int64_t>(ceil_div(g->nlight_det, kBlock), (ctx->sms * 32));
-          pull_light_kernel<<<lgl, kBlock, 0, s>>>(g->light_det, g->nlight_det, g->col, psh.ptr,
-                                                   D, ct, fmode, pq.ptr, ctx->d_counters);
+        const LightView light = g->view(1, kPullLight), mid = g->view(kPullLight + 1, kDetBig);
+        if (light.end > light.beg) {
+          pull_light_kernel<<<light_grid(ctx, light), kBlock, 0, s>>>(
+              light, psh.ptr, D, ct, fmode, pq.ptr, ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
-        if (g->ndet_mid > 0) {
-          const int mg = (int)std::min<int64_t>(ceil_div(g->ndet_mid, kBlock), (ctx->sms * 32));
-          pull_mid_det_kernel<<<mg, kBlock, 0, s>>>(g->off, g->col, g->det_mid, g->ndet_mid,
-                                                    psh.ptr, D, ct, fmode, pq.ptr,
-                                                    ctx->d_counters);
+        if (mid.end > mid.beg) {
+          pull_mid_det_kernel<<<light_grid(ctx, mid), kBlock, 0, s>>>(
+              mid, psh.ptr, D, ct, fmode, pq.ptr, ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
         if (g->nbig > 0) {  // lists longer than kDetBig, folded segment-parallel
@@ -1842,11 +1843,10 @@ struct PushWork {
         // (ORing their vertices in); the two in one grid measured slower
         auto gather = [&](auto* shv) {
           using SH = std::remove_const_t<std::remove_pointer_t<decltype(shv)>>;
-          if (g->nlight > 0) {
-            const int lgl = (int)std::min<int64_t>(ceil_div(g->nlight, kBlock), (ctx->sms * 32));
-            pull_light_fx_kernel<SH><<<lgl, kBlock, 0, s>>>(g->light, g->nlight, g->col, shv,
-                                                             prange.ptr, gb, D, ct, fmode, pq.ptr,
-                                                             ctx->d_counters);
+          const LightView light = g->view(1, g->pull_light);
+          if (light.end > light.beg) {
+            pull_light_fx_kernel<SH><<<light_grid(ctx, light), kBlock, 0, s>>>(
+                light, shv, prange.ptr, gb, D, ct, fmode, pq.ptr, ctx->d_counters);
             LGC_COUNT_LAUNCH(ctx);
           }
           if (g->nitems > 0) {
@@ -2216,19 +2216,17 @@ int autotune_pull(lgc_ctx* ctx, lgc_graph* g) {
         st = LGC_ECUDA;
         break;
       }
+      const LightView light = g->view(1, g->pull_light);
       for (int sb : {16, 8}) {
         float light_ms = 0.f;
         auto light_of = [&](auto* shv) {
           using SH = std::remove_pointer_t<decltype(shv)>;
-          const int lgl = (int)std::max<int64_t>(
-              1, std::min<int64_t>(ceil_div(g->nlight, kBlock), (ctx->sms * 32)));
           timed([&] {
-            pull_light_fx_kernel<SH><<<lgl, kBlock, 0, s>>>(g->light, g->nlight, g->col, shv,
-                                                           range, gb, D, lite_thr(1.0),
-                                                           kFmThreshold, q, ctx->d_counters);
+            pull_light_fx_kernel<SH><<<light_grid(ctx, light), kBlock, 0, s>>>(
+                light, shv, range, gb, D, lite_thr(1.0), kFmThreshold, q, ctx->d_counters);
           }, &light_ms);
         };
-        if (g->nlight > 0) {
+        if (light.end > light.beg) {
           if (sb == 16) light_of(shx);
           else light_of(shd);
         }

@@ -200,20 +200,21 @@ __device__ inline int ranked_before(uint32_t ru, uint32_t r) { return ru - 1u < 
 
 // Vertices of degree 1..light, one thread each, from the graph's list
 // grouped by degree; four edges' loads in flight.
-__global__ void sweep_cross_light_kernel(const LightItem* __restrict__ items, int64_t nl,
-                                         const int32_t* __restrict__ col,
-                                         const int32_t* __restrict__ drank,
+__global__ void sweep_cross_light_kernel(LightView V, const int32_t* __restrict__ drank,
                                          int32_t* __restrict__ before) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nl;
+  const int stride = V.stride();
+  for (int64_t i = V.first() + (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < V.end;
        i += (int64_t)gridDim.x * blockDim.x) {
-    const LightItem it = items[i];
+    if (i < V.beg) continue;
+    const LightItem it = V.items[i];
+    const int32_t* __restrict__ col = V.columns(i, it);
     const uint32_t r = (uint32_t)drank[it.w];
     if (r == 0) continue;
     int cnt = 0;
     for (int k = 0; k < it.d; k += 4) {
       int32_t u[4];
 #pragma unroll
-      for (int j = 0; j < 4; j++) u[j] = k + j < it.d ? col[it.beg + k + j] : -1;
+      for (int j = 0; j < 4; j++) u[j] = k + j < it.d ? col[(k + j) * stride] : -1;
       uint32_t ru[4];
 #pragma unroll
       for (int j = 0; j < 4; j++) ru[j] = u[j] >= 0 ? (uint32_t)drank[u[j]] : 0u;
@@ -601,10 +602,18 @@ int run_sweep(lgc_ctx* ctx, lgc_graph* g, const lgc_svec* p, lgc_cluster** out) 
     if (vertex_centric) {
       // algorithmic bytes: 12 per edge (col 4, rank key 4, rank 4), 24 per vertex
       ProfScope ps(ctx, LGC_PROF_SWEEP, 0.0);
-      if (g->nlight > 0) {
-        const int lg = (int)std::min<int64_t>(ceil_div(g->nlight, kBlock), ctx->sms * 32);
-        sweep_cross_light_kernel<<<lg, kBlock, 0, s>>>(g->light, g->nlight, g->col, drank,
-                                                       before);
+      LightView light = g->view(1, g->pull_light);
+      // A swept vertex's own columns are d / 8 sectors of 32 bytes; a warp's
+      // interleaved ones are 4 d sectors however few of its 32 lists are
+      // walked.  The two meet where all are; the loads (one a column against
+      // one a list and column) already favour the interleaved ones at a few.
+      if (n0 < g->n / 4) {
+        light.col = g->col;
+        light.slice = nullptr;
+      }
+      if (light.end > light.beg) {
+        const int lg = (int)std::min<int64_t>(ceil_div(light.threads(), kBlock), ctx->sms * 32);
+        sweep_cross_light_kernel<<<lg, kBlock, 0, s>>>(light, drank, before);
         LGC_COUNT_LAUNCH(ctx);
       }
       if (g->nitems > 0) {
