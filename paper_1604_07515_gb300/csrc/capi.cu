@@ -117,7 +117,7 @@ __global__ void gather_off_kernel(const int32_t* __restrict__ ids, int64_t k,
     out[i] = off[ids[i]];
 }
 
-// The deterministic pull's vertices of degree > kDetBig with their 256-edge
+// The deterministic pull's vertices of degree > kDetBig, longest lists first, with their 256-edge
 // segments (built on the host from the degree copy; only their list starts are
 // read back).
 int build_big_segments(lgc_ctx* ctx, lgc_graph* g) {
@@ -125,6 +125,8 @@ int build_big_segments(lgc_ctx* ctx, lgc_graph* g) {
   std::vector<int32_t> bw;
   for (int64_t v = 0; v < g->n; v++)
     if (g->hdeg[v] > kDetBig) bw.push_back((int32_t)v);
+  std::stable_sort(bw.begin(), bw.end(),
+                   [&](int32_t a, int32_t b) { return g->hdeg[a] > g->hdeg[b]; });
   g->nbig = (int64_t)bw.size();
   if (g->nbig == 0) return LGC_OK;
   std::vector<int64_t> starts(g->nbig), seg0(g->nbig + 1, 0);
@@ -212,8 +214,12 @@ int build_slices(lgc_ctx* ctx, lgc_graph* g) {
   size_t avail = 0, all = 0;
   LGC_CUDA_TRY(cudaMemGetInfo(&avail, &all));
   if (bytes > avail / 8) return LGC_OK;
-  LGC_TRY(dalloc_t(ctx, &g->slice_at, nslices + 1));
-  LGC_TRY(dalloc_t(ctx, &g->slice_col, at[nslices]));
+  if (dalloc_t(ctx, &g->slice_at, nslices + 1) != LGC_OK ||
+      dalloc_t(ctx, &g->slice_col, at[nslices]) != LGC_OK) {
+    dfree(ctx, g->slice_at);
+    g->slice_at = nullptr;
+    return LGC_OK;
+  }
   LGC_CUDA_TRY(cudaMemcpyAsync(g->slice_at, at.data(), 8 * (nslices + 1), cudaMemcpyHostToDevice,
                                s));
   slice_fill_kernel<<<std::min(grid_for(k), ctx->sms * 16), kBlock, 0, s>>>(

@@ -367,6 +367,7 @@ namespace lgc {
 constexpr int kPullLight = 32;  // default of lgc_graph::pull_light; the deterministic bin
 constexpr int kDetBig = 1024;  // longer lists fold segment-parallel in deterministic mode
 constexpr int kDetSeg = 256;
+constexpr int64_t kDetKeep = int64_t{1} << 18;  // segments whose gathered shares are kept (512 MB)
 constexpr int kPullItem = 4096;
 }  // namespace lgc
 

@@ -555,64 +555,74 @@ __device__ inline int pull_finish(const Table& D, int32_t w, int64_t d, double a
 
 // Deterministic mode, vertices of degree (kPullLight, kDetBig]: one lane per
 // vertex folds its in-frontier shares in adjacency order with FP64 adds --
-// the fold's definition, so bit-identical by construction.  The vertices are
-// taken longest list first and a warp's lanes have lists of similar length,
-// so every add is issued for (nearly) all 32 lanes; each lane loads eight
-// columns, then their eight shares, before folding them.
-__global__ void __launch_bounds__(kBlock)
+// the fold's definition, so bit-identical by construction (a vertex outside
+// the frontier has the share +0.0, which adds nothing to a value of at least
+// +0.0).  The vertices are taken longest list first and a warp's lanes have
+// lists of similar length, so every add is issued for (nearly) all 32 lanes.
+//
+// A quarter of an SM takes an FP64 warp instruction every 64 cycles, dependent
+// or not, so two warps a quarter keep its pipe busy, and what matters is that
+// the longest lists lie one to a quarter: a block an SM, its warps' first
+// slices dealt across the blocks (longest first), the others taken as warps
+// come free.  A batch's shares and the next one's columns are read before the
+// adds of the batch before.  The 15.1M edges of a scale-20 R-MAT graph's middle
+// lists: 137 us with neighbouring slices in one block, 104 dealt to two blocks
+// of 8 warps an SM, 88 so; 94 with 12 warps, 96 with 16, 111 with 24 and
+// batches of 8; 195 with the shares copied ahead to shared memory.  Of it 60
+// are the adds and 75 the loads, each by itself.
+constexpr int kMidB = 16;
+
+__global__ void __launch_bounds__(kBlock, 1)
     pull_mid_det_kernel(LightView V, const double* __restrict__ sh, Table D, LiteThr c, int fmode,
-                        uint32_t* __restrict__ qbits, Counters* C) {
+                        uint32_t* __restrict__ qbits, unsigned* __restrict__ ticket, Counters* C) {
+  const int lane = threadIdx.x & 31;
   const int stride = V.stride();
-  int64_t nins = 0;  // keys inserted here, counted once per block
-  for (int64_t base = V.first() + (int64_t)blockIdx.x * blockDim.x; base < V.end;
-       base += (int64_t)gridDim.x * blockDim.x) {
-    const int64_t i = base + threadIdx.x;
-    int ins = 0;
-    if (i >= V.beg && i < V.end) {
-      const LightItem it = V.items[i];
-      const int32_t* col = V.columns(i, it);
-      const int32_t w = it.w, d = it.d;
-      const uint32_t m = 1u << (w & 31);
-      const bool present = (D.bits[w >> 5] & m) != 0;
-      double acc = present ? D.dval[w] : 0.0;
-      bool touched = present;
-      // software-pipelined: the next batch's shares and the batch after's
-      // columns are read before this batch's adds, so a batch costs the
-      // larger of one memory trip and its sixteen dependent adds, not both
-      int32_t u[16], un[16];
-      double x[16];
-#pragma unroll
-      for (int j = 0; j < 16; j++) u[j] = j < d ? col[j * stride] : -1;
-#pragma unroll
-      for (int j = 0; j < 16; j++) un[j] = 16 + j < d ? col[(16 + j) * stride] : -1;
-#pragma unroll
-      for (int j = 0; j < 16; j++) x[j] = u[j] >= 0 ? sh[u[j]] : 0.0;
-      for (int k = 0; k < d; k += 16) {
-        double xn[16];
-#pragma unroll
-        for (int j = 0; j < 16; j++) xn[j] = un[j] >= 0 ? sh[un[j]] : 0.0;
-#pragma unroll
-        for (int j = 0; j < 16; j++) u[j] = k + 32 + j < d ? col[(k + 32 + j) * stride] : -1;
-#pragma unroll
-        for (int j = 0; j < 16; j++) {
-          if (pull_member(x[j])) {  // in order: j ascending is adjacency order
-            acc = acc + x[j];
-            touched = true;
-          }
-        }
-#pragma unroll
-        for (int j = 0; j < 16; j++) {
-          x[j] = xn[j];
-          un[j] = u[j];
-        }
-      }
-      if (touched) {
-        D.dval[w] = acc;
-        if (!present && !(atomicOr(&D.bits[w >> 5], m) & m)) ins = 1;
-        if (pull_qualifies(acc, d, c, fmode)) atomicOr(&qbits[w >> 5], m);
-      }
+  int64_t nins = 0;  // keys inserted here
+  unsigned t = (threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  for (bool own = true;; own = false) {
+    if (!own) {
+      if (lane == 0) t = gridDim.x * (kBlock / 32) + atomicAdd(ticket, 1u);
+      t = __shfl_sync(0xffffffffu, t, 0);
     }
-    nins += ins;
+    const int64_t base = V.first() + 32 * (int64_t)t;
+    if (base >= V.end) break;
+    const int64_t i = base + lane;
+    if (i < V.beg || i >= V.end) continue;
+    const LightItem it = V.items[i];
+    const int32_t* __restrict__ col = V.columns(i, it);
+    const int32_t w = it.w, d = it.d;
+    const uint32_t m = 1u << (w & 31);
+    const bool present = (D.bits[w >> 5] & m) != 0;
+    double acc = present ? D.dval[w] : 0.0;
+    uint64_t any = 0;
+    int32_t u[kMidB];
+    double x[kMidB];
+    auto columns = [&](int k) {
+#pragma unroll
+      for (int j = 0; j < kMidB; j++) u[j] = k + j < d ? col[(k + j) * stride] : -1;
+    };
+    columns(0);
+#pragma unroll
+    for (int j = 0; j < kMidB; j++) x[j] = u[j] >= 0 ? sh[u[j]] : 0.0;
+    columns(kMidB);
+    for (int k = 0; k < d; k += kMidB) {
+      double xn[kMidB];
+#pragma unroll
+      for (int j = 0; j < kMidB; j++) xn[j] = u[j] >= 0 ? sh[u[j]] : 0.0;
+      columns(k + 2 * kMidB);
+#pragma unroll
+      for (int j = 0; j < kMidB; j++) {  // in order: j ascending is adjacency order
+        acc = acc + x[j];
+        any |= (uint64_t)__double_as_longlong(x[j]);
+      }
+#pragma unroll
+      for (int j = 0; j < kMidB; j++) x[j] = xn[j];
+    }
+    if (present || any) {
+      D.dval[w] = acc;
+      if (!present && !(atomicOr(&D.bits[w >> 5], m) & m)) nins++;
+      if (pull_qualifies(acc, d, c, fmode)) atomicOr(&qbits[w >> 5], m);
+    }
   }
   flush_count(nins, &C->inserted);
 }
@@ -620,24 +630,30 @@ __global__ void __launch_bounds__(kBlock)
 // ---------------------------------------------------------------------------
 // Deterministic mode, vertices of degree > kDetBig: the fold of the whole
 // list is split into 256-edge segments that are worked on in parallel.
-//  1. det_seg_sum: each segment's plain sum and whether it holds a member.
+//  1. det_seg_sum: each segment's sum to about 20 bits and whether it holds a
+//     member; the gathered shares are kept for 3 and 4 (up to kDetKeep
+//     segments, beyond which those gather again).
 //  2. det_seg_predict: per vertex, a running sum of the segment sums
-//     predicts the binade the fold is in at each segment's start (the fold
-//     differs from the exact prefix sum by rounding only, so the prediction
-//     misses only next to a power of two).
+//     predicts the binade the fold is in at each segment's start (the
+//     prediction misses only next to a power of two).
 //  3. det_seg_step: each segment's composed integer step (see fold_step) for
 //     its predicted binade.
-//  4. det_seg_verify: one warp per vertex walks its segments in order: when
-//     the fold's actual binade is the predicted one and the composed step
-//     keeps the value below 2^53, the step is the exact fold of the segment
-//     (the value only grows, so no intermediate value left the binade);
-//     otherwise the segment is folded element by element (fold_batch).
+//  4. det_seg_verify: one warp per vertex walks its segments in order, up to
+//     32 at a time: while the fold's actual binade is the predicted one and
+//     the steps composed so far keep the value below 2^53, they are the exact
+//     fold of their segments (the value only grows, so no intermediate value
+//     left the binade); the segment that does not is folded element by
+//     element (fold_batch), its shares loaded ahead where the next one's
+//     prediction tells it.
 // The result is the sequential fold, bit for bit.
 // ---------------------------------------------------------------------------
+// A sum for prediction only: the shares' leading 21 bits in units of the
+// largest one's last, in 32-bit integers (256 of them stay below 2^29).  The
+// plain sum's 13 FP64 adds a segment were the pass's bound.
 __global__ void det_seg_sum_kernel(const int32_t* __restrict__ col,
                                    const DetSeg* __restrict__ segs, int64_t nsegs,
                                    const double* __restrict__ sh, double* __restrict__ segsum,
-                                   int32_t* __restrict__ segany) {
+                                   int32_t* __restrict__ segany, double* __restrict__ kept) {
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
@@ -646,18 +662,30 @@ __global__ void det_seg_sum_kernel(const int32_t* __restrict__ col,
     int32_t u[8];
 #pragma unroll
     for (int j = 0; j < 8; j++) u[j] = 32 * j + lane < S.len ? col[S.beg + 32 * j + lane] : -1;
-    double x = 0.0;
+    double v[8];
+#pragma unroll
+    for (int j = 0; j < 8; j++) v[j] = u[j] >= 0 ? sh[u[j]] : 0.0;
+    uint32_t top = 0;
     bool mem = false;
 #pragma unroll
     for (int j = 0; j < 8; j++) {
-      const double v = u[j] >= 0 ? sh[u[j]] : 0.0;
-      x += v;
-      mem = mem || pull_member(v);
+      if (kept) kept[kDetSeg * k + 32 * j + lane] = v[j];
+      mem = mem || pull_member(v[j]);
+      top = max(top, (uint32_t)__double2hiint(v[j]) >> 20 & 2047u);
     }
-    for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    top = __reduce_max_sync(0xffffffffu, top);
+    uint32_t x = 0;
+#pragma unroll
+    for (int j = 0; j < 8; j++) {
+      const uint32_t hi = (uint32_t)__double2hiint(v[j]);
+      const uint32_t be = hi >> 20 & 2047u;
+      if (be) x += ((hi & 0xFFFFFu) | 0x100000u) >> min(top - be, 31u);
+    }
+    x = __reduce_add_sync(0xffffffffu, x);
     const bool any = __any_sync(0xffffffffu, mem);
     if (lane == 0) {
-      segsum[k] = x;
+      // x * 2^(top - 1043); below 2^-1002 predicted as nothing
+      segsum[k] = top > 20 ? (double)x * __hiloint2double((int)((top - 20) << 20), 0) : 0.0;
       segany[k] = any ? 1 : 0;
     }
   }
@@ -667,57 +695,104 @@ __global__ void det_seg_predict_kernel(const int32_t* __restrict__ big_w,
                                        const int64_t* __restrict__ seg0, int64_t nbig, Table D,
                                        const double* __restrict__ segsum,
                                        int32_t* __restrict__ pred) {
-  for (int64_t b = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; b < nbig;
-       b += (int64_t)gridDim.x * blockDim.x) {
+  const int lane = threadIdx.x & 31;
+  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  for (int64_t b = warp0; b < nbig; b += nwarps) {
     const int32_t w = big_w[b];
     const bool present = (D.bits[w >> 5] >> (w & 31)) & 1u;
     double acc = present ? D.dval[w] : 0.0;
-    for (int64_t k = seg0[b]; k < seg0[b + 1]; k++) {
-      pred[k] = fold_binade(acc);
-      acc += segsum[k];
+    const int64_t k1 = seg0[b + 1];
+    for (int64_t k0 = seg0[b]; k0 < k1; k0 += 32) {
+      const int64_t k = k0 + lane;
+      double x = k < k1 ? segsum[k] : 0.0;
+      for (int o = 1; o < 32; o <<= 1) {
+        const double y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      double before = __shfl_up_sync(0xffffffffu, x, 1);
+      if (lane == 0) before = 0.0;
+      if (k < k1) pred[k] = fold_binade(acc + before);
+      acc += __shfl_sync(0xffffffffu, x, 31);
     }
   }
+}
+
+// Lane l's eight shares of segment k (positions 8 l .. 8 l + 7).
+__device__ inline void det_seg_shares(const double* __restrict__ kept,
+                                      const int32_t* __restrict__ col,
+                                      const DetSeg* __restrict__ segs,
+                                      const double* __restrict__ sh, int64_t k, int lane,
+                                      double (&v)[8]) {
+  if (kept) {
+    const double2* p = reinterpret_cast<const double2*>(kept + kDetSeg * k + 8 * lane);
+#pragma unroll
+    for (int q = 0; q < 4; q++) {
+      const double2 x = p[q];
+      v[2 * q] = x.x;
+      v[2 * q + 1] = x.y;
+    }
+    return;
+  }
+  const DetSeg S = segs[k];
+  int32_t u[8];
+#pragma unroll
+  for (int q = 0; q < 8; q++) u[q] = 8 * lane + q < S.len ? col[S.beg + 8 * lane + q] : -1;
+#pragma unroll
+  for (int q = 0; q < 8; q++) v[q] = u[q] >= 0 ? sh[u[q]] : 0.0;
 }
 
 __global__ void det_seg_step_kernel(const int32_t* __restrict__ col,
                                     const DetSeg* __restrict__ segs, int64_t nsegs,
                                     const double* __restrict__ sh,
+                                    const double* __restrict__ kept,
                                     const int32_t* __restrict__ pred,
                                     FoldStep* __restrict__ step) {
   const int lane = threadIdx.x & 31;
   const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   for (int64_t k = warp0; k < nsegs; k += nwarps) {
-    const DetSeg S = segs[k];
     const int bu = pred[k];
-    int32_t u[8];
+    double v[8];
+    det_seg_shares(kept, col, segs, sh, k, lane, v);
+    int64_t x0 = 0, x1 = 1;  // the lane's steps from an even and from an odd value
+    bool par = false;
 #pragma unroll
-    for (int j = 0; j < 8; j++) u[j] = 8 * lane + j < S.len ? col[S.beg + 8 * lane + j] : -1;
-    FoldStep F = {0, 0};
-#pragma unroll
-    for (int j = 0; j < 8; j++)
-      F = fold_compose(F, fold_step(u[j] >= 0 ? sh[u[j]] : 0.0, bu));
-    // ordered reduction: lane l's steps come before lane l+1's
-    for (int o = 1; o < 32; o <<= 1) {
-      FoldStep q;
-      q.g0 = __shfl_down_sync(0xffffffffu, F.g0, o);
-      q.g1 = __shfl_down_sync(0xffffffffu, F.g1, o);
-      if ((lane & (2 * o - 1)) == 0) F = fold_compose(F, q);
+    for (int j = 0; j < 8; j++) {
+      const FoldNear f = fold_near(v[j], bu);
+      x0 = fold_take(f, x0);
+      x1 = fold_take(f, x1);
+      par = par || f.tie;
     }
-    if (lane == 0) step[k] = F;
+    FoldStep F = {x0, x1 - 1};
+    if (!__any_sync(0xffffffffu, par)) {  // no ties: plain sums
+      for (int o = 16; o > 0; o >>= 1) F.g0 += __shfl_xor_sync(0xffffffffu, F.g0, o);
+      F.g1 = F.g0;
+    } else {
+      // ordered reduction: lane l's steps come before lane l+1's
+      for (int o = 1; o < 32; o <<= 1) {
+        FoldStep q;
+        q.g0 = __shfl_down_sync(0xffffffffu, F.g0, o);
+        q.g1 = __shfl_down_sync(0xffffffffu, F.g1, o);
+        if ((lane & (2 * o - 1)) == 0) F = fold_compose(F, q);
+      }
+    }
+    // a step past 2^53 is never taken; capped, 32 of them stay in 64 bits
+    if (lane == 0) step[k] = {min(F.g0, kFoldBig), min(F.g1, kFoldBig)};
   }
 }
 
-__global__ void __launch_bounds__(kBlock)
+__global__ void __launch_bounds__(kBlock, 3)
     det_seg_verify_kernel(const int64_t* __restrict__ off, const int32_t* __restrict__ col,
                           const DetSeg* __restrict__ segs, const int32_t* __restrict__ big_w,
                           const int64_t* __restrict__ seg0, int64_t nbig,
-                          const double* __restrict__ sh, const int32_t* __restrict__ pred,
-                          const FoldStep* __restrict__ step, const int32_t* __restrict__ segany,
-                          Table D, LiteThr c, int fmode, uint32_t* __restrict__ qbits,
-                          Counters* C) {
+                          const double* __restrict__ sh, const double* __restrict__ kept,
+                          const int32_t* __restrict__ pred, const FoldStep* __restrict__ step,
+                          const int32_t* __restrict__ segany, Table D, LiteThr c, int fmode,
+                          uint32_t* __restrict__ qbits, Counters* C) {
   const int lane = threadIdx.x & 31;
-  const int64_t warp0 = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  // the vertices are longest first: neighbours go to different blocks
+  const int64_t warp0 = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;
   for (int64_t b = warp0; b < nbig; b += nwarps) {
@@ -725,38 +800,89 @@ __global__ void __launch_bounds__(kBlock)
     const bool present = (D.bits[w >> 5] >> (w & 31)) & 1u;
     double acc = present ? D.dval[w] : 0.0;  // >= +0, the same in every lane
     bool touched = present;
-    const int64_t k1 = seg0[b + 1];
-    for (int64_t k0 = seg0[b]; k0 < k1; k0 += 32) {
-      // 32 segments' predictions and steps, one per lane, walked in order
-      const int64_t kl = k0 + lane;
-      const bool ok = kl < k1;
-      const int pl = ok ? pred[kl] : 0;
-      const FoldStep sl = ok ? step[kl] : FoldStep{0, 0};
-      touched = touched || __any_sync(0xffffffffu, ok && segany[kl] != 0);
+    const int64_t kb = seg0[b], k1 = seg0[b + 1];
+    // 32 segments' predictions and steps, one per lane
+    int pn = -1;
+    FoldStep sn = {0, 0};
+    int an = 0;
+    auto fetch = [&](int64_t k) {
+      pn = k < k1 ? pred[k] : -1;
+      sn = k < k1 ? step[k] : FoldStep{0, 0};
+      an = k < k1 ? segany[k] : 0;
+    };
+    fetch(kb + lane);
+    for (int64_t k0 = kb; k0 < k1; k0 += 32) {
+      const int pl = pn;
+      const FoldStep sl = sn;
+      touched = touched || __any_sync(0xffffffffu, an != 0);
+      fetch(k0 + 32 + lane);
       const int cnt = (int)min((int64_t)32, k1 - k0);
-      for (int j = 0; j < cnt; j++) {
-        const int pj = __shfl_sync(0xffffffffu, pl, j);
-        FoldStep sj;
-        sj.g0 = __shfl_sync(0xffffffffu, sl.g0, j);
-        sj.g1 = __shfl_sync(0xffffffffu, sl.g1, j);
+      // segments after which another binade is predicted: the fold leaves
+      // its binade in them; the first one's shares are on their way while
+      // those before it are taken
+      int after = __shfl_down_sync(0xffffffffu, pl, 1);
+      const int next = __shfl_sync(0xffffffffu, pn, 0);
+      if (lane == 31) after = next;
+      unsigned cross = __ballot_sync(0xffffffffu, lane < cnt && after != pl && after >= 0);
+      double v[8];
+      int held = -1;  // the segment v belongs to
+      auto ahead = [&](int j) {
+        cross &= j < 32 ? 0xffffffffu << j : 0u;
+        if (cross) {
+          held = __ffs(cross) - 1;
+          det_seg_shares(kept, col, segs, sh, k0 + held, lane, v);
+        }
+      };
+      ahead(0);
+      for (int j = 0; j < cnt;) {
         const int bu = fold_binade(acc);
-        if (bu == pj) {
-          const int64_t A = fold_apply(sj, fold_int(acc));
-          if (A < kFoldTop) {
-            acc = fold_double(A, bu);
-            continue;
+        // the segments from j on that are predicted in this binade
+        const unsigned same = __ballot_sync(0xffffffffu, lane < cnt && pl == bu) >> j;
+        const int run = same == 0xffffffffu ? 32 : __ffs(~same) - 1;
+        if (run > 0) {
+          const bool in = lane >= j && lane < j + run;
+          FoldStep P = in ? sl : FoldStep{0, 0};
+          if (!__any_sync(0xffffffffu, P.g0 != P.g1)) {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              const int64_t q = __shfl_up_sync(0xffffffffu, P.g0, o);
+              if (lane >= o) P.g0 += q;
+            }
+            P.g1 = P.g0;
+          } else {
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+              FoldStep q;
+              q.g0 = __shfl_up_sync(0xffffffffu, P.g0, o);
+              q.g1 = __shfl_up_sync(0xffffffffu, P.g1, o);
+              if (lane >= o) P = fold_compose(q, P);
+            }
           }
+          const int64_t A = fold_apply(P, fold_int(acc));
+          const unsigned over = __ballot_sync(0xffffffffu, in && A >= kFoldTop);
+          const int t = over ? __ffs(over) - 1 : j + run;
+          if (t > j) acc = fold_double(__shfl_sync(0xffffffffu, A, t - 1), bu);
+          j = t;
+          if (j >= cnt) break;
         }
         // the prediction missed or the segment leaves the binade: fold it
         // element by element
-        const DetSeg S = segs[k0 + j];
-        double v[8];
+        if (held != j) det_seg_shares(kept, col, segs, sh, k0 + j, lane, v);
+        if (acc == 0.0) {
+          // a fold that starts leaves its binade every few of the first
+          // shares, and fold_batch starts again each time: those
+          // by FP64 adds (shares 0 .. 31 are in lanes 0 .. 3)
 #pragma unroll
-        for (int q = 0; q < 8; q++) {
-          const int pos = 8 * lane + q;
-          v[q] = pos < S.len ? sh[col[S.beg + pos]] : 0.0;
+          for (int l = 0; l < 4; l++)
+#pragma unroll
+            for (int q = 0; q < 8; q++) acc = acc + __shfl_sync(0xffffffffu, v[q], l);
+          if (lane < 4)
+#pragma unroll
+            for (int q = 0; q < 8; q++) v[q] = 0.0;
         }
         acc = fold_batch(acc, v, lane);
+        j++;
+        ahead(j);
       }
     }
     if (lane == 0)
@@ -1518,7 +1644,7 @@ struct PushWork {
   DBuf<int32_t> phcnt, phtouch;    // per heavy vertex: items done, any frontier neighbour
   // deterministic pull of big vertices: per segment sum, member flag,
   // predicted binade, composed step
-  DBuf<double> dsum;
+  DBuf<double> dsum, dkept;
   DBuf<int32_t> dany, dpred;
   DBuf<FoldStep> dstep;
   bool pull_ready = false;
@@ -1545,6 +1671,7 @@ struct PushWork {
     seli2.release(ctx);
     selcnt.release(ctx);
     dsum.release(ctx);
+    dkept.release(ctx);
     dany.release(ctx);
     dpred.release(ctx);
     dstep.release(ctx);
@@ -1740,7 +1867,7 @@ struct PushWork {
     cudaStream_t s = ctx->stream;
     const int64_t n = g->n, words = (n + 31) / 32;
     if (!pull_ready) {
-      LGC_TRY(pq.reserve(ctx, words));
+      LGC_TRY(pq.reserve(ctx, words + 1));
       pull_ready = true;
     }
     const int sb = pull_share_bytes(det);
@@ -1803,8 +1930,9 @@ struct PushWork {
       ProfScope ps(ctx, det ? LGC_PROF_DET_EDGE : LGC_PROF_PULL,
                    24.0 * (double)F.edges + 24.0 * nf);
       if (det) {
-        // every gather ORs its qualifying vertices into the cleared bitmap
-        LGC_CUDA_TRY(cudaMemsetAsync(pq.ptr, 0, 4 * words, s));
+        // every gather ORs its qualifying vertices into the cleared bitmap (and
+        // the word after it, the middle gather's slice ticket)
+        LGC_CUDA_TRY(cudaMemsetAsync(pq.ptr, 0, 4 * (words + 1), s));
         const LightView light = g->view(1, kPullLight), mid = g->view(kPullLight + 1, kDetBig);
         if (light.end > light.beg) {
           pull_light_kernel<<<light_grid(ctx, light), kBlock, 0, s>>>(
@@ -1812,8 +1940,9 @@ struct PushWork {
           LGC_COUNT_LAUNCH(ctx);
         }
         if (mid.end > mid.beg) {
-          pull_mid_det_kernel<<<light_grid(ctx, mid), kBlock, 0, s>>>(
-              mid, psh.ptr, D, ct, fmode, pq.ptr, ctx->d_counters);
+          const int mg = (int)min64(ceil_div(mid.threads(), 32), ctx->sms);
+          pull_mid_det_kernel<<<mg, kBlock, 0, s>>>(mid, psh.ptr, D, ct, fmode, pq.ptr,
+                                                    pq.ptr + words, ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
         if (g->nbig > 0) {  // lists longer than kDetBig, folded segment-parallel
@@ -1822,20 +1951,23 @@ struct PushWork {
           LGC_TRY(dpred.reserve(ctx, g->nsegs));
           LGC_TRY(dstep.reserve(ctx, g->nsegs));
           const int sg = (int)std::min<int64_t>(ceil_div(g->nsegs, kBlock / 32), (ctx->sms * 16));
+          const bool keep = g->nsegs <= kDetKeep &&
+                            dkept.reserve(ctx, kDetSeg * g->nsegs) == LGC_OK;
           det_seg_sum_kernel<<<sg, kBlock, 0, s>>>(g->col, g->segs, g->nsegs, psh.ptr, dsum.ptr,
-                                                   dany.ptr);
-          LGC_COUNT_LAUNCH(ctx);
-          det_seg_predict_kernel<<<grid_for(g->nbig), kBlock, 0, s>>>(
-              g->big_w, g->big_seg0, g->nbig, D, dsum.ptr, dpred.ptr);
-          LGC_COUNT_LAUNCH(ctx);
-          det_seg_step_kernel<<<sg, kBlock, 0, s>>>(g->col, g->segs, g->nsegs, psh.ptr, dpred.ptr,
-                                                    dstep.ptr);
+                                                   dany.ptr, keep ? dkept.ptr : nullptr);
           LGC_COUNT_LAUNCH(ctx);
           const int vg = (int)std::min<int64_t>(ceil_div(g->nbig, kBlock / 32), (ctx->sms * 16));
-          det_seg_verify_kernel<<<vg, kBlock, 0, s>>>(g->off, g->col, g->segs, g->big_w,
-                                                      g->big_seg0, g->nbig, psh.ptr, dpred.ptr,
-                                                      dstep.ptr, dany.ptr, D, ct, fmode, pq.ptr,
-                                                      ctx->d_counters);
+          det_seg_predict_kernel<<<vg, kBlock, 0, s>>>(g->big_w, g->big_seg0, g->nbig, D, dsum.ptr,
+                                                       dpred.ptr);
+          LGC_COUNT_LAUNCH(ctx);
+          det_seg_step_kernel<<<sg, kBlock, 0, s>>>(g->col, g->segs, g->nsegs, psh.ptr,
+                                                    keep ? dkept.ptr : nullptr, dpred.ptr,
+                                                    dstep.ptr);
+          LGC_COUNT_LAUNCH(ctx);
+          det_seg_verify_kernel<<<vg, kBlock, 0, s>>>(
+              g->off, g->col, g->segs, g->big_w, g->big_seg0, g->nbig, psh.ptr,
+              keep ? dkept.ptr : nullptr, dpred.ptr, dstep.ptr, dany.ptr, D, ct, fmode, pq.ptr,
+              ctx->d_counters);
           LGC_COUNT_LAUNCH(ctx);
         }
       } else {

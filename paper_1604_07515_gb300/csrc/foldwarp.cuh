@@ -27,31 +27,32 @@ __device__ inline double fold_batch(double acc, const double (&v)[NL], int lane)
   while (start < 32 * NL) {
     const int bu = fold_binade(acc);
     const int64_t A0 = fold_int(acc);
-    FoldStep st[NL];
-    FoldStep F = {0, 0};
+    // the lane's steps from an even and from an odd value
+    int64_t d[NL];
+    uint32_t tie = 0;
+    int64_t x0 = 0, x1 = 1;
 #pragma unroll
     for (int j = 0; j < NL; j++) {
-      st[j] = NL * lane + j >= start ? fold_step(v[j], bu) : FoldStep{0, 0};
-      F = fold_compose(F, st[j]);
+      FoldNear f = fold_near(v[j], bu);
+      if (NL * lane + j < start) f = {0, false};
+      d[j] = f.d;
+      tie |= (uint32_t)f.tie << j;
+      x0 = fold_take(f, x0);
+      x1 = fold_take(f, x1);
     }
-    // exclusive scan over lanes.  A step depends on the value's parity only
-    // where a share lies half way between two values of the binade: without
-    // one among them the compositions are plain sums
-    FoldStep E;
-    bool par = false;
-#pragma unroll
-    for (int j = 0; j < NL; j++) par = par || st[j].g0 != st[j].g1;
-    if (!__any_sync(0xffffffffu, par)) {
-      int64_t P = F.g0;
+    // exclusive scan over lanes.  A step depends on the value's parity only at
+    // a tie: without one among them the compositions are plain sums
+    int64_t A;
+    if (!__any_sync(0xffffffffu, tie != 0)) {
+      int64_t P = x0;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         const int64_t q = __shfl_up_sync(0xffffffffu, P, o);
         if (lane >= o) P += q;
       }
-      P -= F.g0;
-      E = {P, P};
+      A = A0 + (P - x0);
     } else {
-      FoldStep P = F;
+      FoldStep P = {x0, x1 - 1}, E;
 #pragma unroll
       for (int o = 1; o < 32; o <<= 1) {
         FoldStep q;
@@ -62,13 +63,13 @@ __device__ inline double fold_batch(double acc, const double (&v)[NL], int lane)
       E.g0 = __shfl_up_sync(0xffffffffu, P.g0, 1);
       E.g1 = __shfl_up_sync(0xffffffffu, P.g1, 1);
       if (lane == 0) E = {0, 0};
+      A = fold_apply(E, A0);
     }
-    int64_t A = fold_apply(E, A0);
     int cj = -1;
     int64_t before = 0;
 #pragma unroll
     for (int j = 0; j < NL; j++) {
-      const int64_t nx = fold_apply(st[j], A);
+      const int64_t nx = fold_take({d[j], (tie >> j & 1u) != 0}, A);
       if (cj < 0 && nx >= kFoldTop) {
         cj = j;
         before = A;

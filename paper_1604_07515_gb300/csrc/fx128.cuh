@@ -299,27 +299,32 @@ LGC_HD double fold_double(int64_t A, int bu) {
   return fx_from_bits(((uint64_t)(bu - 1) << 52) + (uint64_t)A);
 }
 
-LGC_HD FoldStep fold_step(double s, int bu) {
+// A share's step as the addition of d and, at a tie, the rounding of the sum
+// to even: at a tie f = 1/2 and d = Q + 1, so A + d - 1 and A + d are the two
+// nearest and the even one of them is A + d with its last bit cleared.
+struct FoldNear {
+  int64_t d;
+  bool tie;
+};
+
+LGC_HD FoldNear fold_near(double s, int bu) {
   const uint64_t b = fx_bits(s) & kFxMask;  // -0.0 adds nothing
-  if (b == 0) return {0, 0};
-  const int be = fx_bexp(b);
-  uint64_t m = b & ((1ull << 52) - 1);
-  if (be) m |= 1ull << 52;
-  const int sh = fx_lsb(be) - (bu - 1075);
-  if (sh >= 2) return {kFoldBig, kFoldBig};
-  if (sh >= 0) {
-    const int64_t Q = (int64_t)(m << sh);
-    return {Q, Q};
-  }
-  const int rs = -sh;
-  if (rs >= 64) return {0, 0};  // s < u / 2^10: rounds away
-  const int64_t Q = (int64_t)(m >> rs);
-  const uint64_t R = m & ((1ull << rs) - 1), half = 1ull << (rs - 1);
-  if (R != half) {
-    const int64_t D = Q + (R > half ? 1 : 0);
-    return {D, D};
-  }
-  return {Q + (Q & 1), Q + ((Q + 1) & 1)};
+  const int be = (int)(b >> 52);
+  const uint64_t m = (b & ((1ull << 52) - 1)) | (be ? 1ull << 52 : 0);
+  const int rs = bu - (be > 1 ? be : 1);  // s / u = m / 2^rs
+  // rs >= 54 rounds away, as 63 does
+  const int q = rs < 1 ? 1 : rs > 63 ? 63 : rs;
+  const uint64_t t = m + (1ull << (q - 1));
+  const int64_t d = (int64_t)(t >> q);
+  if (rs >= 1) return {d, t << (64 - q) == 0};
+  return {m == 0 ? 0 : rs < -1 ? kFoldBig : (int64_t)(m << -rs), false};
+}
+
+LGC_HD int64_t fold_take(FoldNear f, int64_t A) { return (A + f.d) & ~(int64_t)f.tie; }
+
+LGC_HD FoldStep fold_step(double s, int bu) {
+  const FoldNear f = fold_near(s, bu);
+  return {fold_take(f, 0), fold_take(f, 1) - 1};
 }
 
 // first a, then b
