@@ -19,10 +19,12 @@
 #include <string.h>
 
 #include <algorithm>
+#include <type_traits>
 #include <vector>
 
 #include "batch.cuh"
 #include "common.cuh"
+#include "edges.cuh"
 #include "prim.cuh"
 
 namespace lgc {
@@ -166,60 +168,55 @@ __device__ inline int batch_find(const int64_t* s_epos, int cnt, int64_t e, int6
   return j;
 }
 
-// edgeMap (atomic mode) over all seeds' edges.  Each thread takes kItemsB
-// edges and runs them through the phases side by side, as the single-seed
-// push does: every item's column, then every item's first probe, then the
-// slots, then all the adds, so that a thread keeps kItemsB independent
-// memory trips in flight instead of walking one edge's chain after another.
-// Keys inserted are counted once per (warp, seed).
+// edgeMap (atomic mode) over all seeds' edges, chunks of up to kChunkTiles
+// tiles of 32 * kItemsB consecutive edges a warp.  A tile's edges go through
+// the phases side by side, as the single-seed push does: every item's column,
+// then every item's first probe, then the slots, then all the adds, so that a
+// thread keeps kItemsB independent memory trips in flight.
+//
+// What bounds it is adds to one address, 2.9 ns each: neighbouring edges
+// belong to one seed, whose hub takes 0.6% of them and whose three counters
+// took an add per warp and appended vertex.  A warp sums the counters and the
+// adds to the graph's hot vertices (HotSet) of the seed it is in, and writes
+// them when its chunk ends or the next seed begins; a tile of several seeds
+// adds everything at once.  Longer chunks would spread the grid over more
+// tables than L2 holds.
+constexpr int kChunkTiles = 16;
+
 __global__ void __launch_bounds__(kBlock)
     batch_emap_kernel(const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
                       const double* __restrict__ share, const int64_t* __restrict__ epos,
                       const int64_t* __restrict__ foff, const int32_t* __restrict__ fseed,
-                      int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev,
+                      int64_t nf, int64_t E_host, const int64_t* __restrict__ E_dev, HotSet H,
                       const Table* __restrict__ tabs, const SeedParam* __restrict__ prm,
                       int32_t* nseed, int32_t* nfv, int32_t* nfs, int32_t ncap, int32_t* gsize,
                       int32_t* gerr, SeedCount* sc) {
-  __shared__ int64_t s_epos[kTileB + 1];
-  __shared__ int64_t s_off[kTileB];
-  __shared__ double s_share[kTileB];
-  __shared__ int32_t s_seed[kTileB];
-  __shared__ int64_t s_i0, s_i1;
+  __shared__ HotShared s_tab;
+  hot_load(H, s_tab);
   const int lane = threadIdx.x & 31;
+  const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   const int64_t E = min(E_host, *E_dev);
-  const int64_t ntiles = (E + kTileB - 1) / kTileB;
-  for (int64_t tile = blockIdx.x; tile < ntiles; tile += gridDim.x) {
-    const int64_t e0 = tile * kTileB, e1 = min(E, e0 + kTileB);
-    const int cntsrc = batch_stage(epos, nf, E, e0, e1, &s_i0, &s_i1, s_epos);
-    const int64_t i0 = s_i0;
-    for (int j = threadIdx.x; j < cntsrc; j += kBlock) {
-      s_off[j] = foff[i0 + j];
-      s_share[j] = share[i0 + j];
-      s_seed[j] = fseed[i0 + j];
-    }
-    __syncthreads();
-    int32_t seed[kItemsB], w[kItemsB];
-    double sh[kItemsB];
-#pragma unroll
-    for (int k = 0; k < kItemsB; k++) {
-      const int64_t e = e0 + k * kBlock + threadIdx.x;
-      int64_t q = 0;
-      const int j = e < e1 ? batch_find(s_epos, cntsrc, e, &q) : -1;
-      seed[k] = -1;
-      w[k] = -1;
-      sh[k] = 0.0;
-      if (j >= 0) {
-        seed[k] = s_seed[j];
-        w[k] = col[s_off[j] + q];
-        sh[k] = s_share[j];
-      }
-    }
+  constexpr int64_t kTileW = 32 * kItemsB;
+  const int64_t chunk =
+      kTileW * max((int64_t)1, min((int64_t)kChunkTiles, E / (kTileW * nwarps)));
+
+  // what the warp holds back of seed cs
+  int32_t cs = -1;
+  HotLane<double> S;
+  int32_t c_ins = 0, c_size = 0;
+  int64_t c_edges = 0;
+
+  // Adds x to the seeds' values of w (-1: nothing), the arrays' entries side
+  // by side; one: all of seed cs.
+  auto push = [&](auto& seed, auto& w, auto& x, bool one) {
+    constexpr int N = std::extent_v<std::remove_reference_t<decltype(w)>>;
     // the item's table: a dense one is the value array and the presence
     // bitmap (slot = vertex), a hashed one its slots and hash shift
-    const Table* tp[kItemsB];
-    int32_t probe[kItemsB];
+    const Table* tp[N];
+    int32_t probe[N];
 #pragma unroll
-    for (int k = 0; k < kItemsB; k++) {
+    for (int k = 0; k < N; k++) {
       probe[k] = 0;
       tp[k] = nullptr;
       if (w[k] >= 0) {
@@ -228,10 +225,10 @@ __global__ void __launch_bounds__(kBlock)
                                 : __ldcg(&tp[k]->s[hash_slot(w[k], tp[k]->shift)].key);
       }
     }
-    int32_t slot[kItemsB];
-    int ins[kItemsB];
+    int32_t slot[N];
+    int ins[N];
 #pragma unroll
-    for (int k = 0; k < kItemsB; k++) {
+    for (int k = 0; k < N; k++) {
       slot[k] = -1;
       ins[k] = 0;
       if (w[k] < 0) continue;
@@ -245,34 +242,123 @@ __global__ void __launch_bounds__(kBlock)
         slot[k] = (int32_t)ht_find_or_insert(*tp[k], w[k], &ins[k], &sc[seed[k]].err);
       }
     }
-    double old[kItemsB];
+    __syncwarp();
+    double old[N];
 #pragma unroll
-    for (int k = 0; k < kItemsB; k++)
-      old[k] = slot[k] >= 0 ? atomicAdd(tb_val(*tp[k], slot[k]), sh[k]) : 0.0;
+    for (int k = 0; k < N; k++)
+      old[k] = slot[k] >= 0 ? atomicAdd(tb_val(*tp[k], slot[k]), x[k]) : 0.0;
+    unsigned m[N];
+    int32_t dw[N];
+    int total = 0;
 #pragma unroll
-    for (int k = 0; k < kItemsB; k++) {
+    for (int k = 0; k < N; k++) {
       bool pred = false;
-      int64_t dw = 0;
+      dw[k] = 0;
       if (slot[k] >= 0) {
-        const double nv = old[k] + sh[k];
+        const double nv = old[k] + x[k];
         const double eps = prm[seed[k]].eps;
-        if (nv >= eps) {  // eps*d(w) >= eps for d(w) >= 1: cheap pre-test
-          dw = deg[w[k]];
-          const double thr = eps * (double)dw;
+        // eps*d(w) >= eps for d(w) >= 1: a pre-test, of the bits (both are
+        // positive, and a comparison is an FP64 instruction)
+        if (__double_as_longlong(nv) >= __double_as_longlong(eps)) {
+          dw[k] = deg[w[k]];
+          const double thr = eps * (double)dw[k];
           pred = old[k] < thr && nv >= thr;
         }
       }
-      // inserted keys, one atomic per (warp, seed)
-      const unsigned im = __ballot_sync(0xffffffffu, ins[k] != 0);
-      if (im) {
-        const unsigned peers = __match_any_sync(0xffffffffu, seed[k]);
-        if (seed[k] >= 0 && lane == __ffs(peers) - 1 && (im & peers))
-          atomicAdd((unsigned long long*)&sc[seed[k]].inserted,
-                    (unsigned long long)__popc(im & peers));
+      __syncwarp();
+      m[k] = __ballot_sync(0xffffffffu, pred);
+      total += __popc(m[k]);
+      if (!pred) dw[k] = 0;
+      if (one) {
+        c_ins += ins[k];
+        c_size += pred;
+        c_edges += dw[k];
+      } else {
+        const unsigned im = __ballot_sync(0xffffffffu, ins[k] != 0);
+        if (im) {  // one atomic per (warp, seed)
+          const unsigned peers = __match_any_sync(0xffffffffu, seed[k]);
+          if (seed[k] >= 0 && lane == __ffs(peers) - 1 && (im & peers))
+            atomicAdd((unsigned long long*)&sc[seed[k]].inserted,
+                      (unsigned long long)__popc(im & peers));
+        }
+        if (pred) {
+          atomicAdd(&sc[seed[k]].next_size, 1);
+          atomicAdd((unsigned long long*)&sc[seed[k]].next_edges, (unsigned long long)dw[k]);
+        }
       }
-      batch_append(pred, seed[k], w[k], slot[k], dw, nseed, nfv, nfs, ncap, gsize, gerr, sc);
     }
-    __syncthreads();
+    if (total == 0) return;
+    int32_t at = 0;
+    if (lane == 0) at = atomicAdd(gsize, total);
+    at = __shfl_sync(0xffffffffu, at, 0);
+#pragma unroll
+    for (int k = 0; k < N; k++) {
+      if (m[k] >> lane & 1u) {
+        const int32_t pos = at + __popc(m[k] & ((1u << lane) - 1u));
+        if (pos < ncap) {
+          nseed[pos] = seed[k];
+          nfv[pos] = w[k];
+          nfs[pos] = slot[k];
+        } else {
+          atomicOr(gerr, kErrFrontierOverflow);
+        }
+      }
+      at += __popc(m[k]);
+    }
+  };
+  auto flush = [&] {
+    if (cs < 0) return;
+    if (H.tab && __any_sync(0xffffffffu, S.any)) {
+      int32_t seed[1] = {cs}, w[1] = {S.any ? H.ids[lane] : -1};
+      double x[1] = {S.a};
+      push(seed, w, x, true);
+      S = {};
+    }
+    c_ins = __reduce_add_sync(0xffffffffu, c_ins);
+    c_size = __reduce_add_sync(0xffffffffu, c_size);
+    for (int o = 16; o > 0; o >>= 1) c_edges += __shfl_xor_sync(0xffffffffu, c_edges, o);
+    if (lane == 0) {
+      if (c_ins) atomicAdd((unsigned long long*)&sc[cs].inserted, (unsigned long long)c_ins);
+      if (c_size) atomicAdd(&sc[cs].next_size, c_size);
+      if (c_edges) atomicAdd((unsigned long long*)&sc[cs].next_edges, (unsigned long long)c_edges);
+    }
+    c_ins = c_size = 0;
+    c_edges = 0;
+    cs = -1;
+  };
+
+  for (int64_t c0 = warp * chunk; c0 < E; c0 += nwarps * chunk) {
+    EdgeWindow W(
+        max((int64_t)0, warp_upper_bound(epos, nf, c0) - 1), nf,
+        [&](int64_t i) { return epos[i]; }, [&](int64_t i) { return foff[i] - epos[i]; });
+    const int64_t c1 = min(E, c0 + chunk);
+    for (int64_t e0 = c0; e0 < c1; e0 += kTileW) {
+      int32_t seed[kItemsB], w[kItemsB];
+      double x[kItemsB];
+#pragma unroll
+      for (int k = 0; k < kItemsB; k++) {
+        const int64_t eb = e0 + 32 * k;
+        int64_t b = 0;
+        const int64_t i = W.find(eb, &b);
+        const bool in = eb + lane < E;
+        seed[k] = in ? fseed[i] : -1;
+        x[k] = in ? share[i] : 0.0;
+        w[k] = in ? col[b + eb + lane] : -1;
+      }
+      // edge e0 exists
+      const int32_t first = __shfl_sync(0xffffffffu, seed[0], 0);
+      bool same = true;
+#pragma unroll
+      for (int k = 0; k < kItemsB; k++) same = same && (seed[k] < 0 || seed[k] == first);
+      const bool one = __all_sync(0xffffffffu, same);
+      if (!one || first != cs) {
+        flush();
+        if (one) cs = first;
+      }
+      if (one && H.tab) hot_take(H, s_tab, S, w, x);
+      push(seed, w, x, one);
+    }
+    flush();
   }
 }
 
@@ -1029,10 +1115,10 @@ int BatchEngine::round() {
   LGC_TRY(scan_i64(ctx, cnt.ptr, epos.ptr, nf, false, total.ptr));
   if (!det) {
     if (E > 0) {
-      const int64_t tiles = ceil_div(E, kTileB);
+      const int64_t tiles = ceil_div(E, kTileB);  // a block's warps take one each at least
       ProfScope ps(ctx, LGC_PROF_EDGEMAP, 24.0 * (double)E + 28.0 * nf);
       batch_emap_kernel<<<(int)std::min<int64_t>(tiles, (ctx->sms * 16)), kBlock, 0, s>>>(
-          g->col, g->deg, share.ptr, epos.ptr, foff.ptr, Fs.ptr, nf, E, total.ptr, d_tabs.ptr,
+          g->col, g->deg, share.ptr, epos.ptr, foff.ptr, Fs.ptr, nf, E, total.ptr, g->hot, d_tabs.ptr,
           d_prm.ptr, Gs.ptr, Gv.ptr, Gslot.ptr, ncap, gsize, gsize + 1, d_sc.ptr);
       LGC_COUNT_LAUNCH(ctx);
     }
