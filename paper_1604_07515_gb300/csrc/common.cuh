@@ -454,6 +454,8 @@ int64_t pow2_at_least(int64_t x);
 // device-to-host copies run at the link's full speed and a host result does
 // not depend on the context that made it), ordinary heap memory if
 // page-locking fails.  Freed blocks are kept for reuse, up to 4 GB.
+// Batched results of at least this many entries on average are copied one by one.
+constexpr int64_t kDirectCopy = 4096;
 void* host_alloc(size_t bytes);
 void host_free(void* p);
 

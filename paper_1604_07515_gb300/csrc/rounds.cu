@@ -45,9 +45,9 @@
 // sequential fold's, bit for bit.  The owner knows its vertex's final r, so
 // it runs the vertex's next V at once (undone where the launch stops before
 // the round).  On the torus: 125 us a round host-driven, 20.8 us with the
-// buckets counted, placed and scattered in phases and V as another, 13.4 us
-// so (24.4 -> 2.9 ms a call); on a 4096-vertex R-MAT graph, whose hubs get
-// about 900 contributions a round, 10-13 -> 2.2-2.6 ms a call.
+// buckets counted, placed and scattered in phases and V as another, 13 us
+// so (24.4 -> 2.75 ms a call); on a 4096-vertex R-MAT graph, whose hubs get
+// about 900 contributions a round, 9.8 -> 2.04 ms a call.
 //
 // Both modes use that r only grows during an edge phase: the vertices that
 // qualify afterwards are those that already did after V (a vertex left

@@ -882,6 +882,8 @@ int run_sweep_batch(lgc_ctx* ctx, lgc_graph* g, int64_t B, const lgc_svec* const
       // S6
       if ((st = scan_i64(ctx, cut, cut, N, true, nullptr)) != LGC_OK) break;
     }
+    // clusters of some size are copied one by one, each its own prefix
+    const bool direct = N / B >= kDirectCopy;
     // S7, per seed
     if ((st = dalloc_t(ctx, &d_best, B)) || (st = dalloc_t(ctx, &d_bvol, B))) break;
     if (N > 0) {
@@ -895,7 +897,7 @@ int run_sweep_batch(lgc_ctx* ctx, lgc_graph* g, int64_t B, const lgc_svec* const
         st = LGC_ECUDA;
         break;
       }
-      if (!ctx->result_on_device) {
+      if (!ctx->result_on_device && !direct) {
         hord = (int32_t*)host_alloc(4 * N);
         if (!hord) {
           st = LGC_ENOMEM;
@@ -943,11 +945,15 @@ int run_sweep_batch(lgc_ctx* ctx, lgc_graph* g, int64_t B, const lgc_svec* const
       } else {
         box->pub.ids = (int32_t*)host_alloc(4 * (size ? size : 1));
         if (!box->pub.ids) st = LGC_ENOMEM;
-        else if (size) memcpy(box->pub.ids, hord + nbeg[b], 4 * size);
+        else if (size && !direct) memcpy(box->pub.ids, hord + nbeg[b], 4 * size);
+        else if (size && cudaMemcpyAsync(box->pub.ids, order + nbeg[b], 4 * size,
+                                         cudaMemcpyDeviceToHost, s))
+          st = LGC_ECUDA;
       }
-      if (st == LGC_OK) out[b] = &box->pub;
-      else lgc_cluster_free(&box->pub);
+      out[b] = &box->pub;
     }
+    // (also after an error: no copy may be on its way into a cluster that is freed)
+    if (direct && cudaStreamSynchronize(s) && st == LGC_OK) st = LGC_ECUDA;
   } while (0);
   if (st != LGC_OK) {
     for (int64_t b = 0; b < B; b++) {
