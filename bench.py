@@ -558,20 +558,18 @@ PULL_TRAFFIC = {"sources": [
                     (_CSRC + "common.cuh", "// Work item of a pull round", "struct lgc_graph {"),
                     (_CSRC + "common.cuh", "// A pull round handles vertices of degree",
                      "}  // namespace lgc")],
-                "sha256": "d70cee2a7faab3841c6347d5dd646370d3072d1abcb34862fa347cb492d939cc",
+                "sha256": "39c451652469a5bb326c457b81e5d6853ac9229468af08c2db2e1113f13b8f05",
                 # bytes per pull round (light + heavy gather), by "degree bin, edges per
                 # lane per batch, lanes per item, bytes per gathered share"
-                "per_round": {"256,16,32,8": 819.3e6, "256,16,16,8": 819.3e6,
-                              "256,8,16,8": 820.1e6, "256,8,32,16": 995.2e6,
-                              "128,16,32,8": 818.6e6, "128,16,16,8": 818.9e6,
-                              "128,8,16,8": 819.6e6, "64,16,32,8": 806.5e6},
-                # ncu --set full of one heavy gather launch (bin 256, shape (16, 32, 8 B)):
+                "per_round": {"256,16,32,8": 701.4e6, "256,16,16,8": 701.8e6,
+                              "256,8,32,8": 702.2e6, "128,16,32,8": 701.7e6,
+                              "128,8,32,8": 702.2e6},
+                # ncu sections of one heavy gather launch (bin 256, shape (16, 32, 8 B)):
                 # the units that bind it, as fractions of their peaks
                 "heavy_gather_full": {"kernel": "pull_heavy_fx_kernel<16, 32, double>",
-                                      "duration_us": 327.6, "dram_gb": 0.454,
-                                      "dram_frac": 0.175, "lts_throughput_frac": 0.285,
-                                      "l1tex_throughput_frac": 0.756, "issue_active_frac": 0.496,
-                                      "l2_hit_rate": 0.769}}
+                                      "duration_us": 324.0, "dram_gb": 0.450,
+                                      "dram_frac": 0.177, "lts_throughput_frac": 0.675,
+                                      "l1tex_throughput_frac": 0.733, "l2_hit_rate": 0.768}}
 
 
 def sources_sha(stretches):
