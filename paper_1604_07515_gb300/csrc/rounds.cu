@@ -1328,9 +1328,12 @@ __global__ void __launch_bounds__(kRdBlock, 1)
       grid.sync();
       rd_fold(B, D, RdSrc{F.v, F.rank, B.share}, F.touched, nf, Cc, s_mem, false,
               [&](bool ok, int4 ts, double old_v, double acc, double) {
+                // a level without a threshold takes every key the round
+                // created: in HK-PR's empty set, every destination
                 const double th = c * (double)ts.w;
                 uint32_t e;
-                rd_append(B, N, C, ok && old_v < th && acc >= th, ts.x, ts.y, ts.w, &e);
+                rd_append(B, N, C, ok && (!thr || (old_v < th && acc >= th)), ts.x, ts.y, ts.w,
+                          &e);
               });
     } else {
       const RdDest dest = {D, Q.keys[set], c, thr};
