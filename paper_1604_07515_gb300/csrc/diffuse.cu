@@ -2794,8 +2794,9 @@ int run_hkpr(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_hkpr_params* prm, 
     lgc_stats& st = W.st;
     int j = 0;
     while (W.F.size > 0) {
-      if (j + 1 < N && rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, false) &&
-          (!det || eps > 0.0)) {
+      // (forced pull rounds gather whatever their size, in both modes)
+      if (j + 1 < N && ctx->pull_policy != 2 && (!det || eps > 0.0) &&
+          rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, false)) {
         if ((status = ensure_room_ahead(ctx, &P, pcount, W.F.size, g->n, nullptr, nullptr, 0)) !=
             LGC_OK)
           break;
