@@ -458,7 +458,10 @@ int rebuild_pull_lists(lgc_ctx* ctx, lgc_graph* g, int L) {
   g->items = nullptr;
   g->nheavy = g->nitems = 0;
   g->pull_light = L;
-  return build_heavy_list(ctx, g);
+  LGC_TRY(build_heavy_list(ctx, g));
+  // other streams (the request loop's, another context's) read the lists next
+  LGC_CUDA_TRY(cudaStreamSynchronize(ctx->stream));
+  return LGC_OK;
 }
 
 }  // namespace lgc
@@ -1018,6 +1021,9 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     if (st == LGC_OK) st = build_shorts(ctx, g);
     if (st == LGC_OK) st = build_recip(ctx, g);
     if (st == LGC_OK) st = build_hot(ctx, g);
+    // complete before the handle is given out: the request loop and other
+    // contexts read the graph on streams of their own
+    if (st == LGC_OK && cudaStreamSynchronize(s) != cudaSuccess) st = LGC_ECUDA;
   } while (0);
   if (st != LGC_OK) {
     dfree(ctx, g->off);
