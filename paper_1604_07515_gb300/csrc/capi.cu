@@ -429,6 +429,80 @@ int build_hot(lgc_ctx* ctx, lgc_graph* g) {
   return st;
 }
 
+// How many entries name each vertex (into named), the entries not above the
+// one before them (into bad[0], less those that begin a list in
+// names_check_kernel) and those that name no vertex (bad[1]).
+__global__ void names_count_kernel(const int32_t* __restrict__ col, int64_t nnz, int64_t n,
+                                   int32_t* __restrict__ named, unsigned long long* bad) {
+  long long down = 0, off_range = 0;
+  for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < nnz;
+       e += (int64_t)gridDim.x * blockDim.x) {
+    const int32_t u = col[e];
+    if (u < 0 || u >= n) {
+      off_range++;
+      continue;
+    }
+    atomicAdd(&named[u], 1);
+    down += e > 0 && col[e - 1] >= u;
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    down += __shfl_xor_sync(0xffffffffu, down, o);
+    off_range += __shfl_xor_sync(0xffffffffu, off_range, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (down) atomicAdd(&bad[0], (unsigned long long)down);
+    if (off_range) atomicAdd(&bad[1], (unsigned long long)off_range);
+  }
+}
+
+__global__ void names_check_kernel(const int64_t* __restrict__ off,
+                                   const int32_t* __restrict__ col, int64_t nnz,
+                                   const int32_t* __restrict__ deg, int64_t n,
+                                   const int32_t* __restrict__ named, unsigned long long* bad) {
+  long long down = 0, other = 0;
+  for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
+       v += (int64_t)gridDim.x * blockDim.x) {
+    const int64_t o = off[v];
+    other += named[v] != deg[v];
+    if (deg[v] > 0 && o > 0 && o < nnz) down += col[o - 1] >= col[o];
+  }
+  for (int o = 16; o > 0; o >>= 1) {
+    down += __shfl_xor_sync(0xffffffffu, down, o);
+    other += __shfl_xor_sync(0xffffffffu, other, o);
+  }
+  if ((threadIdx.x & 31) == 0) {
+    if (down) atomicAdd(&bad[0], (unsigned long long)-down);
+    if (other) atomicAdd(&bad[1], (unsigned long long)other);
+  }
+}
+
+// Sets g->buckets_fit (left false where there is no room for the counts).
+int check_names(lgc_ctx* ctx, lgc_graph* g) {
+  if (g->nnz > kRdEntries) return LGC_OK;
+  cudaStream_t s = ctx->stream;
+  char* buf = nullptr;
+  if (dalloc_t(ctx, &buf, 16 + 4 * (size_t)g->n) != LGC_OK) return LGC_OK;
+  unsigned long long* bad = (unsigned long long*)buf;
+  int32_t* named = (int32_t*)(buf + 16);
+  bool ok = cudaMemsetAsync(buf, 0, 16 + 4 * (size_t)g->n, s) == cudaSuccess;
+  if (ok && g->nnz > 0) {
+    names_count_kernel<<<std::min(grid_for(g->nnz), 16 * ctx->sms), kBlock, 0, s>>>(
+        g->col, g->nnz, g->n, named, bad);
+    LGC_COUNT_LAUNCH(ctx);
+  }
+  if (ok && g->n > 0) {
+    names_check_kernel<<<std::min(grid_for(g->n), 16 * ctx->sms), kBlock, 0, s>>>(
+        g->off, g->col, g->nnz, g->deg, g->n, named, bad);
+    LGC_COUNT_LAUNCH(ctx);
+  }
+  ok = ok && cudaGetLastError() == cudaSuccess &&
+       cudaMemcpyAsync(ctx->h_scratch, bad, 16, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+  dfree(ctx, buf);
+  if (cudaStreamSynchronize(s) != cudaSuccess || !ok) return LGC_ECUDA;
+  g->buckets_fit = ctx->h_scratch[0] == 0 && ctx->h_scratch[1] == 0;
+  return LGC_OK;
+}
+
 // 1 / d by degree (fp64lite.cuh), 16 bytes a degree.
 __global__ void recip_kernel(Recip* __restrict__ recip, int32_t n) {
   for (int32_t d = blockIdx.x * blockDim.x + threadIdx.x; d < n; d += gridDim.x * blockDim.x)
@@ -1021,6 +1095,7 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     if (st == LGC_OK) st = build_shorts(ctx, g);
     if (st == LGC_OK) st = build_recip(ctx, g);
     if (st == LGC_OK) st = build_hot(ctx, g);
+    if (st == LGC_OK) st = check_names(ctx, g);
     // complete before the handle is given out: the request loop and other
     // contexts read the graph on streams of their own
     if (st == LGC_OK && cudaStreamSynchronize(s) != cudaSuccess) st = LGC_ECUDA;

@@ -320,6 +320,11 @@ struct lgc_graph {
   int32_t recip_n = 0;
   lgc::HotSet hot;
   int2* hot_mem = nullptr;  // its table and ids
+  // every list strictly ascending and every vertex named by as many entries as
+  // it has: what the buckets of the deterministic device rounds rely on.  A
+  // CSR that breaks this (one taken without LGC_GRAPH_VALIDATE) stays with the
+  // host-driven rounds, whose records may be any.
+  bool buckets_fit = false;
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
   // the shape of the atomic pull gathers (tuned): edges per lane per batch,
   // lanes per work item (heavy), bytes per gathered share.  Until tuned, the
@@ -367,6 +372,9 @@ namespace lgc {
 constexpr int kPullLight = 32;  // default of lgc_graph::pull_light; the deterministic bin
 constexpr int kDetBig = 1024;  // longer lists fold segment-parallel in deterministic mode
 constexpr int kDetSeg = 256;
+// Graphs of at most this many entries take deterministic rounds on the device,
+// whose buckets are 4 bytes an entry, allocated by every run (2 GB at most).
+constexpr int64_t kRdEntries = int64_t{1} << 29;
 constexpr int64_t kDetKeep = int64_t{1} << 18;  // segments whose gathered shares are kept (512 MB)
 constexpr int kPullItem = 4096;
 }  // namespace lgc

@@ -34,7 +34,8 @@
 // Deterministic mode has to add each destination's contributions in
 // ascending source order, whatever order the frontier list is in.  Every
 // edge files its pushing entry in its destination's bucket: a destination w
-// gets at most d(w) contributions, so its bucket is the stretch
+// gets at most d(w) contributions, no two from one source (lgc_graph::
+// buckets_fit; other graphs do not come here), so its bucket is the stretch
 // [off[w], off[w] + d(w)) of an array as long as the adjacency and needs no
 // placing; the returned old count of the destination is the edge's place.
 // Then every bucket is put in order and folded by its owner: up to 8
@@ -83,8 +84,6 @@ constexpr int kRdMidWords = 2 * kRdWords + 2 * kRdMid;  // 32-bit words of share
 // bitmap and shares in order.
 constexpr int kRdSmemWords = std::max(kRdWarps * kRdMidWords, 2 * kRdWords + 2 * (int)kRdFront);
 constexpr int kRdSelf = 1 << 30;     // count of a destination listed before its first edge
-// Graphs whose buckets (4 bytes an entry) deterministic rounds allocate.
-constexpr int64_t kRdEntries = int64_t{1} << 29;
 
 // Counters a round adds to.  Round t reads its frontier from set t mod 3 and
 // appends to the next; the third is cleared between the round's barriers
@@ -1366,8 +1365,9 @@ bool rounds_take(const lgc_ctx* ctx, const lgc_graph* g, const RoundsMem& M, int
                  bool det, bool beta) {
   if (!ctx->device_rounds || ctx->trace || nf <= 0 || E > rd_emax(g)) return false;
   if (det) {
-    // every deterministic round is to gather, or no room for the buckets
-    if (ctx->pull_policy == 2 || M.no_det || g->nnz > kRdEntries) return false;
+    // every deterministic round is to gather, or no room for the buckets, or
+    // lists that could overflow them
+    if (ctx->pull_policy == 2 || M.no_det || !g->buckets_fit) return false;
     if (rd_ranks(g) && nf > kRdFront) return false;
   }
   return !beta || nf <= kRdFront;
