@@ -459,35 +459,39 @@ __global__ void names_check_kernel(const int64_t* __restrict__ off,
                                    const int32_t* __restrict__ col, int64_t nnz,
                                    const int32_t* __restrict__ deg, int64_t n,
                                    const int32_t* __restrict__ named, unsigned long long* bad) {
-  long long down = 0, other = 0;
+  long long down = 0, other = 0, sinks = 0;
   for (int64_t v = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x) {
     const int64_t o = off[v];
     other += named[v] != deg[v];
+    sinks += deg[v] == 0 && named[v] > 0;
     if (deg[v] > 0 && o > 0 && o < nnz) down += col[o - 1] >= col[o];
   }
   for (int o = 16; o > 0; o >>= 1) {
     down += __shfl_xor_sync(0xffffffffu, down, o);
     other += __shfl_xor_sync(0xffffffffu, other, o);
+    sinks += __shfl_xor_sync(0xffffffffu, sinks, o);
   }
   if ((threadIdx.x & 31) == 0) {
     if (down) atomicAdd(&bad[0], (unsigned long long)-down);
     if (other) atomicAdd(&bad[1], (unsigned long long)other);
+    if (sinks) atomicAdd(&bad[2], (unsigned long long)sinks);
   }
 }
 
-// Sets g->buckets_fit (left false where there is no room for the counts).
+// Sets g->buckets_fit and g->sinks (left at their cautious values where there
+// is no room for the counts).
 int check_names(lgc_ctx* ctx, lgc_graph* g) {
-  if (g->nnz > kRdEntries) return LGC_OK;
   cudaStream_t s = ctx->stream;
+  const size_t bytes = 32 + 4 * (size_t)g->n;
   char* buf = nullptr;
-  if (dalloc_t(ctx, &buf, 16 + 4 * (size_t)g->n) != LGC_OK) return LGC_OK;
+  if (dalloc_t(ctx, &buf, bytes) != LGC_OK) return LGC_OK;
   unsigned long long* bad = (unsigned long long*)buf;
-  int32_t* named = (int32_t*)(buf + 16);
-  bool ok = cudaMemsetAsync(buf, 0, 16 + 4 * (size_t)g->n, s) == cudaSuccess;
+  int32_t* named = (int32_t*)(buf + 32);
+  bool ok = cudaMemsetAsync(buf, 0, bytes, s) == cudaSuccess;
   if (ok && g->nnz > 0) {
-    names_count_kernel<<<std::min(grid_for(g->nnz), 16 * ctx->sms), kBlock, 0, s>>>(
-        g->col, g->nnz, g->n, named, bad);
+    names_count_kernel<<<(int)std::min<int64_t>((g->nnz + kBlock - 1) / kBlock, 16 * ctx->sms),
+                         kBlock, 0, s>>>(g->col, g->nnz, g->n, named, bad);
     LGC_COUNT_LAUNCH(ctx);
   }
   if (ok && g->n > 0) {
@@ -496,10 +500,11 @@ int check_names(lgc_ctx* ctx, lgc_graph* g) {
     LGC_COUNT_LAUNCH(ctx);
   }
   ok = ok && cudaGetLastError() == cudaSuccess &&
-       cudaMemcpyAsync(ctx->h_scratch, bad, 16, cudaMemcpyDeviceToHost, s) == cudaSuccess;
+       cudaMemcpyAsync(ctx->h_scratch, bad, 24, cudaMemcpyDeviceToHost, s) == cudaSuccess;
   dfree(ctx, buf);
   if (cudaStreamSynchronize(s) != cudaSuccess || !ok) return LGC_ECUDA;
   g->buckets_fit = ctx->h_scratch[0] == 0 && ctx->h_scratch[1] == 0;
+  g->sinks = ctx->h_scratch[2] != 0;
   return LGC_OK;
 }
 

@@ -325,6 +325,9 @@ struct lgc_graph {
   // CSR that breaks this (one taken without LGC_GRAPH_VALIDATE) stays with the
   // host-driven rounds, whose records may be any.
   bool buckets_fit = false;
+  // an entry names a vertex without edges (such a CSR only): a frontier may
+  // hold sources without edges
+  bool sinks = true;
   std::vector<int32_t> hdeg;  // host copy of deg (seeds are checked without a device read)
   // the shape of the atomic pull gathers (tuned): edges per lane per batch,
   // lanes per work item (heavy), bytes per gathered share.  Until tuned, the

@@ -415,6 +415,33 @@ __global__ void __launch_bounds__(kBlock)
   flush_count(nins, &C->inserted);
 }
 
+// Sources without edges (lgc_graph::sinks) behind the others, starting where
+// the edges end (EdgeWindow).  has[i]: cnt[i] > 0; pos: its exclusive prefix
+// sums, *npos in all.
+__global__ void has_edges_kernel(const int64_t* __restrict__ cnt, int64_t nf,
+                                 int64_t* __restrict__ has) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf;
+       i += (int64_t)gridDim.x * blockDim.x)
+    has[i] = cnt[i] > 0;
+}
+__global__ void sinks_last_kernel(int64_t nf, const int64_t* __restrict__ cnt,
+                                  const int64_t* __restrict__ pos,
+                                  const int64_t* __restrict__ npos,
+                                  const int64_t* __restrict__ E_dev,
+                                  const double* __restrict__ share,
+                                  const int64_t* __restrict__ epos,
+                                  const int64_t* __restrict__ foff, double* __restrict__ share_out,
+                                  int64_t* __restrict__ epos_out, int64_t* __restrict__ foff_out) {
+  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < nf;
+       i += (int64_t)gridDim.x * blockDim.x) {
+    const bool any = cnt[i] > 0;
+    const int64_t at = any ? pos[i] : *npos + i - pos[i];
+    share_out[at] = share[i];
+    epos_out[at] = any ? epos[i] : *E_dev;
+    foff_out[at] = foff[i];
+  }
+}
+
 // Filter of a dense set after a bulk push, in ascending vertex order.  The
 // push leaves the presence bits of the keys it created to this pass, which
 // reads the values anyway: a vertex with a value that is not zero is a key
@@ -1656,6 +1683,9 @@ struct PushWork {
   DBuf<unsigned long long> selcnt;
   // device-driven rounds
   RoundsMem rmem;
+  // graphs with sinks: the push's arrays in another order
+  DBuf<double> share2;
+  DBuf<int64_t> epos2, foff2, has;
   DBuf<Recip> recip;  // HK-PR pull rounds: 1 / ((j + 1) d) by degree
   lgc_stats st{};
   explicit PushWork(lgc_ctx* c, lgc_graph* gr) : ctx(c), g(gr) {}
@@ -1676,6 +1706,10 @@ struct PushWork {
     dpred.release(ctx);
     dstep.release(ctx);
     rmem.release(ctx);
+    share2.release(ctx);
+    epos2.release(ctx);
+    foff2.release(ctx);
+    has.release(ctx);
     recip.release(ctx);
     share.release(ctx);
     cnt.release(ctx);
@@ -1742,6 +1776,28 @@ struct PushWork {
     ctx->trace_sizes.push_back(F.size);
   }
 
+  // The push's sources without edges behind the others.
+  int sinks_last() {
+    cudaStream_t s = ctx->stream;
+    const int64_t nf = F.size;
+    LGC_TRY(share2.reserve(ctx, nf));
+    LGC_TRY(epos2.reserve(ctx, nf));
+    LGC_TRY(foff2.reserve(ctx, nf));
+    LGC_TRY(has.reserve(ctx, nf + 1));
+    has_edges_kernel<<<grid_for(nf), kBlock, 0, s>>>(cnt.ptr, nf, has.ptr);
+    LGC_COUNT_LAUNCH(ctx);
+    LGC_TRY(scan_i64(ctx, has.ptr, has.ptr, nf, false, has.ptr + nf));
+    sinks_last_kernel<<<grid_for(nf), kBlock, 0, s>>>(nf, cnt.ptr, has.ptr, has.ptr + nf,
+                                                      total.ptr, share.ptr, epos.ptr, foff.ptr,
+                                                      share2.ptr, epos2.ptr, foff2.ptr);
+    LGC_COUNT_LAUNCH(ctx);
+    LGC_CUDA_TRY(cudaGetLastError());
+    std::swap(share, share2);
+    std::swap(epos, epos2);
+    std::swap(foff, foff2);
+    return LGC_OK;
+  }
+
   // edgeMap + filter into table D.  Records per source are cnt[] (scanned
   // into epos by the caller's vertexMap step).  Returns the counters.
   int edge_phase(const Table& D, double c, int fmode, bool det, bool self_rec, int64_t nrec,
@@ -1752,6 +1808,8 @@ struct PushWork {
     // algorithmic bytes: 24 per pushed edge (col 4, key 4, value read-modify-write 16),
     // 24 per frontier source staged (epos, off, share), 8 per next-frontier entry
     const double alg_bytes = 24.0 * (double)(nrec - (self_rec && det ? nf : 0)) + 24.0 * nf;
+    // (with a record of its own every source has one)
+    if (g->sinks && nrec > 0 && !(self_rec && det)) LGC_TRY(sinks_last());
     if (bulk) {
       if (nrec > 0) {
         int64_t tiles = ceil_div(nrec, kEdgeTile);

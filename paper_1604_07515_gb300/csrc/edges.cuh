@@ -32,7 +32,9 @@ __device__ inline int64_t warp_upper_bound(const int64_t* a, int64_t n, int64_t 
 // starts past an edge, the edge's source is known from the window: a tile of
 // 256 edges of an R-MAT frontier (70 a source) takes one load.
 // start(i), i < nf: the first edge of source i; base(i): its list's start less
-// that.
+// that.  Every source has edges: the OR of find counts those with one first
+// edge once.  Sources without any (lgc_graph::sinks) are put behind the others,
+// all starting at the end, by the caller.
 template <class Start, class Base>
 struct EdgeWindow {
   int64_t j, bj;  // the source the window follows, its base
@@ -75,7 +77,7 @@ struct EdgeWindow {
 // Calls fn(src, at) with each lane's edges e0 + 32 k + lane of a tile of
 // 32 * IT edges: their sources src[k] (-1 past the end) and their places at[k]
 // in the adjacency.  epos: the sources' first edges (exclusive prefix sums of
-// their degrees, all at least 1), foff: their lists' starts.  A tile's first
+// their degrees; EdgeWindow), foff: their lists' starts.  A tile's first
 // source comes from a search.  No shared memory and no block barriers: staging
 // tiles of 1024 edges through shared memory, with a binary search per edge,
 // had the bulk push wait on barriers and shared memory half of the time.

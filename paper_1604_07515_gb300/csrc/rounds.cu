@@ -1363,11 +1363,12 @@ bool rd_ranks(const lgc_graph* g) { return g->max_deg > 32; }
 
 bool rounds_take(const lgc_ctx* ctx, const lgc_graph* g, const RoundsMem& M, int64_t nf, int64_t E,
                  bool det, bool beta) {
-  if (!ctx->device_rounds || ctx->trace || nf <= 0 || E > rd_emax(g)) return false;
+  // (EdgeWindow: every source has edges)
+  if (!ctx->device_rounds || ctx->trace || nf <= 0 || E > rd_emax(g) || g->sinks) return false;
   if (det) {
     // every deterministic round is to gather, or no room for the buckets, or
     // lists that could overflow them
-    if (ctx->pull_policy == 2 || M.no_det || !g->buckets_fit) return false;
+    if (ctx->pull_policy == 2 || M.no_det || !g->buckets_fit || g->nnz > kRdEntries) return false;
     if (rd_ranks(g) && nf > kRdFront) return false;
   }
   return !beta || nf <= kRdFront;

@@ -82,3 +82,43 @@ def test_det_pushes(name):
     finally:
         g.close()
         c.close()
+
+
+def sinks(n, out, deg, seed):
+    """Vertices below `out` point anywhere (vertex 1 to half of all), the others
+    nowhere."""
+    rng = np.random.default_rng(seed)
+    size = rng.integers(1, deg + 1, size=out)
+    size[1] = n // 2
+    return csr([sorted(rng.choice(n, size=int(size[v]), replace=False)) if v < out else []
+                for v in range(n)])
+
+
+@pytest.mark.parametrize("form", [0, 1, 2], ids=["auto", "hashed", "dense"])
+@pytest.mark.parametrize("device", [1, 0])
+@pytest.mark.parametrize("n,out,deg", [(3000, 1500, 8), (4000, 400, 300), (900, 600, 1),
+                                       (2500, 40, 2000)])
+def test_vertices_without_edges(n, out, deg, device, form):
+    """Frontiers in which many vertices in a row have no edges."""
+    off, col = sinks(n, out, deg, n)
+    c = lgc.Context(0)
+    g = lgc.Graph(c, off, col)
+    try:
+        c.set_option(lgc.OPT_PULL, 1)
+        c.set_option(lgc.OPT_DEVICE_ROUNDS, device)
+        c.set_option(lgc.OPT_TABLE_FORM, form)
+        for mode in ("det", "atomic"):
+            for ref, (p, st) in (
+                    (oracle.nibble(off, col, 1, 5, 0.0), lgc.nibble(g, 1, 5, 0.0, mode=mode)),
+                    (oracle.hkpr(off, col, 1, 3.0, 6, 0.0),
+                     lgc.hkpr(g, 1, 3.0, 6, 0.0, mode=mode))):
+                assert (st.rounds, st.pushes, st.pushed_edges) == (ref.rounds, ref.pushes,
+                                                                   ref.pushed_edges)
+                assert np.array_equal(p.idx, ref.idx)
+                if mode == "det":
+                    assert np.array_equal(p.val, ref.val)
+                else:  # at most 6 rounds whose sums of up to `out` terms come in another order
+                    assert np.abs(p.val - ref.val).sum() <= 6 * out * 2.0 ** -53 * ref.val.sum()
+    finally:
+        g.close()
+        c.close()
