@@ -64,14 +64,15 @@ __device__ inline int64_t lookback_warp(const unsigned long long* status, int64_
 }
 
 // ---------------------------------------------------------------------------
-// Ordered compaction of a vertex bitmap in two launches.  The bitmap's words
+// Ordered compaction of a vertex bitmap in two launches (three for graphs of
+// more than 2^24 vertices).  The bitmap's words
 // come from a functor called by whole warps (word(w, in): lane l asks for
 // word w = the warp's first + l, `in` saying whether it has one), so that a
 // filter can compute them on the fly, 32 vertices of a word at a time with
 // one lane each.  words_count_kernel keeps the words and counts the set bits
 // of every tile of kCmpTileWords words; words_write_kernel adds up the counts
-// of the tiles before its own (one L2 round trip for a thread's loads) and
-// hands every set bit's vertex v to out.put(position, v), lane l with bit l
+// of the tiles before its own (up to 2^22 vertices 8 loads a thread) and hands
+// every set bit's vertex v to out.put(position, v), lane l with bit l
 // of one word after another, so a warp's positions are consecutive.  put
 // returns a weight, and out.finish(entries so far, is this the last tile,
 // weight of the block's vertices) is called by one thread per tile.
@@ -84,6 +85,14 @@ __device__ inline int64_t lookback_warp(const unsigned long long* status, int64_
 // ---------------------------------------------------------------------------
 constexpr int kCmpWarpWords = 8;  // words a warp writes: one batch of loads each
 constexpr int64_t kCmpTileWords = kCmpWarpWords * (kBlock / 32);
+// More tiles than kCmpPlain have their counts added up in groups of kCmpGroup
+// first: adding those of all tiles before one's own is quadratic, nothing at
+// 2^22 vertices but most of the pass from 2^26 on.  Both launches together, a
+// 16th and half of the words not empty: 2^22 vertices 15 and 17 us (19 and 21
+// with groups), 2^24 37 and 44 (37 and 44), 2^25 78 and 91 (66 and 78), 2^26
+// 185 and 199 (119 and 138), 2^28 1565 and 1669 (443 and 543).
+constexpr int kCmpGroup = 1024;
+constexpr int64_t kCmpPlain = 8192;
 
 template <class WordFn>
 __global__ void __launch_bounds__(kBlock)
@@ -117,7 +126,7 @@ __global__ void __launch_bounds__(kBlock)
 template <class Out>
 __global__ void __launch_bounds__(kBlock)
     words_write_kernel(const uint32_t* __restrict__ kept, int64_t words,
-                       const int32_t* __restrict__ cnt, Out out) {
+                       const int32_t* __restrict__ cnt, const int64_t* __restrict__ grp, Out out) {
   __shared__ int64_t s_pre[kBlock / 32];
   __shared__ int s_wtot[kBlock / 32];
   __shared__ int64_t s_sum[kBlock / 32];
@@ -126,7 +135,9 @@ __global__ void __launch_bounds__(kBlock)
   const int64_t wbase = tile * kCmpTileWords + warp * kCmpWarpWords;
   const uint32_t q = lane < kCmpWarpWords && wbase + lane < words ? kept[wbase + lane] : 0u;
   int64_t p = 0;
-  for (int64_t i = threadIdx.x; i < tile; i += kBlock) p += cnt[i];
+  const int64_t whole = grp ? tile / kCmpGroup : 0;  // groups before the tile's own
+  for (int64_t i = threadIdx.x; i < whole; i += kBlock) p += grp[i];
+  for (int64_t i = whole * kCmpGroup + threadIdx.x; i < tile; i += kBlock) p += cnt[i];
   for (int o = 16; o > 0; o >>= 1) p += __shfl_xor_sync(0xffffffffu, p, o);
   const int c = __popc(q);
   int pre = c;  // set bits of the warp's words before this lane's
@@ -221,7 +232,9 @@ struct FrontierOut {
 
 // The two launches on the context's scratch; bits: the words themselves where
 // word only reads them (nothing is kept then), else nullptr.
-int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt);
+int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt, int64_t** grp);
+// grp[b] = the sum of cnt[b * kCmpGroup ...] (kCmpGroup of them, or what is left).
+int tile_groups(lgc_ctx* ctx, const int32_t* cnt, int64_t ntiles, int64_t* grp);
 
 template <class WordFn, class Out>
 int words_compact(lgc_ctx* ctx, const WordFn& word, const uint32_t* bits, int64_t words,
@@ -230,11 +243,15 @@ int words_compact(lgc_ctx* ctx, const WordFn& word, const uint32_t* bits, int64_
   const unsigned ntiles = (unsigned)((words + kCmpTileWords - 1) / kCmpTileWords);
   uint32_t* kept;
   int32_t* cnt;
-  LGC_TRY(cmp_reserve(ctx, words, &kept, &cnt));
+  int64_t* grp;
+  LGC_TRY(cmp_reserve(ctx, words, &kept, &cnt, &grp));
   words_count_kernel<WordFn><<<ntiles, kBlock, 0, ctx->stream>>>(word, words,
                                                                  bits ? nullptr : kept, cnt);
   LGC_COUNT_LAUNCH(ctx);
-  words_write_kernel<Out><<<ntiles, kBlock, 0, ctx->stream>>>(bits ? bits : kept, words, cnt, out);
+  const bool groups = ntiles > kCmpPlain;
+  if (groups) LGC_TRY(tile_groups(ctx, cnt, ntiles, grp));
+  words_write_kernel<Out><<<ntiles, kBlock, 0, ctx->stream>>>(bits ? bits : kept, words, cnt,
+                                                              groups ? grp : nullptr, out);
   LGC_COUNT_LAUNCH(ctx);
   return cudaGetLastError() == cudaSuccess ? LGC_OK : LGC_ECUDA;
 }

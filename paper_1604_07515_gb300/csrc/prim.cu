@@ -776,18 +776,47 @@ int radix_sort_u32(lgc_ctx* ctx, uint32_t* keys, uint32_t* keys_tmp, int64_t n, 
                                             (int32_t*)nullptr, n, bits);
 }
 
-int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt) {
+int cmp_reserve(lgc_ctx* ctx, int64_t words, uint32_t** kept, int32_t** cnt, int64_t** grp) {
   const int64_t ntiles = ceil_div(words, kCmpTileWords);
-  if (words + ntiles > ctx->cmp_cap) {
+  const int64_t at = (words + ntiles + 1) & ~int64_t{1};  // the groups: 8-byte aligned
+  const int64_t need = at + 2 * ceil_div(ntiles, kCmpGroup);
+  if (need > ctx->cmp_cap) {
     dfree(ctx, ctx->cmp);
     ctx->cmp = nullptr;
     ctx->cmp_cap = 0;
-    LGC_TRY(dalloc_t(ctx, &ctx->cmp, (size_t)(words + ntiles)));
-    ctx->cmp_cap = words + ntiles;
+    LGC_TRY(dalloc_t(ctx, &ctx->cmp, (size_t)need));
+    ctx->cmp_cap = need;
   }
   *kept = ctx->cmp;
   *cnt = reinterpret_cast<int32_t*>(ctx->cmp + words);
+  *grp = reinterpret_cast<int64_t*>(ctx->cmp + at);
   return LGC_OK;
+}
+
+namespace {
+__global__ void __launch_bounds__(kBlock)
+    tile_groups_kernel(const int32_t* __restrict__ cnt, int64_t ntiles,
+                       int64_t* __restrict__ grp) {
+  __shared__ int64_t s_sum[kBlock / 32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int64_t t0 = (int64_t)blockIdx.x * kCmpGroup, t1 = min(ntiles, t0 + kCmpGroup);
+  int64_t x = 0;
+  for (int64_t i = t0 + threadIdx.x; i < t1; i += kBlock) x += cnt[i];
+  for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+  if (lane == 0) s_sum[warp] = x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    for (int w = 1; w < kBlock / 32; w++) x += s_sum[w];
+    grp[blockIdx.x] = x;
+  }
+}
+}  // namespace
+
+int tile_groups(lgc_ctx* ctx, const int32_t* cnt, int64_t ntiles, int64_t* grp) {
+  tile_groups_kernel<<<(unsigned)ceil_div(ntiles, kCmpGroup), kBlock, 0, ctx->stream>>>(
+      cnt, ntiles, grp);
+  LGC_COUNT_LAUNCH(ctx);
+  return cudaGetLastError() == cudaSuccess ? LGC_OK : LGC_ECUDA;
 }
 
 namespace {
