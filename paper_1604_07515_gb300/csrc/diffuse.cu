@@ -1636,6 +1636,22 @@ constexpr int64_t kDenseSmall = int64_t{1} << 20;
 // Keys a table has room for ahead of the device-driven rounds.
 constexpr int64_t kRoomKeys = 16384;
 
+// Slots of a hashed table for device-driven rounds that has to take `need`
+// keys: room for `times` as many, so that the rounds to come fit as well, up
+// to `limit` slots, beyond that for twice as many.  Room is cleared (24 bytes
+// a slot, as much again in per-slot sums, three fresh sets a launch) and read
+// through at the end; too little costs a launch and a rehash, 50 us.  Calls on
+// R-MAT graphs, us, without limits and with these: Nibble 2^22 vertices, eps
+// 1e-7 581 and 513, 2^24, 1e-6 504 and 383, 2^26, 1e-7 669 and 750; PR-Nibble
+// 2^22, 3e-7 315 and 317 (2^20 slots: 353), 2^24, 1e-7 405 and 427, 2^26, 1e-7
+// 720 and 524; HK-PR 2^24, 1e-6 615 and 569, 2^26, 1e-7 2535 and 2237.
+constexpr int64_t kRoomKept = int64_t{1} << 22;
+constexpr int64_t kRoomFresh = int64_t{1} << 20;
+int64_t room_slots(int64_t need, int64_t n, int64_t times, int64_t limit) {
+  const int64_t ahead = pow2_at_least(2 * min64(n, std::max<int64_t>(times * need, kRoomKeys)));
+  return min64(ahead, std::max(limit, pow2_at_least(2 * min64(n, 2 * need))));
+}
+
 bool dense_small(const lgc_ctx* ctx, int64_t n) {
   return ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
 }
@@ -2113,11 +2129,11 @@ struct PushWork {
     cudaStream_t s = ctx->stream;
     *done = 0;
     *over = false;
-    // fresh sets with room for 8 times this round's keys, in the smaller form
+    // fresh sets with room for more than this round's keys, in the smaller form
     // (a round that would not fit returns to the host, which comes back with
     // bigger ones); dense ones where they are cheap to clear
     const int64_t n = g->n, need = std::min<int64_t>(n, F.size + F.edges);
-    const int64_t cap = pow2_at_least(2 * std::min<int64_t>(n, std::max<int64_t>(kRoomKeys, 8 * need)));
+    const int64_t cap = room_slots(need, n, 8, kRoomFresh);
     const bool dense = want_dense(ctx, need, n) || dense_small(ctx, n) ||
                        (ctx->table_form == 0 && n >= 1024 && 16 * cap >= 8 * n + n / 8);
     Table T[4];
@@ -2303,16 +2319,15 @@ int ensure_capacity(lgc_ctx* ctx, Table* T, int64_t count, int64_t add, int64_t 
 }
 
 // Before device-driven rounds: as ensure_capacity for the next round, with
-// room for 16 times its keys (a hashed table that would take more memory
-// than the dense form becomes dense).
+// room ahead (room_slots; a hashed table that would take more memory than the
+// dense form becomes dense).
 int ensure_room_ahead(lgc_ctx* ctx, Table* T, int64_t count, int64_t add, int64_t n,
                       const int32_t* fv, int32_t* fs, int64_t nf) {
   if (T->dense) return LGC_OK;
   const int64_t need = min64(count + add, n);
   if (want_dense(ctx, need, n) || dense_small(ctx, n)) return table_to_dense(ctx, T, n, fv, fs, nf);
   if (2 * need <= T->cap) return LGC_OK;
-  const int64_t room = min64(n, std::max<int64_t>(16 * need, kRoomKeys));
-  const int64_t cap = pow2_at_least(2 * room);
+  const int64_t cap = room_slots(need, n, 16, kRoomKept);
   if (ctx->table_form == 0 && n >= 1024 && 24 * cap >= 16 * n + n / 8)
     return table_to_dense(ctx, T, n, fv, fs, nf);
   return table_grow(ctx, T, cap, fv, fs, nf);
