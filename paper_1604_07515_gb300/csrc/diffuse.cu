@@ -1631,7 +1631,9 @@ int light_grid(const lgc_ctx* ctx, const LightView& V) {
 
 // Sets of a graph of up to kDenseSmall vertices are dense from the start
 // (automatic form): clearing 16 bytes a vertex costs 4 us at that size,
-// growing and converting a table on the way 40 us and more.
+// growing and converting a table on the way 40 us and more.  For contexts that
+// run device rounds: the request loop's workers, many at once, take memory as
+// their requests were admitted by (request_bytes), from small tables up.
 constexpr int64_t kDenseSmall = int64_t{1} << 20;
 // Keys a table has room for ahead of the device-driven rounds.
 constexpr int64_t kRoomKeys = 16384;
@@ -1653,7 +1655,7 @@ int64_t room_slots(int64_t need, int64_t n, int64_t times, int64_t limit) {
 }
 
 bool dense_small(const lgc_ctx* ctx, int64_t n) {
-  return ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
+  return ctx->device_rounds && ctx->table_form == 0 && n >= 1024 && n <= kDenseSmall;
 }
 
 struct Frontier {
@@ -2616,7 +2618,9 @@ int run_prnibble_set(lgc_ctx* ctx, lgc_graph* g, int64_t k, const int32_t* seeds
   PushWork W(ctx, g);
   Table T;
   if (dense_small(ctx, g->n)) LGC_TRY(table_create_dense(ctx, &T, g->n, true));
-  else LGC_TRY(table_create(ctx, &T, 2 * std::max<int64_t>(k + dsum, kRoomKeys), true));
+  else
+    LGC_TRY(table_create(
+        ctx, &T, 2 * std::max<int64_t>(k + dsum, ctx->device_rounds ? kRoomKeys : 0), true));
   int64_t count = k;  // keys in T
   int status = LGC_OK;
   int32_t* d_x = nullptr;
