@@ -5,6 +5,7 @@
 
 #include <algorithm>
 #include <atomic>
+#include <memory>
 #include <new>
 
 #include "batch.cuh"
@@ -363,8 +364,8 @@ int build_hot(lgc_ctx* ctx, lgc_graph* g) {
   if (g->max_deg < kHotDeg) return LGC_OK;
   cudaStream_t s = ctx->stream;
   const int grid = std::min(grid_for(g->n), 4 * ctx->sms);
-  char* buf = nullptr;
-  LGC_TRY(dalloc_t(ctx, &buf, 512 + sizeof(int2) * kMostHot));
+  char* buf = nullptr;  // without memory for it or the table: no combining
+  if (dalloc_t(ctx, &buf, 512 + sizeof(int2) * kMostHot) != LGC_OK) return LGC_OK;
   int st = LGC_OK;
   do {
     unsigned long long len[33];
@@ -385,14 +386,15 @@ int build_hot(lgc_ctx* ctx, lgc_graph* g) {
     degree_list_kernel<<<grid, kBlock, 0, s>>>(g->deg, g->n, (int32_t)1 << (b - 1), list, kMostHot,
                                                count);
     LGC_COUNT_LAUNCH(ctx);
-    std::vector<int2> h((size_t)many);
-    if (cudaMemcpyAsync(h.data(), list, sizeof(int2) * many, cudaMemcpyDeviceToHost, s) ||
+    const std::unique_ptr<int2[]> h(new (std::nothrow) int2[(size_t)many]);
+    if (!h) break;
+    if (cudaMemcpyAsync(h.get(), list, sizeof(int2) * many, cudaMemcpyDeviceToHost, s) ||
         cudaStreamSynchronize(s)) {
       st = LGC_ECUDA;
       break;
     }
-    const size_t k = std::min<size_t>(h.size(), kHot);
-    std::partial_sort(h.begin(), h.begin() + k, h.end(), [](const int2& x, const int2& y) {
+    const size_t k = std::min<size_t>((size_t)many, kHot);
+    std::partial_sort(h.get(), h.get() + k, h.get() + many, [](const int2& x, const int2& y) {
       return x.x > y.x || (x.x == y.x && x.y < y.y);
     });
     // a multiplier under which no two of them share an entry: one in eight
@@ -414,7 +416,7 @@ int build_hot(lgc_ctx* ctx, lgc_graph* g) {
     }
     if (!ok) break;  // no combining: speed only
     for (int i = 0; i < kHot; i++) ids[i] = i < (int)k ? h[i].y : -1;
-    if ((st = dalloc_t(ctx, &g->hot_mem, kHotTab + kHot)) != LGC_OK) break;
+    if (dalloc_t(ctx, &g->hot_mem, kHotTab + kHot) != LGC_OK) break;
     if (cudaMemcpyAsync(g->hot_mem, tab, sizeof tab, cudaMemcpyHostToDevice, s) ||
         cudaMemcpyAsync(g->hot_mem + kHotTab, ids, sizeof ids, cudaMemcpyHostToDevice, s) ||
         cudaStreamSynchronize(s)) {
@@ -516,7 +518,7 @@ __global__ void recip_kernel(Recip* __restrict__ recip, int32_t n) {
 
 int build_recip(lgc_ctx* ctx, lgc_graph* g) {
   const int32_t n = (int32_t)std::min<int64_t>((int64_t)g->max_deg + 1, kRecipMax);
-  LGC_TRY(dalloc_t(ctx, &g->recip, (size_t)n));
+  if (dalloc_t(ctx, &g->recip, (size_t)n) != LGC_OK) return LGC_OK;  // divisions then
   recip_kernel<<<std::min(grid_for(n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(g->recip, n);
   LGC_COUNT_LAUNCH(ctx);
   LGC_CUDA_TRY(cudaGetLastError());

@@ -1650,8 +1650,11 @@ constexpr int64_t kRoomKeys = 16384;
 constexpr int64_t kRoomKept = int64_t{1} << 22;
 constexpr int64_t kRoomFresh = int64_t{1} << 20;
 int64_t room_slots(int64_t need, int64_t n, int64_t times, int64_t limit) {
+  constexpr int64_t kMostSlots = int64_t{1} << 31;  // of any table
+  const int64_t least = pow2_at_least(2 * min64(n, need));
   const int64_t ahead = pow2_at_least(2 * min64(n, std::max<int64_t>(times * need, kRoomKeys)));
-  return min64(ahead, std::max(limit, pow2_at_least(2 * min64(n, 2 * need))));
+  const int64_t twice = pow2_at_least(2 * min64(n, 2 * need));
+  return std::max(least, min64(kMostSlots, min64(ahead, std::max(limit, twice))));
 }
 
 bool dense_small(const lgc_ctx* ctx, int64_t n) {
@@ -2148,6 +2151,10 @@ struct PushWork {
       st_ = rounds_fresh(ctx, g, rmem, q, T, P, pcount ? *pcount : 0, F.v.ptr, F.s.ptr, F.size,
                          F.edges, det, pull_min(), rounds_left, key_limit(T[0]),
                          P ? key_limit(*P) : 0, &o);
+    else if (st_ == LGC_ENOMEM) {  // no room for the sets: the rounds stay on the host
+      rmem.give_up(ctx);
+      st_ = LGC_OK;
+    }
     if (st_ != LGC_OK || o.rounds == 0) {
       for (int k = 0; k < 3; k++) table_destroy(ctx, &T[k]);
       return st_;
@@ -2509,9 +2516,12 @@ int prnibble_rounds(lgc_ctx* ctx, lgc_graph* g, PushWork& W, Table& T, int64_t& 
     if (rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, beta < 1.0)) {
       // room for the rounds to come: the set grows with them, and a table
       // that fills up costs another launch
-      if ((status = ensure_room_ahead(ctx, &T, count, W.F.edges, g->n, W.F.v.ptr, W.F.s.ptr,
-                                      W.F.size)) != LGC_OK)
-        return status;
+      status = ensure_room_ahead(ctx, &T, count, W.F.edges, g->n, W.F.v.ptr, W.F.s.ptr, W.F.size);
+      if (status == LGC_ENOMEM) {  // no room ahead: host rounds, which take less
+        W.rmem.give_up(ctx);
+        continue;
+      }
+      if (status != LGC_OK) return status;
       status = W.device_rounds_prnibble(T, &count, alpha, cs, cn, eps, prm->rule, det, beta,
                                         max_rounds - st.rounds);
       if (status != LGC_OK) return status;
@@ -2617,10 +2627,13 @@ int run_prnibble_set(lgc_ctx* ctx, lgc_graph* g, int64_t k, const int32_t* seeds
 
   PushWork W(ctx, g);
   Table T;
-  if (dense_small(ctx, g->n)) LGC_TRY(table_create_dense(ctx, &T, g->n, true));
-  else
-    LGC_TRY(table_create(
-        ctx, &T, 2 * std::max<int64_t>(k + dsum, ctx->device_rounds ? kRoomKeys : 0), true));
+  // with room ahead for device rounds, without where there is no memory for it
+  int made = LGC_ENOMEM;
+  if (dense_small(ctx, g->n)) made = table_create_dense(ctx, &T, g->n, true);
+  if (made == LGC_ENOMEM && ctx->device_rounds)
+    made = table_create(ctx, &T, 2 * std::max<int64_t>(k + dsum, kRoomKeys), true);
+  if (made == LGC_ENOMEM) made = table_create(ctx, &T, 2 * (k + dsum), true);
+  LGC_TRY(made);
   int64_t count = k;  // keys in T
   int status = LGC_OK;
   int32_t* d_x = nullptr;
@@ -2874,9 +2887,12 @@ int run_hkpr(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_hkpr_params* prm, 
       // (forced pull rounds gather whatever their size, in both modes)
       if (j + 1 < N && ctx->pull_policy != 2 && (!det || eps > 0.0) &&
           rounds_take(ctx, g, W.rmem, W.F.size, W.F.edges, det, false)) {
-        if ((status = ensure_room_ahead(ctx, &P, pcount, W.F.size, g->n, nullptr, nullptr, 0)) !=
-            LGC_OK)
-          break;
+        status = ensure_room_ahead(ctx, &P, pcount, W.F.size, g->n, nullptr, nullptr, 0);
+        if (status == LGC_ENOMEM) {
+          W.rmem.give_up(ctx);
+          continue;
+        }
+        if (status != LGC_OK) break;
         int64_t done = 0, rcount = 0;
         bool over = false;
         RoundsFresh q;
@@ -2914,10 +2930,10 @@ int run_hkpr(lgc_ctx* ctx, lgc_graph* g, int32_t x, const lgc_hkpr_params* prm, 
         // one reciprocal per degree in place of a division per vertex, where
         // there are more vertices than degrees (b = (j + 1) d is exact and
         // within div_by's range)
-        const int32_t tab_n =
+        int32_t tab_n =
             nf >= 4 * (int64_t)g->max_deg && j < (1 << 16) ? std::min(g->max_deg + 1, kRecipMax) : 0;
+        if (tab_n > 0 && W.recip.reserve(ctx, tab_n) != LGC_OK) tab_n = 0;
         if (tab_n > 0) {
-          if ((status = W.recip.reserve(ctx, tab_n)) != LGC_OK) break;
           recip_level_kernel<<<std::min(grid_for(tab_n), 4 * ctx->sms), kBlock, 0, ctx->stream>>>(
               W.recip.ptr, tab_n, last ? 1.0 : (double)(j + 1));
           LGC_COUNT_LAUNCH(ctx);

@@ -1364,11 +1364,12 @@ bool rd_ranks(const lgc_graph* g) { return g->max_deg > 32; }
 bool rounds_take(const lgc_ctx* ctx, const lgc_graph* g, const RoundsMem& M, int64_t nf, int64_t E,
                  bool det, bool beta) {
   // (EdgeWindow: every source has edges)
-  if (!ctx->device_rounds || ctx->trace || nf <= 0 || E > rd_emax(g) || g->sinks) return false;
+  if (!ctx->device_rounds || ctx->trace || nf <= 0 || E > rd_emax(g) || g->sinks || M.no_room)
+    return false;
   if (det) {
-    // every deterministic round is to gather, or no room for the buckets, or
-    // lists that could overflow them
-    if (ctx->pull_policy == 2 || M.no_det || !g->buckets_fit || g->nnz > kRdEntries) return false;
+    // every deterministic round is to gather, or lists that could overflow the
+    // buckets
+    if (ctx->pull_policy == 2 || !g->buckets_fit || g->nnz > kRdEntries) return false;
     if (rd_ranks(g) && nf > kRdFront) return false;
   }
   return !beta || nf <= kRdFront;
@@ -1383,7 +1384,7 @@ struct RdLaunch {
 };
 
 // fresh_keys: room for the key lists of fresh sets (else null); levels: room
-// for that many thresholds (device) in *levels.  no_room set: M.no_det is.
+// for that many thresholds (device) in *levels.  *no_room: M has given up.
 int rd_prepare(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, int64_t slots, const int32_t* fv,
                const int32_t* fs, int64_t nf, bool det, bool sel, bool staged, int64_t x_min,
                int64_t max_rounds, int64_t key_limit, int32_t** fresh_keys, int64_t levels,
@@ -1397,14 +1398,18 @@ int rd_prepare(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, int64_t slots, const in
   // a next frontier has at most nf + E entries, all distinct
   const int64_t fcap = std::min<int64_t>(g->n, 2 * kRdEdges);
   const int64_t f_max = sel || (det && rd_ranks(g)) ? std::min<int64_t>(kRdFront, fcap) : fcap;
-  // the buckets first: without room for them the rounds stay on the host
-  if (det && !M.bucket) {
-    if (dalloc_t(ctx, &M.bucket, (size_t)g->nnz) != LGC_OK) {
-      M.bucket = nullptr;
-      M.no_det = true;
+  // without room for all of it the rounds stay on the host
+  auto take = [&](auto** p, size_t count) {
+    const int st = dalloc_t(ctx, p, count);
+    if (st == LGC_ENOMEM) {
+      M.give_up(ctx);
       *no_room = true;
-      return LGC_OK;
     }
+    return st;
+  };
+  if (det && !M.bucket) {
+    const int st = take(&M.bucket, (size_t)g->nnz);
+    if (st != LGC_OK) return *no_room ? LGC_OK : st;
   }
   const int64_t tiles = e_max / 32 + 1;
   // carve one slab; staged: a V phase writes the shares (else the entries' owners)
@@ -1449,7 +1454,8 @@ int rd_prepare(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, int64_t slots, const in
     dfree(ctx, M.slab);
     M.slab = nullptr;
     M.slab_bytes = 0;
-    LGC_TRY(dalloc_t(ctx, &M.slab, at));
+    const int st = take(&M.slab, at);
+    if (st != LGC_OK) return *no_room ? LGC_OK : st;
     M.slab_bytes = at;
   }
   base = M.slab;
@@ -1463,7 +1469,8 @@ int rd_prepare(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, int64_t slots, const in
       M.per_slot = nullptr;
       M.slots = 0;
       const size_t bytes = (4 + (wide ? sizeof(Fx) : 0)) * (size_t)slots;
-      LGC_TRY(dalloc_t(ctx, &M.per_slot, bytes));
+      const int st = take(&M.per_slot, bytes);
+      if (st != LGC_OK) return *no_room ? LGC_OK : st;
       M.slots = slots;
       LGC_CUDA_TRY(cudaMemsetAsync(M.per_slot, 0, bytes, s));
     }

@@ -9,19 +9,24 @@ namespace lgc {
 // slab for the frontier buffers and lists, the per-slot counters of
 // deterministic rounds or counters and sums of wide atomic rounds (zero
 // between launches; a run keeps one mode), and the deterministic rounds'
-// buckets (4 bytes per adjacency entry; no_det: there was no room for them).
+// buckets (4 bytes per adjacency entry).  no_room: there was no device memory
+// for one of them; the run's rounds stay on the host.
 struct RoundsMem {
   char* slab = nullptr;
   size_t slab_bytes = 0;
   char* per_slot = nullptr;
   int64_t slots = 0;
   int32_t* bucket = nullptr;
-  bool no_det = false;
+  bool no_room = false;
   void release(lgc_ctx* ctx) {
     dfree(ctx, slab);
     dfree(ctx, per_slot);
     dfree(ctx, bucket);
     *this = RoundsMem();
+  }
+  void give_up(lgc_ctx* ctx) {
+    release(ctx);
+    no_room = true;
   }
 };
 
@@ -45,7 +50,7 @@ bool rounds_take(const lgc_ctx* ctx, const lgc_graph* g, const RoundsMem& M, int
 // round is not one for the device; runs at least one round when rounds_take
 // holds, count + E is within key_limit and max_rounds > 0.  Atomic rounds of
 // x_min edges or more sum as pull rounds do.  rounds 0 in *out: there was no
-// room (M.no_det is set), nothing has changed.
+// room (M.no_room is set), nothing has changed.
 int rounds_prnibble(lgc_ctx* ctx, lgc_graph* g, RoundsMem& M, const Table& T, const int32_t* fv,
                     const int32_t* fs, int64_t nf, int64_t E, int64_t count, double alpha,
                     double cs, double cn, double eps, int rule, bool det, double beta,
