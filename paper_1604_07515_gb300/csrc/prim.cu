@@ -3,6 +3,7 @@
 
 #include "lookback.cuh"
 #include "prim.cuh"
+#include "ranksort.cuh"
 
 namespace lgc {
 
@@ -593,7 +594,6 @@ unsigned long long* lb_counter(lgc_ctx* ctx) { return ctx->sort_aux + 8 * kRadix
 // 64-bit keys.  Entries before the block's own count where their key is not
 // larger and those behind where it is smaller, so equal keys keep their order.
 constexpr int kRankItems = 16;
-constexpr int64_t kRankWork = 50 << 20;  // comparisons per digit pass spared
 
 template <class K, class V>
 __global__ void __launch_bounds__(kBlock)
@@ -697,11 +697,8 @@ int radix_sort_impl(lgc_ctx* ctx, K* keys, V* vals, K* keys_tmp, V* vals_tmp, in
     LGC_COUNT_LAUNCH(ctx);
     return cudaGetLastError() == cudaSuccess ? LGC_OK : LGC_ECUDA;
   }
-  // A digit pass over so few entries is a launch and a chain of look-backs,
-  // 8.5 us, and eight with their histogram 75; the n^2 comparisons of 64-bit
-  // keys and the copy back take 18 us at 8,274 entries and 56 at 19,117.
   const int D = (bits + 7) / 8;
-  if (n * n <= D * kRankWork) {
+  if (rank_sort_takes(n, D)) {
     const K mask = D >= (int)sizeof(K) ? ~(K)0 : (K)((((K)1) << (8 * D)) - 1);
     rank_sort_kernel<K, V><<<(unsigned)ceil_div(n, kRankItems), kBlock, 0, st>>>(
         keys, vals, (int)n, mask, keys_tmp, vals_tmp, vals != nullptr);
