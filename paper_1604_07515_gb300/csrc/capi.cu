@@ -481,33 +481,20 @@ __global__ void names_check_kernel(const int64_t* __restrict__ off,
   }
 }
 
-// Sets g->buckets_fit and g->sinks (left at their cautious values where there
-// is no room for the counts).
-int check_names(lgc_ctx* ctx, lgc_graph* g) {
+// Launches the checks behind g->buckets_fit and g->sinks: three counts into
+// bad, the entries that name each vertex into named (both zero before).
+void check_names(lgc_ctx* ctx, const lgc_graph* g, unsigned long long* bad, int32_t* named) {
   cudaStream_t s = ctx->stream;
-  const size_t bytes = 32 + 4 * (size_t)g->n;
-  char* buf = nullptr;
-  if (dalloc_t(ctx, &buf, bytes) != LGC_OK) return LGC_OK;
-  unsigned long long* bad = (unsigned long long*)buf;
-  int32_t* named = (int32_t*)(buf + 32);
-  bool ok = cudaMemsetAsync(buf, 0, bytes, s) == cudaSuccess;
-  if (ok && g->nnz > 0) {
+  if (g->nnz > 0) {
     names_count_kernel<<<(int)std::min<int64_t>((g->nnz + kBlock - 1) / kBlock, 16 * ctx->sms),
                          kBlock, 0, s>>>(g->col, g->nnz, g->n, named, bad);
     LGC_COUNT_LAUNCH(ctx);
   }
-  if (ok && g->n > 0) {
+  if (g->n > 0) {
     names_check_kernel<<<std::min(grid_for(g->n), 16 * ctx->sms), kBlock, 0, s>>>(
         g->off, g->col, g->nnz, g->deg, g->n, named, bad);
     LGC_COUNT_LAUNCH(ctx);
   }
-  ok = ok && cudaGetLastError() == cudaSuccess &&
-       cudaMemcpyAsync(ctx->h_scratch, bad, 24, cudaMemcpyDeviceToHost, s) == cudaSuccess;
-  dfree(ctx, buf);
-  if (cudaStreamSynchronize(s) != cudaSuccess || !ok) return LGC_ECUDA;
-  g->buckets_fit = ctx->h_scratch[0] == 0 && ctx->h_scratch[1] == 0;
-  g->sinks = ctx->h_scratch[2] != 0;
-  return LGC_OK;
 }
 
 // 1 / d by degree (fp64lite.cuh), 16 bytes a degree.
@@ -1061,9 +1048,15 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
       st = LGC_ECUDA;
       break;
     }
+    // the flags and largest degree, the list checks' counts, and how many
+    // entries name each vertex (without room for those the checks are left out)
     int* dflags = nullptr;
-    if ((st = dalloc_t(ctx, &dflags, 2)) != LGC_OK) break;
-    cudaMemsetAsync(dflags, 0, 8, s);
+    bool names = true;
+    if (dalloc_t(ctx, &dflags, 8 + n) != LGC_OK) {
+      names = false;
+      if ((st = dalloc_t(ctx, &dflags, 8)) != LGC_OK) break;
+    }
+    cudaMemsetAsync(dflags, 0, names ? 32 + 4 * (size_t)n : 32, s);
     if (n > 0) {
       if (flags & LGC_GRAPH_VALIDATE) {
         validate_kernel<<<grid_for(n), kBlock, 0, s>>>(g->off, g->col, n, nnz, dflags);
@@ -1073,11 +1066,16 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
                                                                        dflags + 1);
       LGC_COUNT_LAUNCH(ctx);
     }
-    cudaMemcpyAsync(ctx->h_scratch, dflags, 8, cudaMemcpyDeviceToHost, s);
+    if (names) check_names(ctx, g, (unsigned long long*)(dflags + 2), dflags + 8);
+    cudaMemcpyAsync(ctx->h_scratch, dflags, 32, cudaMemcpyDeviceToHost, s);
     dfree(ctx, dflags);
     if (cudaStreamSynchronize(s) != cudaSuccess || cudaGetLastError() != cudaSuccess) {
       st = LGC_ECUDA;
       break;
+    }
+    if (names) {
+      g->buckets_fit = ctx->h_scratch[1] == 0 && ctx->h_scratch[2] == 0;
+      g->sinks = ctx->h_scratch[3] != 0;
     }
     int32_t* hf = (int32_t*)ctx->h_scratch;
     if (hf[0] != 0) {
@@ -1102,7 +1100,6 @@ int lgc_graph_create(lgc_ctx* ctx, int64_t n, const int64_t* offsets, const int3
     if (st == LGC_OK) st = build_shorts(ctx, g);
     if (st == LGC_OK) st = build_recip(ctx, g);
     if (st == LGC_OK) st = build_hot(ctx, g);
-    if (st == LGC_OK) st = check_names(ctx, g);
     // complete before the handle is given out: the request loop and other
     // contexts read the graph on streams of their own
     if (st == LGC_OK && cudaStreamSynchronize(s) != cudaSuccess) st = LGC_ECUDA;

@@ -2140,7 +2140,7 @@ struct PushWork {
     const int64_t n = g->n, need = std::min<int64_t>(n, F.size + F.edges);
     const int64_t cap = room_slots(need, n, 8, kRoomFresh);
     const bool dense = want_dense(ctx, need, n) || dense_small(ctx, n) ||
-                       (ctx->table_form == 0 && n >= 1024 && 16 * cap >= 8 * n + n / 8);
+                       (ctx->table_form == 0 && n >= 1024 && 16 * cap >= 8 * n);
     Table T[4];
     T[3] = S;
     int st_ = LGC_OK;
