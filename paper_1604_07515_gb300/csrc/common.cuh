@@ -261,6 +261,10 @@ struct HotSet {
   const int32_t* ids = nullptr;
   uint32_t mult = 1;
 };
+// Graphs of at most this many entries take deterministic rounds on the device.
+// Their buckets are 4 bytes an entry, allocated by every run: the limit keeps
+// that to 2 GB (the kernels' 32-bit list starts would allow 2^31 - 1 entries).
+constexpr int64_t kRdEntries = int64_t{1} << 29;
 }  // namespace lgc
 
 // Work item of a pull round: edges [beg, beg + len) of heavy vertex w, the
@@ -375,9 +379,6 @@ namespace lgc {
 constexpr int kPullLight = 32;  // default of lgc_graph::pull_light; the deterministic bin
 constexpr int kDetBig = 1024;  // longer lists fold segment-parallel in deterministic mode
 constexpr int kDetSeg = 256;
-// Graphs of at most this many entries take deterministic rounds on the device,
-// whose buckets are 4 bytes an entry, allocated by every run (2 GB at most).
-constexpr int64_t kRdEntries = int64_t{1} << 29;
 constexpr int64_t kDetKeep = int64_t{1} << 18;  // segments whose gathered shares are kept (512 MB)
 constexpr int kPullItem = 4096;
 }  // namespace lgc

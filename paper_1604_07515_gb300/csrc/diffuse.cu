@@ -31,8 +31,6 @@
 #include <vector>
 #include <string.h>
 
-#include <cooperative_groups.h>
-
 #include "common.cuh"
 #include "edges.cuh"
 #include "foldwarp.cuh"
@@ -41,8 +39,6 @@
 #include "lookback.cuh"
 #include "prim.cuh"
 #include "rounds.cuh"
-
-namespace cg = cooperative_groups;
 
 namespace lgc {
 
@@ -84,23 +80,20 @@ __device__ inline void count_inserted(int ins, int64_t* counter) {
 // PR-Nibble, Fig. alg:pr-nibble (rule 1) / alg:pr-nibble2 (rule 0).  T holds
 // r in slot.val and p in T.p[slot]; r' is updated in place (every read of r
 // in the round is of a frontier vertex, done here before the edgeMap).
-// The vertexMap bodies take the frontier entries [i0, i1) in steps of `step`
-// (a block-uniform start: the grid's stride, or a block's own chunk) and
-// return the sum of the record counts this thread wrote.
-__device__ inline int64_t prnibble_vmap_body(int64_t i0, int64_t i1, int64_t step,
-                                             const int32_t* fv, const int32_t* fs, Table T,
-                                             const int64_t* __restrict__ off, double alpha,
-                                             double cs, double cn, double eps, int rule, int det,
-                                             int self_append, double* share, int64_t* cnt,
-                                             int64_t* foff, int32_t* nfv, int32_t* nfs,
-                                             int32_t ncap, Counters* C) {
-  int64_t csum = 0;
-  for (int64_t base = i0; base < i1; base += step) {
+__global__ void vmap_prnibble_kernel(int64_t nf, const int32_t* __restrict__ fv,
+                                     const int32_t* __restrict__ fs, Table T,
+                                     const int64_t* __restrict__ off, double alpha, double cs,
+                                     double cn, double eps, int rule, int det, int self_append,
+                                     double* __restrict__ share, int64_t* __restrict__ cnt,
+                                     int64_t* __restrict__ foff, int32_t* nfv, int32_t* nfs,
+                                     int32_t ncap, Counters* C) {
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nf;
+       base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = base + threadIdx.x;
     bool pred = false;
     int32_t v = 0, s = 0;
     int64_t d = 0;
-    if (i < i1) {
+    if (i < nf) {
       v = fv[i];
       s = fs[i];
       const bool ok = s >= 0;  // always true unless a table overflowed (flagged)
@@ -120,44 +113,31 @@ __device__ inline int64_t prnibble_vmap_body(int64_t i0, int64_t i1, int64_t ste
       if (ok) *tb_val(T, s) = rbase;
       share[i] = sh;
       cnt[i] = d + (det ? 1 : 0);
-      csum += cnt[i];
       foff[i] = o0;
       pred = ok && self_append && rule == 1 && rbase >= eps * (double)d;
     }
     frontier_append(pred, v, s, d, nfv, nfs, C, ncap);
   }
-  return csum;
-}
-
-__global__ void vmap_prnibble_kernel(int64_t nf, const int32_t* __restrict__ fv,
-                                     const int32_t* __restrict__ fs, Table T,
-                                     const int64_t* __restrict__ off, double alpha, double cs,
-                                     double cn, double eps, int rule, int det, int self_append,
-                                     double* __restrict__ share, int64_t* __restrict__ cnt,
-                                     int64_t* __restrict__ foff, int32_t* nfv, int32_t* nfs,
-                                     int32_t ncap, Counters* C) {
-  prnibble_vmap_body((int64_t)blockIdx.x * blockDim.x, nf, (int64_t)gridDim.x * blockDim.x, fv,
-                     fs, T, off, alpha, cs, cn, eps, rule, det, self_append, share, cnt, foff,
-                     nfv, nfs, ncap, C);
 }
 
 // Nibble, Fig. alg:nibble: p'[v] = p[v]/2 on the frontier (S = p, D = p',
 // fresh), share p[v]/(2 d(v)).
-__device__ inline int64_t nibble_vmap_body(int64_t i0, int64_t i1, int64_t step,
-                                           const int32_t* fv, const int32_t* fs, Table S,
-                                           Table D, const int64_t* __restrict__ off, double eps,
-                                           int fmode, int det, int self_append, double* share,
-                                           int64_t* cnt, int64_t* foff, int32_t* nfv,
-                                           int32_t* nfs, int32_t ncap, Counters* C) {
+__global__ void vmap_nibble_kernel(int64_t nf, const int32_t* __restrict__ fv,
+                                   const int32_t* __restrict__ fs, Table S, Table D,
+                                   const int64_t* __restrict__ off, double eps, int fmode,
+                                   int det, int self_append, double* __restrict__ share,
+                                   int64_t* __restrict__ cnt,
+                                   int64_t* __restrict__ foff, int32_t* nfv, int32_t* nfs,
+                                   int32_t ncap, Counters* C) {
   int64_t nins = 0;  // counted once per block
-  int64_t csum = 0;
-  for (int64_t base = i0; base < i1; base += step) {
+  for (int64_t base = (int64_t)blockIdx.x * blockDim.x; base < nf;
+       base += (int64_t)gridDim.x * blockDim.x) {
     const int64_t i = base + threadIdx.x;
     bool pred = false;
     int ins = 0;
     int32_t v = 0, ds = 0;
     int64_t d = 0;
-    if (i < i1) {
+    if (i < nf) {
       v = fv[i];
       const double pv = fs[i] >= 0 ? *tb_val(S, fs[i]) : 0.0;
       const int64_t o0 = off[v];
@@ -167,7 +147,6 @@ __device__ inline int64_t nibble_vmap_body(int64_t i0, int64_t i1, int64_t step,
       if (ds >= 0) *tb_val(D, ds) = self;
       share[i] = pv / (2.0 * (double)d);
       cnt[i] = d + (det ? 1 : 0);
-      csum += cnt[i];
       foff[i] = o0;
       if (self_append && ds >= 0)
         pred = fmode == kFmInserted ? true : self >= eps * (double)d;
@@ -176,18 +155,6 @@ __device__ inline int64_t nibble_vmap_body(int64_t i0, int64_t i1, int64_t step,
     frontier_append(pred, v, ds, d, nfv, nfs, C, ncap);
   }
   flush_count(nins, &C->aux);
-  return csum;
-}
-
-__global__ void vmap_nibble_kernel(int64_t nf, const int32_t* __restrict__ fv,
-                                   const int32_t* __restrict__ fs, Table S, Table D,
-                                   const int64_t* __restrict__ off, double eps, int fmode,
-                                   int det, int self_append, double* __restrict__ share,
-                                   int64_t* __restrict__ cnt,
-                                   int64_t* __restrict__ foff, int32_t* nfv, int32_t* nfs,
-                                   int32_t ncap, Counters* C) {
-  nibble_vmap_body((int64_t)blockIdx.x * blockDim.x, nf, (int64_t)gridDim.x * blockDim.x, fv, fs,
-                   S, D, off, eps, fmode, det, self_append, share, cnt, foff, nfv, nfs, ncap, C);
 }
 
 // HK-PR, Fig. alg:hkpr: p[v] += r[v] on the frontier; share
@@ -224,15 +191,17 @@ __global__ void vmap_hkpr_kernel(int64_t nf, const int32_t* __restrict__ fv,
 // probes, slots, adds and crossings.  Consecutive threads read consecutive
 // col[] entries.
 // ---------------------------------------------------------------------------
-// The warps [warp, nwarps) of the edge push.
-__device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
-                                        const int32_t* __restrict__ deg, const double* share,
-                                        const int64_t* epos, const int64_t* foff, int64_t nf,
-                                        int64_t E, const HotSet& H, Table D, double c, int fmode,
-                                        int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
+__global__ void __launch_bounds__(kBlock)
+    emap_atomic_kernel(const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
+                       const double* __restrict__ share, const int64_t* __restrict__ epos,
+                       const int64_t* __restrict__ foff, int64_t nf, int64_t E_host,
+                       const int64_t* __restrict__ E_dev, HotSet H, Table D, double c, int fmode,
+                       int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
   __shared__ HotShared s_tab;
   HotLane<double> S;
   hot_load(H, s_tab);
+  // the device-computed total bounds every edge index, whatever the host passed
+  const int64_t E = min(E_host, *E_dev);
   const int64_t warp = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
   const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
   int64_t nins = 0;  // counted once per block
@@ -332,17 +301,6 @@ __device__ inline void emap_atomic_body(const int32_t* __restrict__ col,
     }
   });
   flush_count(nins, &C->inserted);
-}
-
-__global__ void __launch_bounds__(kBlock)
-    emap_atomic_kernel(const int32_t* __restrict__ col, const int32_t* __restrict__ deg,
-                       const double* __restrict__ share, const int64_t* __restrict__ epos,
-                       const int64_t* __restrict__ foff, int64_t nf, int64_t E_host,
-                       const int64_t* __restrict__ E_dev, HotSet H, Table D, double c, int fmode,
-                       int32_t* nfv, int32_t* nfs, int32_t ncap, Counters* C) {
-  // the device-computed total bounds every edge index, whatever the host passed
-  emap_atomic_body(col, deg, share, epos, foff, nf, min(E_host, *E_dev), H, D, c, fmode, nfv, nfs,
-                   ncap, C);
 }
 
 // ---------------------------------------------------------------------------
@@ -2050,8 +2008,8 @@ struct PushWork {
           LGC_COUNT_LAUNCH(ctx);
         }
       } else {
-        // light vertices (writing every bitmap word), then the heavy items
-        // (ORing their vertices in); the two in one grid measured slower
+        // light vertices, then the heavy items, both ORing their vertices into
+        // the cleared bitmap; the two in one grid measured slower
         auto gather = [&](auto* shv) {
           using SH = std::remove_const_t<std::remove_pointer_t<decltype(shv)>>;
           const LightView light = g->view(1, g->pull_light);
