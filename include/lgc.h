@@ -163,15 +163,22 @@ enum {
                                    n/8 keys; in lgc_prnibble_batch, once a seed's hashed
                                    table would take more memory than the dense form), 1
                                    always hashed, 2 always dense (lgc_prnibble_batch: as 0) */
-  LGC_OPT_PULL = 7,             /* deterministic rounds gather from the frontier instead of
-                                   sorting pushed records: 0 automatic (rounds of >= 2m/16
-                                   edges), 1 never, 2 always; same results either way */
-  LGC_OPT_DEVICE_ROUNDS = 8,    /* 1 (default): consecutive small rounds of PR-Nibble (both
-                                   modes, seed sets and beta fractions too; deterministic
-                                   ones unless LGC_OPT_PULL is 2) and of atomic-mode Nibble
-                                   run in one cooperative launch without returning to the
-                                   host in between; 0: one launch per step.  Request-loop
-                                   workers never use it.  Same results either way */
+  LGC_OPT_PULL = 7,             /* rounds gather from the frontier instead of pushing (in
+                                   deterministic mode: of sorting pushed records): 0 automatic
+                                   (rounds of >= 2m/16 edges), 1 never, 2 always (atomic
+                                   PR-Nibble and Nibble: where a round is not a device round);
+                                   the same results in deterministic mode, within rounding in
+                                   atomic mode, whose gathers round each sum once */
+  LGC_OPT_DEVICE_ROUNDS = 8,    /* 1 (default): consecutive small rounds (up to 2^20 edges) of
+                                   PR-Nibble (seed sets and beta fractions too), Nibble and
+                                   HK-PR, in both modes, run in one cooperative launch without
+                                   returning to the host in between; 0: one launch per step.
+                                   Not used with LGC_OPT_PULL 2 in deterministic mode and by
+                                   HK-PR, by traced contexts and request-loop workers, where
+                                   its device memory cannot be had, and on graphs that break
+                                   the conventions above (one-way edges; in deterministic mode
+                                   repeated or unsorted ones too).  The same results in
+                                   deterministic mode, within rounding in atomic mode */
   LGC_OPT_PULL_BATCH = 9,       /* edges per lane per batch in the heavy-vertex pull gather:
                                    0 (default) the graph's tuned value (see
                                    lgc_graph_autotune), or 4, 8, 16 */
@@ -214,7 +221,8 @@ int lgc_ctx_synchronize(lgc_ctx *ctx);
 /* ---- graph ---- */
 #define LGC_GRAPH_VALIDATE 1     /* check symmetry, order, no self loops / duplicates */
 #define LGC_GRAPH_DEVICE_INPUT 2 /* offsets / cols are device pointers */
-/* Copies the CSR (Sec. 2) to the device.  Errors: LGC_EINVAL for n < 0, NULL
+/* Copies the CSR (Sec. 2) to the device; the graph is complete when the call
+ * returns, for the streams of other contexts too.  Errors: LGC_EINVAL for n < 0, NULL
  * arrays, or a failed validation; LGC_ENOMEM. */
 int lgc_graph_create(lgc_ctx *ctx, int64_t n, const int64_t *offsets, const int32_t *cols,
                      int flags, lgc_graph **out);
