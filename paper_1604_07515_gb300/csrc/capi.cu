@@ -577,24 +577,38 @@ struct Serve {
 // behind it.
 constexpr int kMaxBypass = 16;
 
+// The long lists' shares that deterministic gathers keep (kDetKeep), as their
+// buffer rounds up.
+static int64_t kept_share_bytes(const lgc_graph* g) {
+  return g->nsegs > 0 && g->nsegs <= kDetKeep ? 8 * pow2_at_least(kDetSeg * g->nsegs) : 0;
+}
+
 // Device memory a worker request may need: its sparse sets in the form they
 // take (hashed while they may stay below n/8 keys at load 1/2, else dense
-// arrays with a presence bitmap), plus frontier and share arrays.
-static int64_t request_bytes(const lgc_graph* g, const lgc_request& r) {
+// arrays with a presence bitmap), plus frontier and share arrays, and what its
+// gathers keep, where its frontiers can be large enough to gather (their
+// degrees add up to 1 / eps at most; HK-PR's to more).  lane: the batched lane
+// takes it, whose rounds push.
+static int64_t request_bytes(const lgc_graph* g, const lgc_request& r, bool lane) {
   const int64_t n = g->n;
   auto slots = [&](int64_t keys) { return pow2_at_least(2 * std::max<int64_t>(keys, 32)); };
   const int64_t dense_set = 8 * n + n / 8;  // values + presence bits
   const int64_t frontier = 16 * n;          // frontier ids, slots, shares, offsets
+  auto gathers = [&](double eps) { return eps * (double)(g->nnz / 16) <= 1.0; };
   switch (r.algo) {
     case LGC_ALGO_PRNIBBLE: {
       double bound = 1.0 + 1.0 / (r.pr.alpha * r.pr.eps);
       int64_t keys = bound < (double)n ? (int64_t)bound : n;
-      return std::min<int64_t>(slots(keys) * 24 + keys * 24, 2 * dense_set + 8 * n + frontier);
+      return std::min<int64_t>(slots(keys) * 24 + keys * 24, 2 * dense_set + 8 * n + frontier) +
+             (!lane && r.pr.mode == LGC_MODE_DET && gathers(r.pr.eps) ? kept_share_bytes(g) : 0);
     }
     case LGC_ALGO_NIBBLE:
-      return std::min<int64_t>(2 * slots(n) * 16 + n * 24, 2 * dense_set + frontier);
+      return std::min<int64_t>(2 * slots(n) * 16 + n * 24, 2 * dense_set + frontier) +
+             (r.nb.mode == LGC_MODE_DET && gathers(r.nb.eps) ? kept_share_bytes(g) : 0);
     case LGC_ALGO_HKPR:
-      return std::min<int64_t>(3 * slots(n) * 16 + n * 24, 3 * dense_set + frontier);
+      return std::min<int64_t>(3 * slots(n) * 16 + n * 24, 3 * dense_set + frontier) +
+             (int64_t)sizeof(Recip) * std::min<int64_t>((int64_t)g->max_deg + 1, kRecipMax) +
+             (r.hk.mode == LGC_MODE_DET ? kept_share_bytes(g) : 0);
     default:
       return r.rh.n_walks * 40;
   }
@@ -1338,9 +1352,10 @@ int lgc_submit(lgc_ctx* ctx, lgc_graph* g, const lgc_request* req, uint64_t* tic
     it.g = g;
     it.req = *req;
     it.submit_s = now_seconds();
-    it.bytes = request_bytes(g, *req);
+    const bool lane = req->algo == LGC_ALGO_PRNIBBLE && S->lane_ctx;
+    it.bytes = request_bytes(g, *req, lane);
     it.bypassed = 0;
-    if (req->algo == LGC_ALGO_PRNIBBLE && S->lane_ctx) S->prq.push_back(it);
+    if (lane) S->prq.push_back(it);
     else S->queue.push_back(it);
     S->known[it.ticket] = 1;
     *ticket = it.ticket;
